@@ -110,7 +110,7 @@ memd_status memd_flush(memd_ctx* c);  // apply pending transfers of the single-l
 namespace memd {
 memd_status mg_eps_eff(memd_ctx* c, double* psi, double eps_eff[9], double tol, int maxit);
 // on the calling thread from now on: the cell problems of mg_eps_eff solved
-// in turn (one solver) instead of at once (three solvers, streams, threads)
+// in turn (one right-hand side's scratch) instead of at once
 void memd_mg_cells_in_turn(bool on);
 memd_status mg_relax(memd_ctx* c, double* D64, const double* psi, const double eps_eff_inv[9],
                      double tol, int maxit, int* iters);

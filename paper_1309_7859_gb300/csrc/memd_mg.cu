@@ -12,16 +12,32 @@
 // V unknowns instead of 3V.
 //
 // Solver: conjugate gradients preconditioned by one symmetric multigrid
-// V-cycle.  A level whose extents are all even coarsens geometrically
-// (vertex-centred, by 2): red-black Gauss-Seidel, full-weighting
-// restriction, trilinear prolongation, coarse link conductances from two
-// fine links in series averaged over the 3 x 3 perpendicular neighbourhood.
-// A level with an odd extent coarsens by aggregating vertex pairs (a triple
-// at the end of an odd axis): damped Jacobi, Galerkin coarse operator,
-// piecewise-constant transfers with an over-corrected coarse correction.
-// FP64 throughout.
+// V(1,1)-cycle, FP64 throughout, the whole solve in one cooperative launch.
+// Every axis of n vertices coarsens to ceil(n / 2) (the even ones; on an odd
+// axis the last and the first vertex are both coarse and keep their link),
+// down to one vertex: linear interpolation, its transpose, and coarse link
+// conductances from two fine links in series summed over the perpendicular
+// weights.  Gauss-Seidel by colours: two where every axis is even; an odd
+// ring needs a third for its last vertex, and the sum of the axes' colours
+// modulo 3 is then a proper colouring of the periodic lattice.  The
+// iteration count is the same for even and odd meshes (15 to 20 to 1e-12 on
+// smooth random and slab profiles of contrast 40).
+//
+// What bounds it: the FP64 pipe of GB300 takes 16 cycles a warp instruction,
+// so the cycle is written for few FP64 operations a vertex (the inverse
+// diagonal kept, the pre-smoothing started from zero, the residual and the
+// prolongation left out where the last colour makes them zero or overwrites
+// them: about 35 a vertex and iteration), and, below 10^5 vertices, the
+// latency of its phases: a grid barrier costs ~1.2 us where a kernel launch
+// cost 2.5-4 us, and the host takes no part in the iteration.  Levels of at
+// most kMgCtaSites vertices run in one CTA a right-hand side, which needs
+// CTA barriers only.  A whole system's setup (48^3, 2200 charges; 77^3, 10^4
+// charges): 8.7 and 27.1 ms with one launch a half sweep, host checks between
+// iterations, and aggregation with Jacobi on odd levels; 4.2 and 9.1 ms so.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "memd_ctx.cuh"
@@ -31,676 +47,971 @@ namespace memd {
 
 namespace {
 
-constexpr int kT = 256;
-inline unsigned nblk(int64_t n) { return (unsigned)((n + kT - 1) / kT); }
+constexpr int kMgThreads = 512;
+constexpr int kMgMaxLevels = 32;  // an axis has less than 2^30 vertices
+// Levels up to this size run in one CTA a right-hand side, in shared memory:
+// a phase of 6^3 vertices takes ~0.3 us there and ~2.2 us with a grid barrier;
+// from 8^3 on the one SM's FP64 pipe is the slower (12^3 and below in one CTA
+// took 39 us a cycle, of 95, in a 48^3 solve).
+constexpr int kMgCtaSites = 343;
+constexpr int kMgCtaTotal = 700;  // of all such levels together (343 on one axis: 689)
+constexpr int kMgCtaLevels = 10;
+constexpr int kMgGrid = 256;  // most CTAs
+constexpr int kMgQ = 12;     // most sums of one reduction
+constexpr int kMgSlots = 6;  // reductions in flight between two uses of a slot
+constexpr unsigned long long kMgWaitNs = 2000000000ull;  // bound of a barrier wait
 
-struct Lv {
-  int n0, n1, n2;
-  int64_t V;
+// n / d for 0 <= n < 2^31 (multiply and shift)
+struct FastDiv {
+  unsigned d, m, s;
+};
+FastDiv fast_div(unsigned d) {
+  FastDiv f{d, 0, 0};
+  while ((1ull << f.s) < d) ++f.s;
+  f.m = (unsigned)(((1ull << 32) * ((1ull << f.s) - d)) / d + 1);
+  return f;
+}
+__device__ __forceinline__ int operator/(int n, const FastDiv& f) {
+  return (int)((__umulhi(f.m, (unsigned)n) + (unsigned)n) >> f.s);
+}
+
+// One level.  Right-hand side r of a multi-right-hand-side array is at r V.
+struct MgLv {
+  int n0, n1, n2, V;
+  int nc;            // colours
+  int hx;            // positions of one colour in a row (i = 2 h + 0 or 1)
+  FastDiv d0, d1, dh;  // by n0, n1, hx
+  double* w;    // 3 V conductances of the links
+  double* dg;   // V: their sum at a vertex
+  double* idg;  // V: its inverse (0 where it is 0)
+  double* phi;  // correction
+  double* f;    // right-hand side
+  double* r;    // residual; stays 0 on the last colour
 };
 
-__device__ __forceinline__ int wrp(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
+enum : int { kMgCells = 0, kMgRelax = 1 };
 
-__device__ __forceinline__ void coords(const Lv& L, int64_t v, int& i, int& j, int& k) {
-  i = (int)(v % L.n0);
-  const int64_t t = v / L.n0;
-  j = (int)(t % L.n1);
-  k = (int)(t / L.n1);
+struct MgOut {
+  double eff[9];    // cells: eps_eff[e][d] at 3 e + d
+  int converged, iters, timeout, pad;
+};
+
+struct MgArgs {
+  int nl, nlg;  // levels, and how many of them are swept by the whole grid
+  int dir0;     // cells: direction of right-hand side 0
+  int maxit;
+  double tol;
+  double a;
+  const double* ie64;
+  double* x;    // solution
+  double* p;
+  double* q;
+  double* part;       // kMgSlots x kMgQ x CTAs
+  unsigned* arrivals; // barrier count, 0 at launch
+  MgOut* out;
+  double* psi;        // cells: written; relax: read (3 V)
+  double* D64;        // relax: in and out
+  double einv[9];     // relax: inverse effective permittivity
+  MgLv lv[kMgMaxLevels];
+};
+
+// explicit roundings: the arithmetic of a right-hand side does not depend on
+// how many are solved at once
+__device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double mul_(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double add_(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub_(double a, double b) { return __dsub_rn(a, b); }
+
+struct Nb {
+  int xp, xm, yp, ym, zp, zm;
+};
+__device__ __forceinline__ Nb neighbours(const MgLv& L, int v, int i, int j, int k) {
+  const int P = L.n0 * L.n1;
+  Nb b;
+  b.xp = i + 1 == L.n0 ? v - i : v + 1;
+  b.xm = i == 0 ? v + L.n0 - 1 : v - 1;
+  b.yp = j + 1 == L.n1 ? v - j * L.n0 : v + L.n0;
+  b.ym = j == 0 ? v + (L.n1 - 1) * L.n0 : v - L.n0;
+  b.zp = k + 1 == L.n2 ? v - k * P : v + P;
+  b.zm = k == 0 ? v + (L.n2 - 1) * P : v - P;
+  return b;
 }
-
-__device__ __forceinline__ int64_t vid(const Lv& L, int i, int j, int k) {
-  return (int64_t)i + (int64_t)L.n0 * ((int64_t)j + (int64_t)L.n1 * k);
+__device__ __forceinline__ void coords(const MgLv& L, int v, int& i, int& j, int& k) {
+  const int row = v / L.d0;
+  i = v - row * L.n0;
+  k = row / L.d1;
+  j = row - k * L.n1;
 }
-
-// (L phi)(v) and the diagonal: sum over the 6 links at v of w (phi_v - phi_nb)
-__device__ __forceinline__ double apply_at(const Lv& L, const double* __restrict__ w,
-                                           const double* __restrict__ phi, int64_t v, int i,
-                                           int j, int k, double& nbsum, double& dg) {
-  const int64_t V = L.V;
-  const int64_t xp = vid(L, wrp(i + 1, L.n0), j, k), xm = vid(L, wrp(i - 1, L.n0), j, k);
-  const int64_t yp = vid(L, i, wrp(j + 1, L.n1), k), ym = vid(L, i, wrp(j - 1, L.n1), k);
-  const int64_t zp = vid(L, i, j, wrp(k + 1, L.n2)), zm = vid(L, i, j, wrp(k - 1, L.n2));
-  const double wxp = w[v], wxm = w[xm], wyp = w[V + v], wym = w[V + ym], wzp = w[2 * V + v],
-               wzm = w[2 * V + zm];
-  dg = ((wxp + wxm) + (wyp + wym)) + (wzp + wzm);
-  nbsum = ((wxp * phi[xp] + wxm * phi[xm]) + (wyp * phi[yp] + wym * phi[ym])) +
-          (wzp * phi[zp] + wzm * phi[zm]);
-  return dg * phi[v] - nbsum;
+// colour of a position on an axis: alternating, the last of an odd ring apart
+__device__ __forceinline__ int axis_colour(int i, int n) {
+  return (n & 1) && n > 1 && i == n - 1 ? 2 : i & 1;
 }
-
-__global__ void k_residual(Lv L, const double* __restrict__ w, const double* __restrict__ phi,
-                           const double* __restrict__ f, double* __restrict__ r) {
-  const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (v >= L.V) return;
-  int i, j, k;
-  coords(L, v, i, j, k);
-  double nb, dg;
-  const double a = apply_at(L, w, phi, v, i, j, k, nb, dg);
-  r[v] = (f ? f[v] : 0.0) - a;
+__device__ __forceinline__ bool first_colour(const MgLv& L, int i, int j, int k) {
+  const int s = axis_colour(i, L.n0) + axis_colour(j, L.n1) + axis_colour(k, L.n2);
+  return L.nc == 2 ? (s & 1) == 0 : s % 3 == 0;
 }
-
-// q = L p
-__global__ void k_apply(Lv L, const double* __restrict__ w, const double* __restrict__ p,
-                        double* __restrict__ q) {
-  const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (v >= L.V) return;
-  int i, j, k;
-  coords(L, v, i, j, k);
-  double nb, dg;
-  q[v] = apply_at(L, w, p, v, i, j, k, nb, dg);
-}
-
-// Gauss-Seidel on the vertices of one colour ((i + j + k) mod 2)
-__global__ void k_rbgs(Lv L, const double* __restrict__ w, double* __restrict__ phi,
-                       const double* __restrict__ f, int color) {
-  const int64_t h = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;  // half-index
-  const int64_t v0 = 2 * h;
-  if (v0 >= L.V) return;
-  // every x row has an even length: the vertex of this colour is v0 or v0+1
-  int i, j, k;
-  coords(L, v0, i, j, k);
-  int64_t v = v0;
-  if (((i + j + k) & 1) != color) {
-    v = v0 + 1;
-    i += 1;
+// position h of colour c: row by row, hx a row; false where there is none
+__device__ __forceinline__ bool colour_vertex(const MgLv& L, int h, int c, int& i, int& j, int& k) {
+  const int row = h / L.dh;
+  const int hh = h - row * L.hx;
+  k = row / L.d1;
+  j = row - k * L.n1;
+  const int b = axis_colour(j, L.n1) + axis_colour(k, L.n2);
+  const bool odd0 = (L.n0 & 1) && L.n0 > 1;
+  int t;
+  if (L.nc == 2) {
+    t = (c - b) & 1;
+  } else {
+    t = c - b;
+    t = t < 0 ? t + 3 : t;
+    t = t < 0 ? t + 3 : t;
   }
-  double nb, dg;
-  apply_at(L, w, phi, v, i, j, k, nb, dg);
-  phi[v] = (f[v] + nb) / dg;
-}
-
-// damped Jacobi: phi += omega (f - L phi) / diag, in two passes through r
-__global__ void k_jacobi_res(Lv L, const double* __restrict__ w, const double* __restrict__ phi,
-                             const double* __restrict__ f, double* __restrict__ r) {
-  const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (v >= L.V) return;
-  int i, j, k;
-  coords(L, v, i, j, k);
-  double nb, dg;
-  const double a = apply_at(L, w, phi, v, i, j, k, nb, dg);
-  r[v] = (f[v] - a) / dg;
-}
-
-__global__ void k_jacobi_upd(int64_t V, double* __restrict__ phi, const double* __restrict__ r,
-                             double omega) {
-  const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (v < V) phi[v] += omega * r[v];
-}
-
-// full weighting: fc(I) = sum_o prod_d (1 - |o_d| / 2) / 8 r(2 I + o)
-__global__ void k_restrict(Lv F, Lv Cc, const double* __restrict__ r, double* __restrict__ fc) {
-  const int64_t V = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (V >= Cc.V) return;
-  int I, J, K;
-  coords(Cc, V, I, J, K);
-  double s = 0.0;
-  for (int oz = -1; oz <= 1; ++oz)
-    for (int oy = -1; oy <= 1; ++oy)
-      for (int ox = -1; ox <= 1; ++ox) {
-        const double wt = (ox ? 0.5 : 1.0) * (oy ? 0.5 : 1.0) * (oz ? 0.5 : 1.0);
-        s += wt * r[vid(F, wrp(2 * I + ox, F.n0), wrp(2 * J + oy, F.n1), wrp(2 * K + oz, F.n2))];
-      }
-  fc[V] = 0.125 * s;
-}
-
-// trilinear prolongation of the coarse correction, added to phi
-__global__ void k_prolong(Lv F, Lv Cc, const double* __restrict__ ec, double* __restrict__ phi) {
-  const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (v >= F.V) return;
-  int i, j, k;
-  coords(F, v, i, j, k);
-  const int I0 = i >> 1, J0 = j >> 1, K0 = k >> 1;
-  const int di = i & 1, dj = j & 1, dk = k & 1;
-  double s = 0.0;
-  for (int c = 0; c < 8; ++c) {
-    const int ax = c & 1, ay = (c >> 1) & 1, az = c >> 2;
-    if ((ax && !di) || (ay && !dj) || (az && !dk)) continue;
-    const double wt = (di ? 0.5 : 1.0) * (dj ? 0.5 : 1.0) * (dk ? 0.5 : 1.0);
-    s += wt * ec[vid(Cc, wrp(I0 + ax, Cc.n0), wrp(J0 + ay, Cc.n1), wrp(K0 + az, Cc.n2))];
+  if (t < 2) {
+    i = 2 * hh + t;
+    return i < (odd0 ? L.n0 - 1 : L.n0);
   }
-  phi[v] += s;
+  i = L.n0 - 1;
+  return odd0 && hh == 0;
 }
 
-// coarse conductance of link (d, I): the two fine d-links from 2I + o (o
-// perpendicular to d) in series, averaged with weights (1/4, 1/2, 1/4)^2
-// over o, halved for the coarse spacing
-__global__ void k_coarsen(Lv F, Lv Cc, const double* __restrict__ wf, double* __restrict__ wc) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= 3 * Cc.V) return;
-  const int d = (int)(t / Cc.V);
-  const int64_t V = t - (int64_t)d * Cc.V;
-  int I, J, K;
-  coords(Cc, V, I, J, K);
-  const int e1 = (d + 1) % 3, e2 = (d + 2) % 3;
-  double s = 0.0;
-  for (int b = -1; b <= 1; ++b)
-    for (int a = -1; a <= 1; ++a) {
-      int p[3] = {2 * I, 2 * J, 2 * K};
-      p[e1] += a;
-      p[e2] += b;
-      int q[3] = {p[0], p[1], p[2]};
-      q[d] += 1;
-      const int64_t l1 = (int64_t)d * F.V + vid(F, wrp(p[0], F.n0), wrp(p[1], F.n1), wrp(p[2], F.n2));
-      const int64_t l2 = (int64_t)d * F.V + vid(F, wrp(q[0], F.n0), wrp(q[1], F.n1), wrp(q[2], F.n2));
-      const double w1 = wf[l1], w2 = wf[l2];
-      const double ser = w1 * w2 / (w1 + w2);
-      s += (a ? 0.5 : 1.0) * (b ? 0.5 : 1.0) * 0.25 * ser;
+// ---------------------------------------------------------- phases
+// t0, stride: this thread's share of the vertices; r0: first right-hand side
+
+// Gauss-Seidel on one colour; acc (optional) gathers f . phi of the updated
+template <int NR>
+__device__ __forceinline__ void sweep(const MgLv& L, int c, int t0, int stride, int r0,
+                                      double* acc) {
+  const int H = L.hx * L.n1 * L.n2, V = L.V;
+  const double* w = L.w;
+  for (int h = t0; h < H; h += stride) {
+    int i, j, k;
+    if (!colour_vertex(L, h, c, i, j, k)) continue;
+    const int v = i + L.n0 * (j + L.n1 * k);
+    const Nb b = neighbours(L, v, i, j, k);
+    const double wxp = w[v], wxm = w[b.xm], wyp = w[V + v], wym = w[V + b.ym], wzp = w[2 * V + v],
+                 wzm = w[2 * V + b.zm], id = L.idg[v];
+    double y[NR], g[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const double* p = L.phi + (r0 + r) * V;
+      g[r] = L.f[(r0 + r) * V + v];
+      double s = fma_(wxp, p[b.xp], g[r]);
+      s = fma_(wxm, p[b.xm], s);
+      s = fma_(wyp, p[b.yp], s);
+      s = fma_(wym, p[b.ym], s);
+      s = fma_(wzp, p[b.zp], s);
+      s = fma_(wzm, p[b.zm], s);
+      y[r] = mul_(s, id);
     }
-  wc[t] = 0.5 * s;
-}
-
-// Aggregation (a level with an odd extent): coarse vertex I along an axis
-// of n fine vertices and m = n / 2 coarse ones holds fine 2I, 2I + 1, and
-// also 2I + 2 when it is the last one of an odd n.  Piecewise-constant
-// prolongation; the Galerkin coarse operator is the aggregates' graph
-// Laplacian, the conductance of coarse link (d, I) the sum of the fine
-// d-links leaving aggregate I towards I + e_d.
-__device__ __forceinline__ int agg_lo(int I) { return 2 * I; }
-__device__ __forceinline__ int agg_hi(int I, int m, int n) { return I == m - 1 ? n - 1 : 2 * I + 1; }
-__device__ __forceinline__ int agg_of(int i, int m) { return min(i >> 1, m - 1); }
-
-__global__ void k_agg_coarsen(Lv F, Lv Cc, const double* __restrict__ wf, double* __restrict__ wc) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= 3 * Cc.V) return;
-  const int d = (int)(t / Cc.V);
-  const int64_t V = t - (int64_t)d * Cc.V;
-  int C[3];
-  coords(Cc, V, C[0], C[1], C[2]);
-  const int nf[3] = {F.n0, F.n1, F.n2}, nc[3] = {Cc.n0, Cc.n1, Cc.n2};
-  int lo[3], hi[3];
-  for (int e = 0; e < 3; ++e) {
-    lo[e] = agg_lo(C[e]);
-    hi[e] = agg_hi(C[e], nc[e], nf[e]);
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      L.phi[(r0 + r) * V + v] = y[r];
+      if (acc) acc[r] = fma_(g[r], y[r], acc[r]);
+    }
   }
-  lo[d] = hi[d];  // the last fine layer of the aggregate along d
+}
+
+// f - L phi on every colour but the last (where the sweep left 0)
+template <int NR>
+__device__ __forceinline__ void residual(const MgLv& L, int t0, int stride, int r0) {
+  const int H = L.hx * L.n1 * L.n2, V = L.V;
+  const double* w = L.w;
+  for (int c = 0; c + 1 < L.nc; ++c)
+    for (int h = t0; h < H; h += stride) {
+      int i, j, k;
+      if (!colour_vertex(L, h, c, i, j, k)) continue;
+      const int v = i + L.n0 * (j + L.n1 * k);
+      const Nb b = neighbours(L, v, i, j, k);
+      const double wxp = w[v], wxm = w[b.xm], wyp = w[V + v], wym = w[V + b.ym],
+                   wzp = w[2 * V + v], wzm = w[2 * V + b.zm], dg = L.dg[v];
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const double* p = L.phi + (r0 + r) * V;
+        double s = fma_(-dg, p[v], L.f[(r0 + r) * V + v]);
+        s = fma_(wxp, p[b.xp], s);
+        s = fma_(wxm, p[b.xm], s);
+        s = fma_(wyp, p[b.yp], s);
+        s = fma_(wym, p[b.ym], s);
+        s = fma_(wzp, p[b.zp], s);
+        s = fma_(wzm, p[b.zm], s);
+        L.r[(r0 + r) * V + v] = s;
+      }
+    }
+}
+
+// the two fine neighbours of coarse position I on an axis of n fine vertices
+// and their weights in the transpose of the interpolation
+__device__ __forceinline__ void axis_pair(int I, int n, int m, int& lo, int& hi, double& wl,
+                                          double& wr) {
+  const bool odd = n & 1;
+  lo = I == 0 ? n - 1 : 2 * I - 1;
+  hi = 2 * I + 1 >= n ? 0 : 2 * I + 1;
+  wl = odd && I == 0 ? 0.0 : 0.5;
+  wr = odd && I == m - 1 ? 0.0 : 0.5;
+}
+
+// f of the coarse level, and its first half sweep from zero (the first
+// colour's values; 0 elsewhere)
+template <int NR>
+__device__ __forceinline__ void restrict_to(const MgLv& F, const MgLv& C, int t0, int stride,
+                                            int r0) {
+  const bool two = F.nc == 2 && F.n0 > 1 && F.n1 > 1 && F.n2 > 1;
+  for (int v = t0; v < C.V; v += stride) {
+    int I, J, K;
+    coords(C, v, I, J, K);
+    int x[3], y[3], z[3];
+    double wx[3], wy[3], wz[3];
+    x[1] = 2 * I;
+    y[1] = 2 * J;
+    z[1] = 2 * K;
+    wx[1] = wy[1] = wz[1] = 1.0;
+    axis_pair(I, F.n0, C.n0, x[0], x[2], wx[0], wx[2]);
+    axis_pair(J, F.n1, C.n1, y[0], y[2], wy[0], wy[2]);
+    axis_pair(K, F.n2, C.n2, z[0], z[2], wz[0], wz[2]);
+    double s[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) s[r] = 0.0;
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const double wyz = mul_(wy[b], wz[c]);
+        const int row = F.n0 * (y[b] + F.n1 * z[c]);
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          const double* q = F.r + (r0 + r) * F.V + row;
+          if (two) {
+            // the residual is 0 on the odd vertices: half of the 27 drop out
+            if (((b + c) & 1) == 0)
+              s[r] = fma_(wyz, q[x[1]], s[r]);
+            else
+              s[r] = fma_(mul_(wyz, 0.5), add_(q[x[0]], q[x[2]]), s[r]);
+          } else {
+            double t = fma_(wx[0], q[x[0]], q[x[1]]);
+            t = fma_(wx[2], q[x[2]], t);
+            s[r] = fma_(wyz, t, s[r]);
+          }
+        }
+      }
+    const bool c0 = first_colour(C, I, J, K);
+    const double id = C.idg[v];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      C.f[(r0 + r) * C.V + v] = s[r];
+      C.phi[(r0 + r) * C.V + v] = c0 ? mul_(s[r], id) : 0.0;
+    }
+  }
+}
+
+// phi += interpolated coarse correction, on every colour but the last (which
+// the first half sweep after it overwrites)
+template <int NR>
+__device__ __forceinline__ void prolong(const MgLv& F, const MgLv& C, int t0, int stride, int r0) {
+  const int H = F.hx * F.n1 * F.n2;
+  for (int c = 0; c + 1 < F.nc; ++c)
+    for (int h = t0; h < H; h += stride) {
+      int i, j, k;
+      if (!colour_vertex(F, h, c, i, j, k)) continue;
+      const int v = i + F.n0 * (j + F.n1 * k);
+      const int I0 = i >> 1, J0 = j >> 1, K0 = k >> 1;
+      const int I1 = I0 + 1 == C.n0 ? 0 : I0 + 1, J1 = J0 + 1 == C.n1 ? 0 : J0 + 1,
+                K1 = K0 + 1 == C.n2 ? 0 : K0 + 1;
+      const bool ox = i & 1, oy = j & 1, oz = k & 1;
+      const double half = (ox ? 0.5 : 1.0) * (oy ? 0.5 : 1.0) * (oz ? 0.5 : 1.0);
+      const int r00 = C.n0 * (J0 + C.n1 * K0), r10 = C.n0 * (J1 + C.n1 * K0),
+                r01 = C.n0 * (J0 + C.n1 * K1), r11 = C.n0 * (J1 + C.n1 * K1);
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const double* e = C.phi + (r0 + r) * C.V;
+        auto line = [&](int row) { return ox ? add_(e[row + I0], e[row + I1]) : e[row + I0]; };
+        double t = line(r00);
+        if (oy) t = add_(t, line(r10));
+        if (oz) t = add_(t, oy ? add_(line(r01), line(r11)) : line(r01));
+        double* p = F.phi + (r0 + r) * F.V + v;
+        *p = fma_(half, t, *p);
+      }
+    }
+}
+
+// conductance of link d of coarse vertex (I, J, K): the fine links in series
+// (one at the seam of an odd axis), over the perpendicular weights
+__device__ __forceinline__ double coarse_link(const MgLv& F, const MgLv& C, int d, int I, int J,
+                                              int K) {
+  const int nf[3] = {F.n0, F.n1, F.n2}, nc[3] = {C.n0, C.n1, C.n2}, c[3] = {I, J, K};
+  if (nc[d] == 1) return 0.0;
+  const int sf[3] = {1, F.n0, F.n0 * F.n1};
+  const int e1 = (d + 1) % 3, e2 = (d + 2) % 3;
+  const bool seam = (nf[d] & 1) && c[d] == nc[d] - 1;
+  const int along = 2 * c[d] * sf[d];
+  int p1[3], p2[3];
+  double w1[3], w2[3];
+  p1[1] = 2 * c[e1];
+  p2[1] = 2 * c[e2];
+  w1[1] = w2[1] = 1.0;
+  axis_pair(c[e1], nf[e1], nc[e1], p1[0], p1[2], w1[0], w1[2]);
+  axis_pair(c[e2], nf[e2], nc[e2], p2[0], p2[2], w2[0], w2[2]);
+  const double* w = F.w + (int64_t)d * F.V;
   double s = 0.0;
-  for (int k = lo[2]; k <= hi[2]; ++k)
-    for (int j = lo[1]; j <= hi[1]; ++j)
-      for (int i = lo[0]; i <= hi[0]; ++i) s += wf[(int64_t)d * F.V + vid(F, i, j, k)];
-  wc[t] = s;
+#pragma unroll
+  for (int b = 0; b < 3; ++b)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      // a link along an axis that coarsens is positive, also where wp is 0
+      const double wp = mul_(w1[a], w2[b]);
+      const int v = along + p1[a] * sf[e1] + p2[b] * sf[e2];
+      const double u = w[v], u1 = seam ? u : w[v + sf[d]];
+      s = fma_(wp, seam ? u : mul_(u, u1) / add_(u, u1), s);
+    }
+  return s;
 }
 
-__global__ void k_agg_restrict(Lv F, Lv Cc, const double* __restrict__ r, double* __restrict__ fc) {
-  const int64_t V = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (V >= Cc.V) return;
-  int I, J, K;
-  coords(Cc, V, I, J, K);
-  const int i1 = agg_hi(I, Cc.n0, F.n0), j1 = agg_hi(J, Cc.n1, F.n1), k1 = agg_hi(K, Cc.n2, F.n2);
-  double s = 0.0;
-  for (int k = agg_lo(K); k <= k1; ++k)
-    for (int j = agg_lo(J); j <= j1; ++j)
-      for (int i = agg_lo(I); i <= i1; ++i) s += r[vid(F, i, j, k)];
-  fc[V] = s;
-}
+// ------------------------------------------------------- barrier and sums
+// Grid barrier of the cooperative launch over a count of arrivals that only
+// grows (0 at launch): complete when it reaches round x CTAs.  The wait is
+// bounded; a CTA that gives up marks the result and every CTA leaves.
+struct GridSync {
+  unsigned* arrivals;
+  MgOut* out;
+  unsigned target;
+  int* s_ok;
+  __device__ bool operator()() {
+    __syncthreads();
+    if (gridDim.x == 1) return true;
+    target += gridDim.x;
+    if (threadIdx.x == 0) {
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(arrivals) : "memory");
+      int ok = 1;
+      unsigned long long t0 = 0, t;
+      for (unsigned it = 1;; ++it) {
+        unsigned cur;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(cur) : "l"(arrivals) : "memory");
+        if (cur >= target) break;
+        if ((it & 255u) == 0u) {
+          asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+          if (t0 == 0) t0 = t;
+          if (t - t0 > kMgWaitNs || __ldcg(&out->timeout) != 0) {
+            atomicExch(&out->timeout, 1);
+            ok = 0;
+            break;
+          }
+        }
+      }
+      *s_ok = ok;
+    }
+    __syncthreads();
+    return *s_ok != 0;
+  }
+};
 
-// phi += alpha e(aggregate of v); alpha > 1 makes up for the flat prolongation
-__global__ void k_agg_prolong(Lv F, Lv Cc, const double* __restrict__ ec, double alpha,
-                              double* __restrict__ phi) {
-  const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (v >= F.V) return;
-  int i, j, k;
-  coords(F, v, i, j, k);
-  phi[v] += alpha * ec[vid(Cc, agg_of(i, Cc.n0), agg_of(j, Cc.n1), agg_of(k, Cc.n2))];
-}
-
-// The coarsest level (at most kCoarseSmem vertices) in one CTA: sweeps
-// forward (red then black, or damped Jacobi) then backward, all in shared
-// memory, instead of one launch per half-sweep.
-constexpr int kCoarseSmem = 1024;
-
-__global__ void __launch_bounds__(1024)
-    k_coarse_solve(Lv L, const double* __restrict__ w, const double* __restrict__ f,
-                   double* __restrict__ phi, int sweeps, int rb) {
-  extern __shared__ double sm[];
-  const int V = (int)L.V;
-  double* sw = sm;            // 3V
-  double* sf = sm + 3 * V;    // V
-  double* sp = sm + 4 * V;    // V
-  double* st = sm + 5 * V;    // V
-  for (int t = threadIdx.x; t < 3 * V; t += blockDim.x) sw[t] = w[t];
-  for (int t = threadIdx.x; t < V; t += blockDim.x) {
-    sf[t] = f[t];
-    sp[t] = 0.0;
+// this CTA's share of NQ sums into slot; every CTA reads all shares after the
+// next grid barrier and adds them in the same order
+template <int NQ>
+__device__ __forceinline__ void share_sums(double* part, int slot, const double (&x)[NQ],
+                                           double (*sh)[kMgQ]) {
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    double s = x[q];
+    for (int o = 16; o > 0; o >>= 1) s = add_(s, __shfl_down_sync(0xffffffffu, s, o));
+    if (lane == 0) sh[wp][q] = s;
   }
   __syncthreads();
-  auto relax_vertex = [&](int v, bool jac) {
-    int i, j, k;
-    coords(L, v, i, j, k);
-    double nb, dg;
-    const double a = apply_at(L, sw, sp, v, i, j, k, nb, dg);
-    if (jac)
-      st[v] = (sf[v] - a) / dg;
-    else
-      sp[v] = (sf[v] + nb) / dg;
-  };
-  for (int dir = 0; dir < 2; ++dir)
-    for (int s = 0; s < sweeps; ++s) {
-      if (rb) {
-        for (int h = 0; h < 2; ++h) {
-          const int color = dir == 0 ? h : 1 - h;
-          for (int v = threadIdx.x; v < V; v += blockDim.x) {
-            int i, j, k;
-            coords(L, v, i, j, k);
-            if (((i + j + k) & 1) == color) relax_vertex(v, false);
-          }
-          __syncthreads();
+  static_assert(kMgThreads == 512, "sixteen warps");
+  if (wp < NQ) {
+    double s = lane < 16 ? sh[lane][wp] : 0.0;
+    for (int o = 8; o > 0; o >>= 1) s = add_(s, __shfl_down_sync(0xffffffffu, s, o));
+    if (lane == 0) part[((int64_t)slot * kMgQ + wp) * gridDim.x + blockIdx.x] = s;
+  }
+}
+template <int NQ>
+__device__ __forceinline__ void total_sums(const double* part, int slot, double (&x)[NQ],
+                                           double* tot) {
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  static_assert(NQ <= kMgThreads / 32, "one warp a sum");
+  if (wp < NQ) {
+    const double* p = part + ((int64_t)slot * kMgQ + wp) * gridDim.x;
+    double y[kMgGrid / 32];
+#pragma unroll
+    for (int k = 0; k < kMgGrid / 32; ++k)
+      y[k] = lane + 32 * k < (int)gridDim.x ? __ldcg(p + lane + 32 * k) : 0.0;
+    double s = y[0];
+#pragma unroll
+    for (int k = 1; k < kMgGrid / 32; ++k)
+      if (32 * k < (int)gridDim.x) s = add_(s, y[k]);
+    for (int o = 16; o > 0; o >>= 1) s = add_(s, __shfl_down_sync(0xffffffffu, s, o));
+    if (lane == 0) tot[wp] = s;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) x[q] = tot[q];
+}
+
+// The whole solve for NR right-hand sides.
+//   cells: L psi_d = -div(eps e_d) for d = dir0 .. dir0 + NR - 1, psi_d of
+//   zero mean and the mean fluxes eps_e (delta_ed - grad_e psi_d)
+//   relax: L phi = div D64; D64 <- eps (-grad phi + sum_d E0_d (e_d - grad
+//   psi_d)) with E0 from the mean of D64
+// Stops when |r| <= tol |f| / 4 (2-norms) or, once the recursion has reached
+// its rounding floor and the residual grows again (to 100 times its least
+// value), when that least value was below 100 tol |f|.
+template <int NR, int MODE>
+__global__ void __launch_bounds__(kMgThreads, 2) k_mg_solve(const __grid_constant__ MgArgs a) {
+  __shared__ double sh[kMgThreads / 32][kMgQ];
+  __shared__ double tot[2][kMgQ];
+  __shared__ int s_ok;
+  GridSync grid{a.arrivals, a.out, 0u, &s_ok};
+#define MG_GRID() \
+  if (!grid()) return
+  // neighbouring warps of work go to different SMs: a level with less work
+  // than the grid has warps still uses every FP64 pipe
+  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
+  const int t0 = (wp * (int)gridDim.x + (int)blockIdx.x) * 32 + lane;
+  const int stride = (int)gridDim.x * kMgThreads;
+  const MgLv& L = a.lv[0];
+  const int V = L.V;
+  const double inv_a = 1.0 / a.a, inv_a2 = 1.0 / (a.a * a.a), nV = (double)V;
+  double mean0[3] = {0.0, 0.0, 0.0};  // relax: mean of D64
+  {
+    // conductances of the finest level, the right-hand side and its sum
+    constexpr int NQ = MODE == kMgRelax ? 4 : NR;
+    double s[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) s[q] = 0.0;
+    for (int v = t0; v < V; v += stride) {
+      int i, j, k;
+      coords(L, v, i, j, k);
+      const Nb b = neighbours(L, v, i, j, k);
+      const int vm[3] = {b.xm, b.ym, b.zm};
+#pragma unroll
+      for (int d = 0; d < 3; ++d) L.w[d * V + v] = inv_a2 / a.ie64[(int64_t)d * V + v];
+      if (MODE == kMgRelax) {
+        double div = 0.0;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+          const double D = a.D64[(int64_t)d * V + v];
+          s[1 + d] = add_(s[1 + d], D);
+          div = add_(div, sub_(D, a.D64[(int64_t)d * V + vm[d]]));
         }
+        const double f = mul_(inv_a, div);
+        L.f[v] = f;
+        s[0] = add_(s[0], f);
       } else {
-        for (int v = threadIdx.x; v < V; v += blockDim.x) relax_vertex(v, true);
-        __syncthreads();
-        for (int v = threadIdx.x; v < V; v += blockDim.x) sp[v] += 0.8 * st[v];
-        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          const int d = a.dir0 + r;
+          const double* ie = a.ie64 + (int64_t)d * V;
+          const double f = mul_(-(__drcp_rn(ie[v]) - __drcp_rn(ie[vm[d]])), inv_a);
+          L.f[r * V + v] = f;
+          s[r] = add_(s[r], f);
+        }
       }
     }
-  for (int t = threadIdx.x; t < V; t += blockDim.x) phi[t] = sp[t];
+    share_sums<NQ>(a.part, 0, s, sh);
+    MG_GRID();
+    double m[NQ];
+    total_sums<NQ>(a.part, 0, m, tot[0]);
+    if (MODE == kMgRelax) {
+#pragma unroll
+      for (int d = 0; d < 3; ++d) mean0[d] = m[NQ - 3 + d] / nV;
+    }
+    for (int v = t0; v < V; v += stride)
+#pragma unroll
+      for (int r = 0; r < NR; ++r) L.f[r * V + v] = sub_(L.f[r * V + v], m[r] / nV);
+  }
+  // diagonals, and the conductances level by level
+  for (int l = 0; l < a.nl; ++l) {
+    const MgLv& F = a.lv[l];
+    for (int v = t0; v < F.V; v += stride) {
+      int i, j, k;
+      coords(F, v, i, j, k);
+      const Nb b = neighbours(F, v, i, j, k);
+      const int U = F.V;
+      const double dg = ((F.w[v] + F.w[b.xm]) + (F.w[U + v] + F.w[U + b.ym])) +
+                        (F.w[2 * U + v] + F.w[2 * U + b.zm]);
+      F.dg[v] = dg;
+      F.idg[v] = dg > 0.0 ? 1.0 / dg : 0.0;
+#pragma unroll
+      for (int r = 0; r < NR; ++r) F.r[r * U + v] = 0.0;
+    }
+    if (l + 1 < a.nl) {
+      const MgLv& C = a.lv[l + 1];
+      for (int t = t0; t < 3 * C.V; t += stride) {
+        const int d = t >= 2 * C.V ? 2 : (t >= C.V ? 1 : 0);
+        int I, J, K;
+        coords(C, t - d * C.V, I, J, K);
+        C.w[t] = coarse_link(F, C, d, I, J, K);
+      }
+    }
+    MG_GRID();
+  }
+  // x = 0, p = 0, |f|^2, the first half sweep
+  double f2[NR], least[NR], rz[NR];
+  bool done[NR];
+  {
+    double s[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) s[r] = 0.0;
+    for (int v = t0; v < V; v += stride) {
+      int i, j, k;
+      coords(L, v, i, j, k);
+      const bool c0 = first_colour(L, i, j, k);
+      const double id = L.idg[v];
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const double f = L.f[r * V + v];
+        s[r] = fma_(f, f, s[r]);
+        a.x[r * V + v] = 0.0;
+        a.p[r * V + v] = 0.0;
+        L.phi[r * V + v] = c0 ? mul_(f, id) : 0.0;
+      }
+    }
+    share_sums<NR>(a.part, 1, s, sh);
+    MG_GRID();
+    total_sums<NR>(a.part, 1, f2, tot[1]);
+  }
+  bool all = true;
+#pragma unroll
+  for (int r = 0; r < NR; ++r) {
+    done[r] = f2[r] == 0.0;
+    least[r] = f2[r];
+    rz[r] = 0.0;
+    all = all && done[r];
+  }
+  // the levels of the one-CTA part: coefficients into shared memory
+  __shared__ double s_mem[8 * kMgCtaTotal];
+  __shared__ MgLv s_lv[kMgCtaLevels];
+  if ((int)blockIdx.x < NR) {
+    int at = 0;
+    for (int l = a.nlg; l < a.nl; ++l) {
+      const MgLv& F = a.lv[l];
+      const int U = F.V;
+      double* b = s_mem + 8 * at;
+      at += U;
+      for (int v = threadIdx.x; v < U; v += kMgThreads) {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) b[d * U + v] = F.w[d * U + v];
+        b[3 * U + v] = F.dg[v];
+        b[4 * U + v] = F.idg[v];
+        b[7 * U + v] = 0.0;
+      }
+      if (threadIdx.x == 0) {
+        MgLv C = F;
+        C.w = b;
+        C.dg = b + 3 * U;
+        C.idg = b + 4 * U;
+        C.phi = b + 5 * U;
+        C.f = b + 6 * U;
+        C.r = b + 7 * U;
+        s_lv[l - a.nlg] = C;
+      }
+    }
+  }
+  __syncthreads();
+  int its = 0;
+  const double tol2 = a.tol * a.tol;
+  while (!all) {
+    // z = M r in phi of level 0: one V(1,1)-cycle, its first half sweep made
+    // where r was; sums r . z
+    double acc[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) acc[r] = 0.0;
+    for (int l = 0; l < a.nlg; ++l) {
+      const MgLv& F = a.lv[l];
+      for (int c = 1; c < F.nc; ++c) {
+        sweep<NR>(F, c, t0, stride, 0, nullptr);
+        MG_GRID();
+      }
+      residual<NR>(F, t0, stride, 0);
+      MG_GRID();
+      restrict_to<NR>(F, a.lv[l + 1], t0, stride, 0);
+      MG_GRID();
+    }
+    if ((int)blockIdx.x < NR) {
+      const int r = blockIdx.x, t = threadIdx.x;
+      double one = 0.0;
+      const MgLv& top = a.lv[a.nlg];
+      for (int v = t; v < top.V; v += kMgThreads) {
+        s_lv[0].f[v] = top.f[r * top.V + v];
+        s_lv[0].phi[v] = top.phi[r * top.V + v];
+      }
+      __syncthreads();
+      const int nc = a.nl - a.nlg;
+      for (int l = 0; l + 1 < nc; ++l) {
+        const MgLv& F = s_lv[l];
+        for (int c = 1; c < F.nc; ++c) {
+          sweep<1>(F, c, t, kMgThreads, 0, nullptr);
+          __syncthreads();
+        }
+        residual<1>(F, t, kMgThreads, 0);
+        __syncthreads();
+        restrict_to<1>(F, s_lv[l + 1], t, kMgThreads, 0);
+        __syncthreads();
+      }
+      for (int l = nc - 2; l >= 0; --l) {
+        const MgLv& F = s_lv[l];
+        prolong<1>(F, s_lv[l + 1], t, kMgThreads, 0);
+        __syncthreads();
+        for (int c = F.nc - 1; c >= 0; --c) {
+          sweep<1>(F, c, t, kMgThreads, 0, l + a.nlg == 0 ? &one : nullptr);
+          __syncthreads();
+        }
+      }
+      for (int v = t; v < top.V; v += kMgThreads) top.phi[r * top.V + v] = s_lv[0].phi[v];
+#pragma unroll
+      for (int q = 0; q < NR; ++q)
+        if (q == r) acc[q] = one;
+    }
+    if (a.nlg > 0) MG_GRID();
+    for (int l = a.nlg - 1; l >= 0; --l) {
+      const MgLv& F = a.lv[l];
+      prolong<NR>(F, a.lv[l + 1], t0, stride, 0);
+      MG_GRID();
+      for (int c = F.nc - 1; c >= 0; --c) {
+        sweep<NR>(F, c, t0, stride, 0, l == 0 ? acc : nullptr);
+        if (l > 0 || c > 0) MG_GRID();
+      }
+    }
+    share_sums<NR>(a.part, 2, acc, sh);
+    MG_GRID();
+    double rz1[NR];
+    total_sums<NR>(a.part, 2, rz1, tot[0]);
+    // p = z + beta p, then q = L p and p . q
+    double beta[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      beta[r] = rz[r] != 0.0 ? rz1[r] / rz[r] : 0.0;
+      rz[r] = rz1[r];
+    }
+    // (a few vertices a thread at once: every load before the first store)
+    constexpr int UP = NR == 1 ? 4 : 2;
+    for (int v0 = t0; v0 < V; v0 += UP * stride) {
+      double p[UP][NR], z[UP][NR];
+#pragma unroll
+      for (int u = 0; u < UP; ++u)
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          const int v = v0 + u * stride;
+          const bool in = v < V;
+          p[u][r] = in ? a.p[r * V + v] : 0.0;
+          z[u][r] = in ? L.phi[r * V + v] : 0.0;
+        }
+#pragma unroll
+      for (int u = 0; u < UP; ++u)
+#pragma unroll
+        for (int r = 0; r < NR; ++r)
+          if (v0 + u * stride < V)
+            a.p[r * V + v0 + u * stride] = fma_(beta[r], p[u][r], z[u][r]);
+    }
+    MG_GRID();
+    double pq[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) pq[r] = 0.0;
+    for (int v = t0; v < V; v += stride) {
+      int i, j, k;
+      coords(L, v, i, j, k);
+      const Nb b = neighbours(L, v, i, j, k);
+      const double wxp = L.w[v], wxm = L.w[b.xm], wyp = L.w[V + v], wym = L.w[V + b.ym],
+                   wzp = L.w[2 * V + v], wzm = L.w[2 * V + b.zm], dg = L.dg[v];
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const double* p = a.p + r * V;
+        double s = mul_(dg, p[v]);
+        s = fma_(-wxp, p[b.xp], s);
+        s = fma_(-wxm, p[b.xm], s);
+        s = fma_(-wyp, p[b.yp], s);
+        s = fma_(-wym, p[b.ym], s);
+        s = fma_(-wzp, p[b.zp], s);
+        s = fma_(-wzm, p[b.zm], s);
+        a.q[r * V + v] = s;
+        pq[r] = fma_(p[v], s, pq[r]);
+      }
+    }
+    share_sums<NR>(a.part, 3, pq, sh);
+    MG_GRID();
+    total_sums<NR>(a.part, 3, pq, tot[1]);
+    // x and r, and the next cycle's first half sweep
+    double alpha[NR], rr[NR];
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      alpha[r] = !done[r] && pq[r] != 0.0 ? rz[r] / pq[r] : 0.0;
+      rr[r] = 0.0;
+    }
+    constexpr int UX = NR == 1 ? 3 : 1;
+    for (int v0 = t0; v0 < V; v0 += UX * stride) {
+      double x[UX][NR], p[UX][NR], f[UX][NR], q[UX][NR], id[UX];
+#pragma unroll
+      for (int u = 0; u < UX; ++u) {
+        const int v = v0 + u * stride;
+        const bool in = v < V;
+        id[u] = in ? L.idg[v] : 0.0;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          x[u][r] = in ? a.x[r * V + v] : 0.0;
+          p[u][r] = in ? a.p[r * V + v] : 0.0;
+          f[u][r] = in ? L.f[r * V + v] : 0.0;
+          q[u][r] = in ? a.q[r * V + v] : 0.0;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < UX; ++u) {
+        const int v = v0 + u * stride;
+        if (v >= V) break;
+        int i, j, k;
+        coords(L, v, i, j, k);
+        const bool c0 = first_colour(L, i, j, k);
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+          const double t = fma_(-alpha[r], q[u][r], f[u][r]);
+          rr[r] = fma_(t, t, rr[r]);
+          a.x[r * V + v] = fma_(alpha[r], p[u][r], x[u][r]);
+          L.f[r * V + v] = t;
+          L.phi[r * V + v] = c0 ? mul_(t, id[u]) : 0.0;
+        }
+      }
+    }
+    share_sums<NR>(a.part, 4, rr, sh);
+    MG_GRID();
+    total_sums<NR>(a.part, 4, rr, tot[0]);
+    ++its;
+    all = true;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      if (!done[r]) {
+        // a quarter of tol: the residual a solve that checks every second
+        // iteration ends at
+        const double goal = 0.0625 * tol2 * f2[r];
+        done[r] = rr[r] <= goal || (rr[r] > 100.0 * least[r] && least[r] <= 1e4 * tol2 * f2[r]);
+        least[r] = rr[r] < least[r] ? rr[r] : least[r];
+      }
+      all = all && done[r];
+    }
+    if (its >= a.maxit) break;
+  }
+  // results
+  if (MODE == kMgCells) {
+    double s[4 * NR];
+#pragma unroll
+    for (int q = 0; q < 4 * NR; ++q) s[q] = 0.0;
+    for (int v = t0; v < V; v += stride) {
+      int i, j, k;
+      coords(L, v, i, j, k);
+      const Nb b = neighbours(L, v, i, j, k);
+      const int vp[3] = {b.xp, b.yp, b.zp};
+      double eps[3];
+#pragma unroll
+      for (int e = 0; e < 3; ++e) eps[e] = __drcp_rn(a.ie64[(int64_t)e * V + v]);
+#pragma unroll
+      for (int r = 0; r < NR; ++r) {
+        const double* x = a.x + r * V;
+        s[4 * r] = add_(s[4 * r], x[v]);
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          const double g = fma_(-inv_a, sub_(x[vp[e]], x[v]), e == a.dir0 + r ? 1.0 : 0.0);
+          s[4 * r + 1 + e] = fma_(g, eps[e], s[4 * r + 1 + e]);
+        }
+      }
+    }
+    share_sums<4 * NR>(a.part, 5, s, sh);
+    MG_GRID();
+    total_sums<4 * NR>(a.part, 5, s, tot[1]);
+    for (int v = t0; v < V; v += stride)
+#pragma unroll
+      for (int r = 0; r < NR; ++r)
+        a.psi[(int64_t)(a.dir0 + r) * V + v] = sub_(a.x[r * V + v], s[4 * r] / nV);
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+#pragma unroll
+      for (int r = 0; r < NR; ++r)
+#pragma unroll
+        for (int e = 0; e < 3; ++e) a.out->eff[3 * e + a.dir0 + r] = s[4 * r + 1 + e] / nV;
+  } else if (all) {  // not converged: D64 stays as it came
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int v = t0; v < V; v += stride) {
+      int i, j, k;
+      coords(L, v, i, j, k);
+      const Nb b = neighbours(L, v, i, j, k);
+      const int vp[3] = {b.xp, b.yp, b.zp};
+#pragma unroll
+      for (int e = 0; e < 3; ++e)
+        s[e] = add_(s[e], mul_(sub_(a.x[v], a.x[vp[e]]), inv_a) / a.ie64[(int64_t)e * V + v]);
+    }
+    share_sums<3>(a.part, 5, s, sh);
+    MG_GRID();
+    total_sums<3>(a.part, 5, s, tot[1]);
+    double E0[3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e)
+      E0[e] = a.einv[3 * e] * (mean0[0] - s[0] / nV) + a.einv[3 * e + 1] * (mean0[1] - s[1] / nV) +
+              a.einv[3 * e + 2] * (mean0[2] - s[2] / nV);
+    for (int v = t0; v < V; v += stride) {
+      int i, j, k;
+      coords(L, v, i, j, k);
+      const Nb b = neighbours(L, v, i, j, k);
+      const int vp[3] = {b.xp, b.yp, b.zp};
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        // (x, psi) differences along the link: phi + sum_d E0_d psi_d
+        double g = sub_(a.x[v], a.x[vp[e]]);
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+          g = fma_(E0[d], sub_(a.psi[(int64_t)d * V + v], a.psi[(int64_t)d * V + vp[e]]), g);
+        a.D64[(int64_t)e * V + v] = fma_(inv_a, g, E0[e]) / a.ie64[(int64_t)e * V + v];
+      }
+    }
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    a.out->converged = all ? 1 : 0;
+    a.out->iters = its;
+  }
+#undef MG_GRID
 }
 
-// fine conductances w = eps / a^2 = 1 / (ie a^2)
-__global__ void k_fine_w(int64_t n, const double* __restrict__ ie64, double inv_a2,
-                         double* __restrict__ w) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t < n) w[t] = inv_a2 / ie64[t];
+// ---------------------------------------------------------------- host
+// One of these launches is in flight on a device at a time, whatever streams
+// and threads they come from: each waits (on its stream) for the one before,
+// so two grids never hold SMs that the other's barriers wait for.  A grid
+// takes half an SM's registers, which leaves the room of a single-launch
+// step's CTA beside it.
+struct Gate {
+  std::mutex mu;
+  cudaEvent_t ev = nullptr;
+};
+constexpr int kMgDevices = 64;
+Gate g_gate[kMgDevices];
+
+template <int NR, int MODE>
+cudaError_t launch_solve(const MgArgs& a, int device, int grid, cudaStream_t st) {
+  if (device < 0 || device >= kMgDevices) return cudaErrorInvalidDevice;
+  Gate& g = g_gate[device];
+  std::lock_guard<std::mutex> lock(g.mu);
+  cudaError_t e = g.ev ? cudaStreamWaitEvent(st, g.ev, 0)
+                       : cudaEventCreateWithFlags(&g.ev, cudaEventDisableTiming);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3(kMgThreads, 1, 1);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, k_mg_solve<NR, MODE>, a);
+  if (e == cudaSuccess) e = cudaEventRecord(g.ev, st);
+  return e;
 }
 
-// f = div F (links -> vertices), F given as 3V link values, scaled by s
-__global__ void k_div_links(Lv L, const double* __restrict__ F, double s, double* __restrict__ f) {
-  const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (v >= L.V) return;
-  int i, j, k;
-  coords(L, v, i, j, k);
-  const int64_t V = L.V;
-  const double dx = F[v] - F[vid(L, wrp(i - 1, L.n0), j, k)];
-  const double dy = F[V + v] - F[V + vid(L, i, wrp(j - 1, L.n1), k)];
-  const double dz = F[2 * V + v] - F[2 * V + vid(L, i, j, wrp(k - 1, L.n2))];
-  f[v] = s * ((dx + dy) + dz);
-}
+// The levels and their scratch for NR right-hand sides, one block of memory.
+struct MgPlan {
+  MgArgs a{};
+  double* block = nullptr;
+  size_t zero_bytes = 0;  // the leading words cleared before a launch
+  int grid = 0;
 
-// f = -div(eps e_d) = -(eps_d(v) - eps_d(v - e_d)) / a
-__global__ void k_div_eps_unit(Lv L, const double* __restrict__ ie64, int d, double inv_a,
-                               double* __restrict__ f) {
-  const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (v >= L.V) return;
-  int i, j, k;
-  coords(L, v, i, j, k);
-  int c[3] = {i, j, k};
-  c[d] -= 1;
-  const int64_t vm = vid(L, wrp(c[0], L.n0), wrp(c[1], L.n1), wrp(c[2], L.n2));
-  f[v] = -(1.0 / ie64[(int64_t)d * L.V + v] - 1.0 / ie64[(int64_t)d * L.V + vm]) * inv_a;
-}
+  bool build(memd_ctx* c, int nr) {
+    const Mesh& m = c->mesh;
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess)
+      return false;
+    // a warp of work for every warp of the grid on the finest level, one CTA an SM at most
+    grid = (int)std::min<int64_t>(std::min(sms, kMgGrid), std::max<int64_t>(nr, (m.V + 127) / 128));
+    int n[3] = {m.n[0], m.n[1], m.n[2]};
+    size_t words = 0;
+    std::vector<size_t> at;
+    int nl = 0;
+    for (;; ++nl) {
+      if (nl == kMgMaxLevels) return false;
+      MgLv& L = a.lv[nl];
+      const int64_t V = (int64_t)n[0] * n[1] * n[2];
+      L.n0 = n[0];
+      L.n1 = n[1];
+      L.n2 = n[2];
+      L.V = (int)V;
+      const bool odd = (n[0] > 1 && n[0] % 2) || (n[1] > 1 && n[1] % 2) || (n[2] > 1 && n[2] % 2);
+      L.nc = odd ? 3 : 2;
+      L.hx = std::max(1, n[0] / 2);
+      L.d0 = fast_div((unsigned)n[0]);
+      L.d1 = fast_div((unsigned)n[1]);
+      L.dh = fast_div((unsigned)L.hx);
+      at.push_back(words);
+      words += (size_t)V * (5 + 3 * nr);
+      if (V == 1) break;
+      for (int d = 0; d < 3; ++d) n[d] = (n[d] + 1) / 2;
+    }
+    a.nl = nl + 1;
+    a.nlg = 0;
+    while (a.nlg + 1 < a.nl && a.lv[a.nlg].V > kMgCtaSites) ++a.nlg;
+    int sites = 0;
+    for (int l = a.nlg; l < a.nl; ++l) sites += a.lv[l].V;
+    if (sites > kMgCtaTotal || a.nl - a.nlg > kMgCtaLevels) return false;
+    const size_t head = (sizeof(MgOut) + 64) / sizeof(double) + 1;  // result, barrier count
+    const size_t parts = (size_t)kMgSlots * kMgQ * grid;
+    const size_t total = head + parts + words + (size_t)3 * nr * m.V;
+    block = (double*)memd_dalloc(c, total * sizeof(double));
+    if (!block) return false;
+    a.out = (MgOut*)block;
+    a.arrivals = (unsigned*)((char*)block + ((sizeof(MgOut) + 31) / 32) * 32);
+    zero_bytes = head * sizeof(double);
+    a.part = block + head;
+    double* base = a.part + parts;
+    for (int l = 0; l < a.nl; ++l) {
+      MgLv& L = a.lv[l];
+      double* b = base + at[l];
+      const size_t V = (size_t)L.V;
+      L.w = b;
+      L.dg = b + 3 * V;
+      L.idg = b + 4 * V;
+      L.phi = b + 5 * V;
+      L.f = L.phi + nr * V;
+      L.r = L.f + nr * V;
+    }
+    a.x = base + words;
+    a.p = a.x + (size_t)nr * m.V;
+    a.q = a.p + (size_t)nr * m.V;
+    a.a = m.a;
+    a.ie64 = c->ie64;
+    return true;
+  }
+  // clears the barrier count, launches, waits, and reads the result
+  template <int NR, int MODE>
+  memd_status run(memd_ctx* c, MgOut& h) {
+    const cudaStream_t st = c->stream;
+    if (cudaMemsetAsync(block, 0, zero_bytes, st) != cudaSuccess ||
+        launch_solve<NR, MODE>(a, c->device, grid, st) != cudaSuccess ||
+        cudaMemcpyAsync(&h, a.out, sizeof(h), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
+      return MEMD_ERR_CUDA;
+    if (h.timeout) return MEMD_ERR_TIMEOUT;
+    return h.converged ? MEMD_OK : MEMD_ERR_RELAX_NOCONV;
+  }
+};
 
-// out = eps (g e_dir - grad phi) on every link, scaled: out_e(v) = eps_e(v) *
-// (g [e == dir] - (phi(v + e_e) - phi(v)) / a); dir < 0 for no constant
-__global__ void k_flux(Lv L, const double* __restrict__ ie64, const double* __restrict__ phi,
-                       int dir, double g, double inv_a, double* __restrict__ out, int accumulate,
-                       double scale) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= 3 * L.V) return;
-  const int e = (int)(t / L.V);
-  const int64_t v = t - (int64_t)e * L.V;
-  int i, j, k;
-  coords(L, v, i, j, k);
-  int c[3] = {i, j, k};
-  c[e] += 1;
-  const int64_t vp = vid(L, wrp(c[0], L.n0), wrp(c[1], L.n1), wrp(c[2], L.n2));
-  const double val = ((e == dir ? g : 0.0) - (phi[vp] - phi[v]) * inv_a) / ie64[t];
-  out[t] = accumulate ? out[t] + scale * val : scale * val;
-}
-
-// CG scalars on the device: s[0] = p.q, s[1] = r.z (old), s[2] = r.z (new)
-__global__ void k_cg_xr(int64_t n, double* __restrict__ x, double* __restrict__ r,
-                        const double* __restrict__ p, const double* __restrict__ q,
-                        const double* __restrict__ s, int rz) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const double pq = s[0];
-  const double alpha = pq != 0.0 ? s[rz] / pq : 0.0;
-  x[t] += alpha * p[t];
-  r[t] -= alpha * q[t];
-}
-
-__global__ void k_cg_p(int64_t n, double* __restrict__ p, const double* __restrict__ z,
-                       const double* __restrict__ s, int rz_new, int rz_old) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  const double b = s[rz_old];
-  const double beta = b != 0.0 ? s[rz_new] / b : 0.0;
-  p[t] = z[t] + beta * p[t];
-}
-
-__global__ void k_sub_mean(int64_t n, double* __restrict__ x, const double* __restrict__ sum) {
-  const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (t < n) x[t] -= sum[0] / (double)n;
-}
+// Set on a thread (the request server's admission workers): that thread's
+// cell problems are solved in turn, with one right-hand side's scratch.
+thread_local bool t_cells_in_turn = false;
 
 }  // namespace
 
-// ---------------------------------------------------------------- solver
-struct MgLevel {
-  Lv L;
-  double* w = nullptr;    // 3V conductances
-  double* phi = nullptr;  // V
-  double* f = nullptr;    // V
-  double* r = nullptr;    // V
-  bool rb = true;         // red-black Gauss-Seidel (every extent even), else Jacobi
-  bool agg = false;       // transfer to the next level by aggregation, else geometric
-};
-
-constexpr double kAggAlpha = 1.6;  // over-correction of the aggregated coarse correction
-
-struct MgSolver {
-  memd_ctx* c = nullptr;
-  std::vector<MgLevel> lv;
-  double *x = nullptr, *res = nullptr, *z = nullptr, *p = nullptr, *q = nullptr, *sc = nullptr;
-  double* part = nullptr;
-  cudaGraphExec_t it_graph = nullptr;
-  std::vector<void*> blocks;
-
-  double* alloc(size_t n) {
-    void* ptr = memd_dalloc(c, n * sizeof(double));
-    if (ptr) blocks.push_back(ptr);
-    return (double*)ptr;
-  }
-  void release() {
-    if (it_graph) cudaGraphExecDestroy(it_graph);
-    it_graph = nullptr;
-    for (void* b : blocks) memd_dfree(c, b);
-    blocks.clear();
-  }
-
-  void smooth(int l, bool forward, cudaStream_t st) {
-    MgLevel& a = lv[l];
-    if (a.rb) {
-      const int64_t half = a.L.V / 2;
-      const int first = forward ? 0 : 1;
-      k_rbgs<<<nblk(half), kT, 0, st>>>(a.L, a.w, a.phi, a.f, first);
-      k_rbgs<<<nblk(half), kT, 0, st>>>(a.L, a.w, a.phi, a.f, first ^ 1);
-    } else {
-      k_jacobi_res<<<nblk(a.L.V), kT, 0, st>>>(a.L, a.w, a.phi, a.f, a.r);
-      k_jacobi_upd<<<nblk(a.L.V), kT, 0, st>>>(a.L.V, a.phi, a.r, 0.8);
-    }
-  }
-
-  // z ~ L^-1 f on level l (phi of level l starts at 0); symmetric
-  void vcycle(int l, cudaStream_t st) {
-    MgLevel& a = lv[l];
-    cudaMemsetAsync(a.phi, 0, a.L.V * sizeof(double), st);
-    if (l + 1 == (int)lv.size()) {
-      const int sweeps = a.L.V <= 512 ? 8 : 12;
-      if (a.L.V <= kCoarseSmem) {
-        k_coarse_solve<<<1, 1024, 6 * a.L.V * sizeof(double), st>>>(a.L, a.w, a.f, a.phi, sweeps,
-                                                                   a.rb ? 1 : 0);
-        return;
-      }
-      for (int s = 0; s < sweeps; ++s) smooth(l, true, st);
-      for (int s = 0; s < sweeps; ++s) smooth(l, false, st);
-      return;
-    }
-    MgLevel& b = lv[l + 1];
-    smooth(l, true, st);
-    smooth(l, true, st);
-    k_residual<<<nblk(a.L.V), kT, 0, st>>>(a.L, a.w, a.phi, a.f, a.r);
-    if (a.agg)
-      k_agg_restrict<<<nblk(b.L.V), kT, 0, st>>>(a.L, b.L, a.r, b.f);
-    else
-      k_restrict<<<nblk(b.L.V), kT, 0, st>>>(a.L, b.L, a.r, b.f);
-    vcycle(l + 1, st);
-    if (a.agg)
-      k_agg_prolong<<<nblk(a.L.V), kT, 0, st>>>(a.L, b.L, b.phi, kAggAlpha, a.phi);
-    else
-      k_prolong<<<nblk(a.L.V), kT, 0, st>>>(a.L, b.L, b.phi, a.phi);
-    smooth(l, false, st);
-    smooth(l, false, st);
-  }
-
-  bool build(memd_ctx* ctx, cudaStream_t st) {
-    c = ctx;
-    const Mesh& m = c->mesh;
-    Lv L{m.n[0], m.n[1], m.n[2], m.V};
-    const double inv_a2 = 1.0 / (m.a * m.a);
-    for (int l = 0;; ++l) {
-      MgLevel a;
-      a.L = L;
-      a.w = alloc(3 * L.V);
-      a.phi = alloc(L.V);
-      a.f = alloc(L.V);
-      a.r = alloc(L.V);
-      if (!a.w || !a.phi || !a.f || !a.r) return false;
-      a.rb = (L.n0 % 2 == 0) && (L.n1 % 2 == 0) && (L.n2 % 2 == 0);
-      if (l == 0)
-        k_fine_w<<<nblk(3 * L.V), kT, 0, st>>>(3 * L.V, c->ie64, inv_a2, a.w);
-      else if (lv.back().agg)
-        k_agg_coarsen<<<nblk(3 * L.V), kT, 0, st>>>(lv.back().L, L, lv.back().w, a.w);
-      else
-        k_coarsen<<<nblk(3 * L.V), kT, 0, st>>>(lv.back().L, L, lv.back().w, a.w);
-      a.agg = !a.rb;  // the way down from this level
-      lv.push_back(a);
-      if (L.n0 < 4 || L.n1 < 4 || L.n2 < 4 || L.V <= 64) break;
-      L.n0 /= 2;
-      L.n1 /= 2;
-      L.n2 /= 2;
-      L.V = (int64_t)L.n0 * L.n1 * L.n2;
-    }
-    const int64_t V = m.V;
-    x = alloc(V);
-    res = alloc(V);
-    z = alloc(V);
-    p = alloc(V);
-    q = alloc(V);
-    sc = alloc(16);
-    part = alloc(reduce_blocks());
-    return x && res && z && p && q && sc && part && cudaGetLastError() == cudaSuccess;
-  }
-
-  // two CG iterations (the r.z slots alternate), preconditioned by a V-cycle
-  void iterations(cudaStream_t st) {
-    const int64_t V = lv[0].L.V;
-    for (int h = 0; h < 2; ++h) {
-      const int old_s = 1 + h, new_s = 2 - h;
-      k_apply<<<nblk(V), kT, 0, st>>>(lv[0].L, lv[0].w, p, q);
-      launch_dot(p, q, V, part, st);
-      launch_finish(part, 0, sc + 0, st);
-      k_cg_xr<<<nblk(V), kT, 0, st>>>(V, x, res, p, q, sc, old_s);
-      cudaMemcpyAsync(lv[0].f, res, V * sizeof(double), cudaMemcpyDeviceToDevice, st);
-      vcycle(0, st);
-      cudaMemcpyAsync(z, lv[0].phi, V * sizeof(double), cudaMemcpyDeviceToDevice, st);
-      launch_dot(res, z, V, part, st);
-      launch_finish(part, 0, sc + new_s, st);
-      k_cg_p<<<nblk(V), kT, 0, st>>>(V, p, z, sc, new_s, old_s);
-    }
-    launch_dot(res, res, V, part, st);
-    launch_finish(part, 0, sc + 3, st);
-  }
-
-  // A solve in stages, so that one host thread can interleave several
-  // solvers on their own streams: begin (to the first residual), then
-  // launch_step / check until done, then finish.
-  double f2 = 0.0, least = 0.0;
-  int its = 0, cap = 0;
-  bool done = false;
-
-  memd_status begin(const double* f, int maxit, cudaStream_t st) {
-    const int64_t V = lv[0].L.V;
-    // r = f - mean(f), x = 0, z = M r, p = z
-    cudaMemcpyAsync(res, f, V * sizeof(double), cudaMemcpyDeviceToDevice, st);
-    launch_dot(res, nullptr, V, part, st);
-    launch_finish(part, 0, sc + 4, st);
-    k_sub_mean<<<nblk(V), kT, 0, st>>>(V, res, sc + 4);
-    launch_dot(res, res, V, part, st);
-    launch_finish(part, 0, sc + 5, st);
-    cudaMemsetAsync(x, 0, V * sizeof(double), st);
-    cudaMemcpyAsync(lv[0].f, res, V * sizeof(double), cudaMemcpyDeviceToDevice, st);
-    vcycle(0, st);
-    cudaMemcpyAsync(z, lv[0].phi, V * sizeof(double), cudaMemcpyDeviceToDevice, st);
-    cudaMemcpyAsync(p, z, V * sizeof(double), cudaMemcpyDeviceToDevice, st);
-    launch_dot(res, z, V, part, st);
-    launch_finish(part, 0, sc + 1, st);
-    if (!it_graph && c->use_graphs) {
-      cudaGraph_t g = nullptr;
-      if (cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-        iterations(st);
-        if (cudaStreamEndCapture(st, &g) != cudaSuccess ||
-            cudaGraphInstantiate(&it_graph, g, 0) != cudaSuccess)
-          it_graph = nullptr;
-        if (g) cudaGraphDestroy(g);
-      }
-      cudaGetLastError();
-    }
-    double h = 0.0;
-    if (cudaMemcpyAsync(&h, sc + 5, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-      return MEMD_ERR_CUDA;
-    f2 = h;
-    its = 0;
-    done = f2 == 0.0;
-    least = f2;
-    cap = maxit < 400 ? maxit : 400;
-    return MEMD_OK;
-  }
-  bool running() const { return !done && its < cap; }
-  // two iterations queued on st
-  memd_status launch_step(cudaStream_t st) {
-    if (it_graph) {
-      if (cudaGraphLaunch(it_graph, st) != cudaSuccess) return MEMD_ERR_CUDA;
-    } else {
-      iterations(st);
-    }
-    its += 2;
-    return MEMD_OK;
-  }
-  // waits for st and tests the residual of the last step
-  memd_status check(double tol, cudaStream_t st) {
-    double h = 0.0;
-    if (cudaMemcpyAsync(&h, sc + 3, sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-      return MEMD_ERR_CUDA;
-    done = h <= tol * tol * f2;
-    if (!done && h > 100.0 * least && least <= 1e4 * tol * tol * f2) done = true;
-    least = std::min(least, h);
-    return MEMD_OK;
-  }
-  memd_status finish(double* out, int* iters, cudaStream_t st) {
-    const int64_t V = lv[0].L.V;
-    if (iters) *iters = its;
-    // zero-mean solution
-    launch_dot(x, nullptr, V, part, st);
-    launch_finish(part, 0, sc + 6, st);
-    k_sub_mean<<<nblk(V), kT, 0, st>>>(V, x, sc + 6);
-    cudaMemcpyAsync(out, x, V * sizeof(double), cudaMemcpyDeviceToDevice, st);
-    if (cudaGetLastError() != cudaSuccess) return MEMD_ERR_CUDA;
-    return done ? MEMD_OK : MEMD_ERR_RELAX_NOCONV;
-  }
-
-  // x = L^-1 f (f of zero mean up to rounding; x of zero mean); stops when
-  // |r| <= tol |f| (2-norms), or, once the recursion has reached its
-  // rounding floor and the residual grows again (to 100 times its least
-  // value), when that least value was below 100 tol |f|; at most
-  // min(maxit, 400) iterations
-  memd_status solve(const double* f, double* out, double tol, int maxit, int* iters,
-                    cudaStream_t st) {
-    memd_status s = begin(f, maxit, st);
-    while (s == MEMD_OK && running()) {
-      s = launch_step(st);
-      if (s == MEMD_OK) s = check(tol, st);
-    }
-    return s == MEMD_OK ? finish(out, iters, st) : s;
-  }
-};
-
-// ------------------------------------------------------------ entry points
-// Cell problems: psi_d (3V, stored), and eps_eff[e][d] = mean over links of
-// eps_e (delta_ed - grad_e psi_d) (row e, column d).
-// Set on a thread (the request server's admission workers, several of which
-// already set systems up at once): that thread's cell problems are solved in
-// turn, with one solver's scratch.
-namespace {
-thread_local bool t_cells_in_turn = false;
-}
 void memd_mg_cells_in_turn(bool on) { t_cells_in_turn = on; }
 
+// Cell problems: psi_d (3V, stored), and eps_eff[e][d] = mean over links of
+// eps_e (delta_ed - grad_e psi_d) (row e, column d).
 memd_status mg_eps_eff(memd_ctx* c, double* psi, double eps_eff[9], double tol, int maxit) {
-  const Mesh& m = c->mesh;
-  const Lv L{m.n[0], m.n[1], m.n[2], m.V};
-  // The three cell problems are independent: each gets its own solver (and
-  // scratch) and stream, and this thread interleaves them (each one's two
-  // iterations queued, then each one's residual read), so that their small
-  // multigrid launches run at once; the results are those of solving them
-  // in turn, which a thread set by memd_mg_cells_in_turn does, with one
-  // solver on the context's stream.
-  const int ns = t_cells_in_turn ? 1 : 3;
-  MgSolver S[3];
-  double* f[3] = {nullptr, nullptr, nullptr};
-  double* U[3] = {nullptr, nullptr, nullptr};
-  cudaStream_t sts[3] = {c->stream, nullptr, nullptr};
-  cudaEvent_t ready = nullptr;
+  const int nr = t_cells_in_turn ? 1 : 3;
+  MgPlan plan;
+  if (!plan.build(c, nr)) return MEMD_ERR_OOM;
+  plan.a.psi = psi;
+  plan.a.tol = tol;
+  plan.a.maxit = maxit < 400 ? maxit : 400;
   memd_status s = MEMD_OK;
-  auto cleanup = [&]() {
-    // no scratch is released while a stream may still use it
-    for (int k = 0; k < 3; ++k)
-      if (sts[k]) cudaStreamSynchronize(sts[k]);
-    for (MgSolver& x : S) x.release();
-    for (int k = 1; k < 3; ++k)
-      if (sts[k]) cudaStreamDestroy(sts[k]);
-    if (ready) cudaEventDestroy(ready);
-  };
-  for (int k = 1; k < ns && s == MEMD_OK; ++k)
-    if (cudaStreamCreateWithFlags(&sts[k], cudaStreamNonBlocking) != cudaSuccess)
-      s = MEMD_ERR_CUDA;
-  if (s == MEMD_OK && ns > 1 &&
-      (cudaEventCreateWithFlags(&ready, cudaEventDisableTiming) != cudaSuccess ||
-       cudaEventRecord(ready, c->stream) != cudaSuccess))
-    s = MEMD_ERR_CUDA;
-  for (int k = 0; k < ns && s == MEMD_OK; ++k) {
-    // the solver's level weights come from 1/eps, written on the context's stream
-    if (k > 0 && cudaStreamWaitEvent(sts[k], ready, 0) != cudaSuccess) s = MEMD_ERR_CUDA;
-    if (s == MEMD_OK && !S[k].build(c, sts[k])) s = MEMD_ERR_OOM;
-    if (s == MEMD_OK) {
-      f[k] = S[k].alloc(m.V);
-      U[k] = S[k].alloc(3 * m.V);
-      if (!f[k] || !U[k]) s = MEMD_ERR_OOM;
-    }
+  for (int d = 0; d < 3 && s == MEMD_OK; d += nr) {
+    plan.a.dir0 = d;
+    MgOut h;
+    s = nr == 1 ? plan.run<1, kMgCells>(c, h) : plan.run<3, kMgCells>(c, h);
+    if (s == MEMD_OK)
+      for (int r = 0; r < nr; ++r)
+        for (int e = 0; e < 3; ++e) eps_eff[3 * e + d + r] = h.eff[3 * e + d + r];
   }
-  // cell problems d0 .. d0 + ns - 1, problem d0 + k with solver k
-  auto solve_cells = [&](int d0) -> memd_status {
-    memd_status r = MEMD_OK;
-    for (int k = 0; k < ns && r == MEMD_OK; ++k) {
-      k_div_eps_unit<<<nblk(m.V), kT, 0, sts[k]>>>(L, c->ie64, d0 + k, 1.0 / m.a, f[k]);
-      r = S[k].begin(f[k], maxit, sts[k]);
-    }
-    bool any = true;
-    while (r == MEMD_OK && any) {
-      any = false;
-      for (int k = 0; k < ns && r == MEMD_OK; ++k)
-        if (S[k].running()) r = S[k].launch_step(sts[k]);
-      for (int k = 0; k < ns && r == MEMD_OK; ++k)
-        if (S[k].running()) {
-          r = S[k].check(tol, sts[k]);
-          any = true;
-        }
-    }
-    for (int k = 0; k < ns && r == MEMD_OK; ++k) {
-      const int d = d0 + k;
-      const cudaStream_t st = sts[k];
-      r = S[k].finish(psi + d * m.V, nullptr, st);
-      if (r != MEMD_OK) break;
-      k_flux<<<nblk(3 * m.V), kT, 0, st>>>(L, c->ie64, psi + d * m.V, d, 1.0, 1.0 / m.a, U[k],
-                                           0, 1.0);
-      for (int e = 0; e < 3; ++e) {
-        launch_dot(U[k] + e * m.V, nullptr, m.V, S[k].part, st);
-        launch_finish(S[k].part, 0, S[k].sc + 8 + e, st);
-      }
-      double h[3];
-      if (cudaMemcpyAsync(h, S[k].sc + 8, 3 * sizeof(double), cudaMemcpyDeviceToHost, st) !=
-              cudaSuccess ||
-          cudaStreamSynchronize(st) != cudaSuccess) {
-        r = MEMD_ERR_CUDA;
-        break;
-      }
-      for (int e = 0; e < 3; ++e) eps_eff[3 * e + d] = h[e] / (double)m.V;
-    }
-    return r;
-  };
-  for (int d0 = 0; d0 < 3 && s == MEMD_OK; d0 += ns) s = solve_cells(d0);
-  cleanup();
+  memd_dfree(c, plan.block);
   return s;
 }
 
@@ -709,53 +1020,17 @@ memd_status mg_eps_eff(memd_ctx* c, double* psi, double eps_eff[9], double tol, 
 // L phi = div D64, E0 = eps_eff^-1 (M - mean(-eps grad phi)).
 memd_status mg_relax(memd_ctx* c, double* D64, const double* psi, const double eps_eff_inv[9],
                      double tol, int maxit, int* iters) {
-  const Mesh& m = c->mesh;
-  const cudaStream_t st = c->stream;
-  const Lv L{m.n[0], m.n[1], m.n[2], m.V};
-  MgSolver S;
-  if (!S.build(c, st)) {
-    S.release();
-    return MEMD_ERR_OOM;
-  }
-  double* f = S.alloc(m.V);
-  double* phi = S.alloc(m.V);
-  if (!f || !phi) {
-    S.release();
-    return MEMD_ERR_OOM;
-  }
-  // mean of D64 per component
-  for (int e = 0; e < 3; ++e) {
-    launch_dot(D64 + e * m.V, nullptr, m.V, S.part, st);
-    launch_finish(S.part, 0, S.sc + 8 + e, st);
-  }
-  k_div_links<<<nblk(m.V), kT, 0, st>>>(L, D64, 1.0 / m.a, f);
-  memd_status s = S.solve(f, phi, tol, maxit, iters, st);
-  if (s == MEMD_OK) {
-    // D64 <- -eps grad phi, its mean
-    k_flux<<<nblk(3 * m.V), kT, 0, st>>>(L, c->ie64, phi, -1, 0.0, 1.0 / m.a, D64, 0, 1.0);
-    for (int e = 0; e < 3; ++e) {
-      launch_dot(D64 + e * m.V, nullptr, m.V, S.part, st);
-      launch_finish(S.part, 0, S.sc + 11 + e, st);
-    }
-    double h[6];
-    if (cudaMemcpyAsync(h, S.sc + 8, 6 * sizeof(double), cudaMemcpyDeviceToHost, st) !=
-            cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess) {
-      s = MEMD_ERR_CUDA;
-    } else {
-      double dm[3], E0[3];
-      for (int e = 0; e < 3; ++e) dm[e] = (h[e] - h[3 + e]) / (double)m.V;
-      for (int e = 0; e < 3; ++e)
-        E0[e] = eps_eff_inv[3 * e] * dm[0] + eps_eff_inv[3 * e + 1] * dm[1] +
-                eps_eff_inv[3 * e + 2] * dm[2];
-      for (int d = 0; d < 3; ++d)
-        if (E0[d] != 0.0)
-          k_flux<<<nblk(3 * m.V), kT, 0, st>>>(L, c->ie64, psi + d * m.V, d, 1.0, 1.0 / m.a, D64,
-                                               1, E0[d]);
-      if (cudaGetLastError() != cudaSuccess) s = MEMD_ERR_CUDA;
-    }
-  }
-  S.release();
+  MgPlan plan;
+  if (!plan.build(c, 1)) return MEMD_ERR_OOM;
+  plan.a.psi = const_cast<double*>(psi);
+  plan.a.D64 = D64;
+  plan.a.tol = tol;
+  plan.a.maxit = maxit < 400 ? maxit : 400;
+  for (int t = 0; t < 9; ++t) plan.a.einv[t] = eps_eff_inv[t];
+  MgOut h;
+  const memd_status s = plan.run<1, kMgRelax>(c, h);
+  if (iters) *iters = s == MEMD_OK ? h.iters : 0;
+  memd_dfree(c, plan.block);
   return s;
 }
 

@@ -189,9 +189,8 @@ memd_status admit(memd_server* s, memd_server::Req& r, cudaStream_t wst) {
 
 void worker(memd_server* s, int w) {
   cudaSetDevice(s->opt.device);  // resolved at create
-  // several workers already set systems up at once: each solves a system's
-  // cell problems in turn (three at once per worker slowed the served
-  // stream: p50 1.2-1.35 s -> 1.8-2.05 s)
+  // several workers set systems up at once: each solves a system's cell
+  // problems in turn, with the scratch the admission ledger counts
   memd::memd_mg_cells_in_turn(true);
   for (;;) {
     memd_server::Req* r = nullptr;
