@@ -15,7 +15,7 @@
 // V(1,1)-cycle, FP64 throughout, the whole solve in one cooperative launch.
 // Every axis of n vertices coarsens to ceil(n / 2) (the even ones; on an odd
 // axis the last and the first vertex are both coarse and keep their link),
-// down to one vertex: linear interpolation, its transpose, and coarse link
+// down to at most 32 vertices: linear interpolation, its transpose, and coarse link
 // conductances from two fine links in series summed over the perpendicular
 // weights.  Gauss-Seidel by colours: two where every axis is even; an odd
 // ring needs a third for its last vertex, and the sum of the axes' colours
@@ -33,7 +33,7 @@
 // most kMgCtaSites vertices run in one CTA a right-hand side, which needs
 // CTA barriers only.  A whole system's setup (48^3, 2200 charges; 77^3, 10^4
 // charges): 8.7 and 27.1 ms with one launch a half sweep, host checks between
-// iterations, and aggregation with Jacobi on odd levels; 4.2 and 9.1 ms so.
+// iterations, and aggregation with Jacobi on odd levels; 3.8 and 8.7 ms so.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -50,12 +50,17 @@ namespace {
 constexpr int kMgThreads = 512;
 constexpr int kMgMaxLevels = 32;  // an axis has less than 2^30 vertices
 // Levels up to this size run in one CTA a right-hand side, in shared memory:
-// a phase of 6^3 vertices takes ~0.3 us there and ~2.2 us with a grid barrier;
+// a phase of 6^3 vertices takes ~0.9 us there and ~2.2 us with a grid barrier;
 // from 8^3 on the one SM's FP64 pipe is the slower (12^3 and below in one CTA
-// took 39 us a cycle, of 95, in a 48^3 solve).
-constexpr int kMgCtaSites = 343;
-constexpr int kMgCtaTotal = 700;  // of all such levels together (343 on one axis: 689)
-constexpr int kMgCtaLevels = 10;
+// took 39 us a cycle, of 95, in a 48^3 solve; 18 with 12^3 on the grid).
+constexpr int kMgCtaSites = 256;
+constexpr int kMgCtaTotal = 480;  // of all such levels together (256, 128, 64, 32 on one axis)
+constexpr int kMgCtaLevels = 4;
+// The first level of at most this many vertices is the last: solved exactly
+// by the inverse of its matrix, formed once a solve (a matrix-vector product
+// of 27 vertices takes ~0.4 us; sweeping it and the 2^3 level below took 14
+// phases of 0.9 us, latency of dependent FP64 operations, 70 cycles each).
+constexpr int kMgDirect = 32;
 constexpr int kMgGrid = 256;  // most CTAs
 constexpr int kMgQ = 12;     // most sums of one reduction
 constexpr int kMgSlots = 6;  // reductions in flight between two uses of a slot
@@ -264,73 +269,89 @@ __device__ __forceinline__ void restrict_to(const MgLv& F, const MgLv& C, int t0
     x[1] = 2 * I;
     y[1] = 2 * J;
     z[1] = 2 * K;
-    wx[1] = wy[1] = wz[1] = 1.0;
     axis_pair(I, F.n0, C.n0, x[0], x[2], wx[0], wx[2]);
     axis_pair(J, F.n1, C.n1, y[0], y[2], wy[0], wy[2]);
     axis_pair(K, F.n2, C.n2, z[0], z[2], wz[0], wz[2]);
-    double s[NR];
-#pragma unroll
-    for (int r = 0; r < NR; ++r) s[r] = 0.0;
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        const double wyz = mul_(wy[b], wz[c]);
-        const int row = F.n0 * (y[b] + F.n1 * z[c]);
-#pragma unroll
-        for (int r = 0; r < NR; ++r) {
-          const double* q = F.r + (r0 + r) * F.V + row;
-          if (two) {
-            // the residual is 0 on the odd vertices: half of the 27 drop out
-            if (((b + c) & 1) == 0)
-              s[r] = fma_(wyz, q[x[1]], s[r]);
-            else
-              s[r] = fma_(mul_(wyz, 0.5), add_(q[x[0]], q[x[2]]), s[r]);
-          } else {
-            double t = fma_(wx[0], q[x[0]], q[x[1]]);
-            t = fma_(wx[2], q[x[2]], t);
-            s[r] = fma_(wyz, t, s[r]);
-          }
-        }
-      }
     const bool c0 = first_colour(C, I, J, K);
     const double id = C.idg[v];
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-      C.f[(r0 + r) * C.V + v] = s[r];
-      C.phi[(r0 + r) * C.V + v] = c0 ? mul_(s[r], id) : 0.0;
+      const double* q = F.r + (r0 + r) * F.V;
+      auto row = [&](int b, int c) { return q + F.n0 * (y[b] + F.n1 * z[c]); };
+      double s;
+      if (two) {
+        // the residual is 0 on the odd vertices: the centre and the twelve
+        // diagonal neighbours remain
+        const double* c1 = row(1, 1);
+        double e = add_(add_(row(0, 1)[x[0]], row(0, 1)[x[2]]),
+                        add_(row(2, 1)[x[0]], row(2, 1)[x[2]]));
+        e = add_(e, add_(add_(row(1, 0)[x[0]], row(1, 0)[x[2]]),
+                         add_(row(1, 2)[x[0]], row(1, 2)[x[2]])));
+        e = add_(e, add_(add_(row(0, 0)[x[1]], row(2, 0)[x[1]]),
+                         add_(row(0, 2)[x[1]], row(2, 2)[x[1]])));
+        s = fma_(0.25, e, c1[x[1]]);
+      } else {
+        auto line = [&](int b, int c) {
+          const double* l = row(b, c);
+          return fma_(wx[2], l[x[2]], fma_(wx[0], l[x[0]], l[x[1]]));
+        };
+        auto plane = [&](int c) {
+          return fma_(wy[2], line(2, c), fma_(wy[0], line(0, c), line(1, c)));
+        };
+        s = fma_(wz[2], plane(2), fma_(wz[0], plane(0), plane(1)));
+      }
+      C.f[(r0 + r) * C.V + v] = s;
+      C.phi[(r0 + r) * C.V + v] = c0 ? mul_(s, id) : 0.0;
     }
   }
 }
 
-// phi += interpolated coarse correction, on every colour but the last (which
-// the first half sweep after it overwrites)
+// phi += interpolated coarse correction: a thread takes the (up to) eight
+// fine vertices 2 I + {0, 1} of a coarse one, which share their sums (and
+// run without divergence).  With two colours only the even ones: the first
+// half sweep after it overwrites the last colour.
 template <int NR>
 __device__ __forceinline__ void prolong(const MgLv& F, const MgLv& C, int t0, int stride, int r0) {
-  const int H = F.hx * F.n1 * F.n2;
-  for (int c = 0; c + 1 < F.nc; ++c)
-    for (int h = t0; h < H; h += stride) {
-      int i, j, k;
-      if (!colour_vertex(F, h, c, i, j, k)) continue;
-      const int v = i + F.n0 * (j + F.n1 * k);
-      const int I0 = i >> 1, J0 = j >> 1, K0 = k >> 1;
-      const int I1 = I0 + 1 == C.n0 ? 0 : I0 + 1, J1 = J0 + 1 == C.n1 ? 0 : J0 + 1,
-                K1 = K0 + 1 == C.n2 ? 0 : K0 + 1;
-      const bool ox = i & 1, oy = j & 1, oz = k & 1;
-      const double half = (ox ? 0.5 : 1.0) * (oy ? 0.5 : 1.0) * (oz ? 0.5 : 1.0);
-      const int r00 = C.n0 * (J0 + C.n1 * K0), r10 = C.n0 * (J1 + C.n1 * K0),
-                r01 = C.n0 * (J0 + C.n1 * K1), r11 = C.n0 * (J1 + C.n1 * K1);
+  const bool two = F.nc == 2 && F.n0 > 1 && F.n1 > 1 && F.n2 > 1;
+  for (int v = t0; v < C.V; v += stride) {
+    int I, J, K;
+    coords(C, v, I, J, K);
+    const int I1 = I + 1 == C.n0 ? 0 : I + 1, J1 = J + 1 == C.n1 ? 0 : J + 1,
+              K1 = K + 1 == C.n2 ? 0 : K + 1;
+    const int c00 = C.n0 * (J + C.n1 * K), c10 = C.n0 * (J1 + C.n1 * K),
+              c01 = C.n0 * (J + C.n1 * K1), c11 = C.n0 * (J1 + C.n1 * K1);
+    const int u = 2 * I + F.n0 * (2 * J + F.n1 * 2 * K);
+    const int sy = F.n0, sz = F.n0 * F.n1;
 #pragma unroll
-      for (int r = 0; r < NR; ++r) {
-        const double* e = C.phi + (r0 + r) * C.V;
-        auto line = [&](int row) { return ox ? add_(e[row + I0], e[row + I1]) : e[row + I0]; };
-        double t = line(r00);
-        if (oy) t = add_(t, line(r10));
-        if (oz) t = add_(t, oy ? add_(line(r01), line(r11)) : line(r01));
-        double* p = F.phi + (r0 + r) * F.V + v;
-        *p = fma_(half, t, *p);
+    for (int r = 0; r < NR; ++r) {
+      const double* e = C.phi + (r0 + r) * C.V;
+      double* p = F.phi + (r0 + r) * F.V + u;
+      const double q00 = e[c00 + I], q10 = e[c10 + I], q01 = e[c01 + I], q11 = e[c11 + I];
+      const double x00 = add_(q00, e[c00 + I1]), x10 = add_(q10, e[c10 + I1]),
+                   x01 = add_(q01, e[c01 + I1]);
+      if (two) {
+        const double a0 = p[0], a1 = p[1 + sy], a2 = p[1 + sz], a3 = p[sy + sz];
+        p[0] = add_(a0, q00);
+        p[1 + sy] = fma_(0.25, add_(x00, x10), a1);
+        p[1 + sz] = fma_(0.25, add_(x00, x01), a2);
+        p[sy + sz] = fma_(0.25, add_(add_(q00, q10), add_(q01, q11)), a3);
+        continue;
+      }
+      const bool ox = 2 * I + 1 < F.n0, oy = 2 * J + 1 < F.n1, oz = 2 * K + 1 < F.n2;
+      const double x11 = add_(q11, e[c11 + I1]);
+      const double y0 = add_(q00, q10), y1 = add_(x00, x10);
+      p[0] = add_(p[0], q00);
+      if (ox) p[1] = fma_(0.5, x00, p[1]);
+      if (oy) p[sy] = fma_(0.5, y0, p[sy]);
+      if (ox && oy) p[1 + sy] = fma_(0.25, y1, p[1 + sy]);
+      if (oz) {
+        p[sz] = fma_(0.5, add_(q00, q01), p[sz]);
+        if (ox) p[1 + sz] = fma_(0.25, add_(x00, x01), p[1 + sz]);
+        if (oy) p[sy + sz] = fma_(0.25, add_(y0, add_(q01, q11)), p[sy + sz]);
+        if (ox && oy) p[1 + sy + sz] = fma_(0.125, add_(y1, add_(x01, x11)), p[1 + sy + sz]);
       }
     }
+  }
 }
 
 // conductance of link d of coarse vertex (I, J, K): the fine links in series
@@ -444,6 +465,52 @@ __device__ __forceinline__ void total_sums(const double* part, int slot, double 
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < NQ; ++q) x[q] = tot[q];
+}
+
+// The inverse of a level's matrix plus a multiple of the all-ones matrix
+// (which acts on the constants alone: right-hand sides have none), by
+// Gauss-Jordan steps in place; the whole CTA calls it.
+__device__ void invert_level(const MgLv& L, double* A) {
+  const int n = L.V, U = n * n;
+  const double shift = L.dg[0] / n;
+  for (int t = threadIdx.x; t < U; t += kMgThreads) {
+    const int u = t / n, v = t - u * n;
+    double y = u == v ? add_(L.dg[u], shift) : shift;
+    if (u != v) {
+      // the links from u to v and from v to u (on an axis of two, both)
+      int i, j, k;
+      coords(L, u, i, j, k);
+      const Nb b = neighbours(L, u, i, j, k);
+      coords(L, v, i, j, k);
+      const Nb c = neighbours(L, v, i, j, k);
+      const int bu[3] = {b.xp, b.yp, b.zp}, bv[3] = {c.xp, c.yp, c.zp};
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        if (bu[d] == v) y = sub_(y, L.w[d * n + u]);
+        if (bv[d] == u) y = sub_(y, L.w[d * n + v]);
+      }
+    }
+    A[t] = y;
+  }
+  __syncthreads();
+  for (int k = 0; k < n; ++k) {
+    const double p = 1.0 / A[k * n + k];
+    for (int t = threadIdx.x; t < U; t += kMgThreads) {
+      const int i = t / n, j = t - i * n;
+      if (i != k && j != k) A[t] = fma_(-mul_(A[i * n + k], p), A[k * n + j], A[t]);
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < 2 * n; t += kMgThreads) {
+      const int i = t < n ? t : t - n;
+      if (i == k) continue;
+      if (t < n)
+        A[i * n + k] = mul_(-A[i * n + k], p);
+      else
+        A[k * n + i] = mul_(A[k * n + i], p);
+    }
+    if (threadIdx.x == 0) A[k * n + k] = p;
+    __syncthreads();
+  }
 }
 
 // The whole solve for NR right-hand sides.
@@ -580,7 +647,10 @@ __global__ void __launch_bounds__(kMgThreads, 2) k_mg_solve(const __grid_constan
   // the levels of the one-CTA part: coefficients into shared memory
   __shared__ double s_mem[8 * kMgCtaTotal];
   __shared__ MgLv s_lv[kMgCtaLevels];
+  __shared__ double s_inv[kMgDirect * kMgDirect];
   if ((int)blockIdx.x < NR) {
+    const MgLv& D = a.lv[a.nl - 1];
+    invert_level(D, s_inv);
     int at = 0;
     for (int l = a.nlg; l < a.nl; ++l) {
       const MgLv& F = a.lv[l];
@@ -645,6 +715,23 @@ __global__ void __launch_bounds__(kMgThreads, 2) k_mg_solve(const __grid_constan
         residual<1>(F, t, kMgThreads, 0);
         __syncthreads();
         restrict_to<1>(F, s_lv[l + 1], t, kMgThreads, 0);
+        __syncthreads();
+      }
+      {
+        // four threads a row of the inverse
+        const MgLv& D = s_lv[nc - 1];
+        const int v = t >> 2, n = D.V;
+        double y = 0.0;
+        if (v < n)
+          for (int j = t & 3; j < n; j += 4) y = fma_(s_inv[v * n + j], D.f[j], y);
+        if (t < 4 * kMgDirect) {
+          y = add_(y, __shfl_xor_sync(0xffffffffu, y, 1));
+          y = add_(y, __shfl_xor_sync(0xffffffffu, y, 2));
+        }
+        if (v < n && (t & 3) == 0) {
+          D.phi[v] = y;
+          if (a.nl == 1) one = mul_(D.f[v], y);
+        }
         __syncthreads();
       }
       for (int l = nc - 2; l >= 0; --l) {
@@ -934,7 +1021,7 @@ struct MgPlan {
       L.dh = fast_div((unsigned)L.hx);
       at.push_back(words);
       words += (size_t)V * (5 + 3 * nr);
-      if (V == 1) break;
+      if (V <= kMgDirect) break;
       for (int d = 0; d < 3; ++d) n[d] = (n[d] + 1) / 2;
     }
     a.nl = nl + 1;
