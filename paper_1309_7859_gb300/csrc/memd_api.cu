@@ -990,6 +990,7 @@ memd_status memd_init_field(memd_ctx* c, int64_t n, const double* pos, const int
   if (tot % m.V != 0)
     return fail(c, MEMD_ERR_INVALID, "non-neutral system needs an integer background per vertex");
   const long long bg = (long long)(tot / m.V);
+  c->bg = bg;
   drop_graphs(c);
   harvest_timing(c);
   CK(cudaStreamSynchronize(st));
@@ -1309,36 +1310,27 @@ memd_status memd_energy(memd_ctx* c, memd_energy_terms* out) {
   double* sc = scal(c);
   const StepParams sp = step_params(c, 0, 0, 0);
   launch_field_energy(m, c->prec, c->D(), c->B(), c->ie, sp.coefB, part, part + R, st);
-  launch_finish(part, 0, sc + 8, st);
-  launch_finish(part + R, 0, sc + 9, st);
   launch_particle_energy(m, sp, c->P, c->ie64, part + 2 * R, part + 3 * R, st);
-  launch_finish(part + 2 * R, 0, sc + 10, st);
-  launch_finish(part + 3 * R, 0, sc + 11, st);
-  long long qtot = 0;
-  long long* Q = (long long*)dalloc(c, sizeof(long long) * m.V + 64);
+  launch_finish(part, 0, sc + 8, st, 4);
+  long long* Q = (long long*)dalloc(c, sizeof(long long) * m.V);
   if (!Q) return fail(c, MEMD_ERR_OOM, "energy scratch");
-  unsigned long long* mism = (unsigned long long*)(Q + m.V);
-  // background of a non-neutral system, from the valences on the device
-  std::vector<int> hq(c->P.n > 0 ? c->P.n : 1);
-  if (c->P.n > 0)
-    CK(cudaMemcpyAsync(hq.data(), c->P.q, c->P.n * sizeof(int), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  for (int64_t p = 0; p < c->P.n; ++p) qtot += hq[p];
-  const long long bg = (long long)(((__int128)qtot << 48) / m.V);
-  launch_cic(m, c->P, Q, bg, st);
+  launch_cic(m, c->P, Q, c->bg, st);
+  unsigned long long* mism = (unsigned long long*)(sc + 13);
   CK(cudaMemsetAsync(mism, 0, sizeof(unsigned long long), st));
   launch_gauss_check(m, c->prec, c->D(), c->Lg, Q, m.a * m.a, part, mism, st);
   launch_finish(part, 1, sc + 12, st);
   CKL();
-  double h[5];
-  unsigned long long bad = 0;
-  long long Pl[3], step = 0;
-  CK(cudaMemcpyAsync(h, sc + 8, 5 * sizeof(double), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(&bad, mism, sizeof(bad), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(Pl, c->ds->Plast, sizeof(Pl), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(&step, &c->ds->step, sizeof(step), cudaMemcpyDeviceToHost, st));
+  // the sums, the residual and the mismatches; then P and the step counter,
+  // which lie together in the state
+  double h[6];
+  long long w[4];
+  CK(cudaMemcpyAsync(h, sc + 8, 6 * sizeof(double), cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(w, c->ds->Plast, sizeof(w), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   dfree(c, Q);
+  unsigned long long bad = 0;
+  std::memcpy(&bad, &h[5], sizeof(bad));
+  const long long *Pl = w, step = w[3];
   const double a3 = m.a * m.a * m.a;
   out->electric = h[0] * a3;
   out->magnetic = h[1] * 0.5 * c->c * c->c * a3;
@@ -1647,19 +1639,27 @@ memd_status memd_get_fields(memd_ctx* c, double* D, double* B, int64_t* Lg) {
   }
   const size_t n3 = 3 * (size_t)c->mesh.V;
   const cudaStream_t st = c->stream;
-  double* tmp = (double*)dalloc(c, n3 * sizeof(double));
-  if (!tmp) return fail(c, MEMD_ERR_OOM, "get_fields scratch");
-  if (D) {
-    launch_widen(c->prec, tmp, c->D(), (int64_t)n3, st);
-    CK(cudaMemcpyAsync(D, tmp, n3 * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
+  // one scratch of 3 V words for what has to be converted: FP32 fields, and
+  // the ledger's order (without scratch the copy engine gathers the ledger)
+  double* tmp = c->prec == MEMD_FP32 || Lg ? (double*)dalloc(c, n3 * sizeof(double)) : nullptr;
+  if (!tmp && c->prec == MEMD_FP32 && (D || B)) return fail(c, MEMD_ERR_OOM, "get_fields scratch");
+  auto field = [&](double* out, const void* dev) {
+    const void* src = dev;
+    if (c->prec == MEMD_FP32) {
+      launch_widen(c->prec, tmp, dev, (int64_t)n3, st);
+      src = tmp;
+    }
+    return cudaMemcpyAsync(out, src, n3 * sizeof(double), cudaMemcpyDeviceToHost, st);
+  };
+  if (D) CK(field(D, c->D()));
+  if (B) CK(field(B, c->B()));
+  if (Lg && tmp) {
+    launch_ledger_pack(c->mesh, c->Lg, (long long*)tmp, st);
+    CK(cudaMemcpyAsync(Lg, tmp, n3 * sizeof(double), cudaMemcpyDeviceToHost, st));
+  } else if (Lg) {
+    CK(ledger_to_host(c, Lg, st));
   }
-  if (B) {
-    launch_widen(c->prec, tmp, c->B(), (int64_t)n3, st);
-    CK(cudaMemcpyAsync(B, tmp, n3 * sizeof(double), cudaMemcpyDeviceToHost, st));
-    CK(cudaStreamSynchronize(st));
-  }
-  if (Lg) CK(ledger_to_host(c, Lg, st));
+  CKL();
   CK(cudaStreamSynchronize(st));
   dfree(c, tmp);
   return MEMD_OK;
@@ -1674,19 +1674,23 @@ memd_status memd_set_fields(memd_ctx* c, const double* D, const double* B, const
   }
   const size_t n3 = 3 * (size_t)c->mesh.V;
   const cudaStream_t st = c->stream;
-  double* tmp = (double*)dalloc(c, n3 * sizeof(double));
-  if (!tmp) return fail(c, MEMD_ERR_OOM, "set_fields scratch");
-  if (D) {
-    CK(cudaMemcpyAsync(tmp, D, n3 * sizeof(double), cudaMemcpyHostToDevice, st));
-    launch_cast(c->prec, c->D(), tmp, (int64_t)n3, st);
-    CK(cudaStreamSynchronize(st));
+  double* tmp = c->prec == MEMD_FP32 || Lg ? (double*)dalloc(c, n3 * sizeof(double)) : nullptr;
+  if (!tmp && c->prec == MEMD_FP32 && (D || B)) return fail(c, MEMD_ERR_OOM, "set_fields scratch");
+  auto field = [&](void* dev, const double* in) {
+    if (c->prec != MEMD_FP32)
+      return cudaMemcpyAsync(dev, in, n3 * sizeof(double), cudaMemcpyHostToDevice, st);
+    const cudaError_t e = cudaMemcpyAsync(tmp, in, n3 * sizeof(double), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) launch_cast(c->prec, dev, tmp, (int64_t)n3, st);
+    return e;
+  };
+  if (D) CK(field(c->D(), D));
+  if (B) CK(field(c->B(), B));
+  if (Lg && tmp) {
+    CK(cudaMemcpyAsync(tmp, Lg, n3 * sizeof(double), cudaMemcpyHostToDevice, st));
+    launch_ledger_unpack(c->mesh, (const long long*)tmp, c->Lg, 0, st);
+  } else if (Lg) {
+    CK(ledger_from_host(c, Lg, st));
   }
-  if (B) {
-    CK(cudaMemcpyAsync(tmp, B, n3 * sizeof(double), cudaMemcpyHostToDevice, st));
-    launch_cast(c->prec, c->B(), tmp, (int64_t)n3, st);
-    CK(cudaStreamSynchronize(st));
-  }
-  if (Lg) CK(ledger_from_host(c, Lg, st));
   CKL();
   CK(cudaStreamSynchronize(st));
   dfree(c, tmp);
@@ -1733,27 +1737,45 @@ memd_status memd_save_state(memd_ctx* c, void* buf, int64_t bytes) {
     h.box[d] = c->mesh.L[d];
   }
   h.n = (int64_t)n;
-  CK(cudaMemcpyAsync(&h.step, &c->ds->step, sizeof(long long), cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(h.Plast, c->ds->Plast, 3 * sizeof(long long), cudaMemcpyDeviceToHost, st));
   char* p = (char*)buf + sizeof(StateHeader);
   bool ok = true;
   auto get = [&](const void* src, size_t b) {
     if (b && cudaMemcpyAsync(p, src, b, cudaMemcpyDeviceToHost, st) != cudaSuccess) ok = false;
     p += b;
   };
+  // the ledger and the particle arrays packed into one block (their order on
+  // the host); without memory for it, array by array
+  const size_t tail = V3 * 8 + n * 120;
+  char* pack = (char*)dalloc(c, tail);
+  if (pack) {
+    launch_ledger_pack(c->mesh, c->Lg, (long long*)pack, st);
+    launch_state_particles(true, c->P, pack + V3 * 8, st);
+    if (cudaGetLastError() != cudaSuccess) ok = false;
+  }
   get(c->D(), V3 * es);
   get(c->B(), V3 * es);
-  if (ok && ledger_to_host(c, p, st) != cudaSuccess) ok = false;
-  p += V3 * 8;
-  get(c->P.x, 3 * n * 8);
-  get(c->P.v, 3 * n * 8);
-  get(c->P.F, 3 * n * 8);
-  get(c->P.Ft, 3 * n * 8);
-  get(c->P.img, 3 * n * 4);
-  get(c->P.q, n * 4);
-  get(c->P.m, n * 8);
+  if (pack) {
+    get(pack, tail);
+  } else {
+    if (ok && ledger_to_host(c, p, st) != cudaSuccess) ok = false;
+    p += V3 * 8;
+    get(c->P.x, 3 * n * 8);
+    get(c->P.v, 3 * n * 8);
+    get(c->P.F, 3 * n * 8);
+    get(c->P.Ft, 3 * n * 8);
+    get(c->P.img, 3 * n * 4);
+    get(c->P.q, n * 4);
+    get(c->P.m, n * 8);
+  }
+  // P and the step counter lie together
+  long long w[4] = {0, 0, 0, 0};
+  if (ok && cudaMemcpyAsync(w, c->ds->Plast, sizeof(w), cudaMemcpyDeviceToHost, st) != cudaSuccess)
+    ok = false;
+  if (cudaStreamSynchronize(st) != cudaSuccess) ok = false;
+  dfree(c, pack);
   if (!ok) return fail(c, MEMD_ERR_CUDA, "state copy");
-  CK(cudaStreamSynchronize(st));
+  for (int d = 0; d < 3; ++d) h.Plast[d] = w[d];
+  h.step = w[3];
   std::memcpy(buf, &h, sizeof(h));
   return check_err(c);
 }
@@ -1771,6 +1793,7 @@ memd_status memd_load_state(memd_ctx* c, const void* buf, int64_t bytes) {
       h.box[1] != c->mesh.L[1] || h.box[2] != c->mesh.L[2])
     return fail(c, MEMD_ERR_INVALID, "saved state of another mesh, precision or particle count");
   if (bytes < memd_state_bytes(c)) return fail(c, MEMD_ERR_INVALID, "state buffer too small");
+  long long qtot = 0;
   {
     // the particle arrays are checked before anything is copied: a saved
     // state holds folded positions (the deposition indexes cells by them),
@@ -1793,8 +1816,10 @@ memd_status memd_load_state(memd_ctx* c, const void* buf, int64_t bytes) {
       if (qi > 32767 || qi < -32767) return fail(c, MEMD_ERR_INVALID, "saved valence out of range");
       if (!(mi > 0.0) || !std::isfinite(mi))
         return fail(c, MEMD_ERR_INVALID, "saved mass not positive and finite");
+      qtot += qi;
     }
   }
+  const long long bg = (long long)(((__int128)qtot << 48) / c->mesh.V);
   CK(cudaSetDevice(c->device));
   const cudaStream_t st = c->stream;
   drop_graphs(c);
@@ -1809,27 +1834,36 @@ memd_status memd_load_state(memd_ctx* c, const void* buf, int64_t bytes) {
   };
   put(c->D(), V3 * es);
   put(c->B(), V3 * es);
-  if (ok && ledger_from_host(c, p, st) != cudaSuccess) ok = false;
-  p += V3 * 8;
-  put(c->P.x, 3 * n * 8);
-  put(c->P.v, 3 * n * 8);
-  put(c->P.F, 3 * n * 8);
-  put(c->P.Ft, 3 * n * 8);
-  put(c->P.img, 3 * n * 4);
-  put(c->P.q, n * 4);
-  put(c->P.m, n * 8);
-  if (!ok) return fail(c, MEMD_ERR_CUDA, "state copy");
   // transfers none pending, the step counter and last dipole of the saved
   // state, the accumulators clear; the per-particle constants are formed
   // again from the masses at the next step
-  CK(clear_transfers(c, c->Tb, st));
-  if (c->Tb2) CK(cudaMemsetAsync(c->Tb2, 0, kLT * 3 * c->mesh.V * sizeof(long long), st));
+  const size_t tail = V3 * 8 + n * 120;
+  char* pack = (char*)dalloc(c, tail);
+  if (pack) {
+    put(pack, tail);
+    launch_ledger_unpack(c->mesh, (const long long*)pack, c->Lg, 1, st);
+    launch_state_particles(false, c->P, pack + V3 * 8, st);
+  } else {
+    if (ok && ledger_from_host(c, p, st) != cudaSuccess) ok = false;
+    p += V3 * 8;
+    put(c->P.x, 3 * n * 8);
+    put(c->P.v, 3 * n * 8);
+    put(c->P.F, 3 * n * 8);
+    put(c->P.Ft, 3 * n * 8);
+    put(c->P.img, 3 * n * 4);
+    put(c->P.q, n * 4);
+    put(c->P.m, n * 8);
+    if (ok && clear_transfers(c, c->Tb, st) != cudaSuccess) ok = false;
+  }
+  if (ok && c->Tb2 &&
+      cudaMemsetAsync(c->Tb2, 0, kLT * 3 * c->mesh.V * sizeof(long long), st) != cudaSuccess)
+    ok = false;
+  launch_state_counters(c->ds, h.step, reinterpret_cast<const long long*>(h.Plast), st);
+  if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) ok = false;
+  dfree(c, pack);
+  if (!ok) return fail(c, MEMD_ERR_CUDA, "state copy");
   c->pending = false;
-  CK(cudaMemcpyAsync(&c->ds->step, &h.step, sizeof(long long), cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(c->ds->Plast, h.Plast, 3 * sizeof(long long), cudaMemcpyHostToDevice, st));
-  CK(cudaMemsetAsync(c->ds->Pacc, 0, sizeof(c->ds->Pacc), st));
-  CK(cudaMemsetAsync(&c->ds->ticket, 0, sizeof(unsigned int), st));
-  CK(cudaStreamSynchronize(st));
+  c->bg = bg;
   c->sig_ready = false;
   c->gen += 1;
   return check_err(c);

@@ -47,6 +47,7 @@ struct memd_ctx {
   double* psi = nullptr;        // cell-problem potentials of the scalar solver (3V), or null
   double* pin = nullptr;        // memd_set_particles staging (3n doubles + 3n ints)
   long long* Tb2 = nullptr;     // second transfer buffer of the single-launch step
+  long long bg = 0;             // neutralising background a vertex (units of e 2^-48)
   bool pending = false;         // transfers of the last single-launch step not yet applied
   // particles
   Particles P{};

@@ -222,8 +222,8 @@ void launch_dot(const double* x, const double* y, int64_t n, double* partial, cu
 // partial[b] = block max of |x[i]| (|x[i] y[i]| when y is given)
 void launch_absmax(const double* x, const double* y, int64_t n, double* partial,
                    cudaStream_t st);
-// out[0] = op over partial[0..reduce_blocks())  (op 0 = sum, 1 = max)
-void launch_finish(const double* partial, int op, double* out, cudaStream_t st);
+// out[k] = op over partial[k reduce_blocks() ..], k < count (op 0 = sum, 1 = max)
+void launch_finish(const double* partial, int op, double* out, cudaStream_t st, int count = 1);
 
 // ------------------------------------------------------- particle kernels
 // (memd_particles.cu, built with -fmad=false)
@@ -279,6 +279,13 @@ cudaError_t launch_step_coop(const Mesh& m, int prec, const StepParams& sp, Part
                              const void* Din, const void* Bin, const void* ie, void* Dout,
                              void* Bout, const double* ie64, long long* Tprev, long long* Tcur,
                              long long* Lg, DevState* ds, int grid, int zchunk, cudaStream_t st);
+// a state's host copies (memd_setup.cu): the ledger's component-major words
+// (3 V) and the particle arrays in a saved state's order (120 bytes a charge)
+void launch_ledger_pack(const Mesh& m, const long long* Lg, long long* out, cudaStream_t st);
+void launch_ledger_unpack(const Mesh& m, const long long* in, long long* Lg, int clear,
+                          cudaStream_t st);
+void launch_state_particles(bool pack, Particles p, void* io, cudaStream_t st);
+void launch_state_counters(DevState* ds, long long step, const long long P[3], cudaStream_t st);
 void launch_fold_init(const Mesh& m, Particles p, const double* pos_in, const int* img_in,
                       unsigned int* err, cudaStream_t st);
 // byte offsets of the host I/O block of n particles (memd_step_io)

@@ -384,7 +384,7 @@ class Memd:
                     "memd_step")
 
     def forces(self, out=None):
-        out = np.zeros((self.n, 3)) if out is None else out
+        out = np.empty((self.n, 3)) if out is None else out
         self._check(self._L.memd_forces(self._h, _ptr(out, C.c_double)), "memd_forces")
         return out
 
@@ -399,9 +399,9 @@ class Memd:
         return e.as_dict()
 
     def particles(self):
-        x = np.zeros((self.n, 3))
-        v = np.zeros((self.n, 3))
-        img = np.zeros((self.n, 3), dtype=np.int32)
+        x = np.empty((self.n, 3))
+        v = np.empty((self.n, 3))
+        img = np.empty((self.n, 3), dtype=np.int32)
         self._check(self._L.memd_get_particles(self._h, _ptr(x, C.c_double), _ptr(v, C.c_double),
                                                _ptr(img, C.c_int32)), "memd_get_particles")
         return x, v, img
@@ -443,7 +443,7 @@ class Memd:
     def save_state(self):
         """The whole dynamical state as bytes (memd_save_state)."""
         nb = self._L.memd_state_bytes(self._h)
-        buf = np.zeros(nb, dtype=np.uint8)
+        buf = np.empty(nb, dtype=np.uint8)
         self._check(self._L.memd_save_state(self._h, buf.ctypes.data, nb), "memd_save_state")
         return buf
 
@@ -479,9 +479,9 @@ class Memd:
 
     def fields(self):
         Nx, Ny, Nz = self.mesh
-        D = np.zeros((3, Nz, Ny, Nx))
-        B = np.zeros((3, Nz, Ny, Nx))
-        Lg = np.zeros((3, Nz, Ny, Nx), dtype=np.int64)
+        D = np.empty((3, Nz, Ny, Nx))   # every word is written (a failure raises)
+        B = np.empty((3, Nz, Ny, Nx))
+        Lg = np.empty((3, Nz, Ny, Nx), dtype=np.int64)
         self._check(self._L.memd_get_fields(self._h, _ptr(D, C.c_double), _ptr(B, C.c_double),
                                             _ptr(Lg, C.c_int64)), "memd_get_fields")
         return D, B, Lg
@@ -500,7 +500,7 @@ class Memd:
         """memd_eps_from_density: the permittivity from the local |q| density
         (vertex values returned as [Nz, Ny, Nx])."""
         rule = (C.c_double * 5)(eps0, slope, eps_lo, eps_hi, sigma)
-        out = np.zeros(self.V, dtype=np.float64)
+        out = np.empty(self.V, dtype=np.float64)
         self._check(self._L.memd_eps_from_density(self._h, C.byref(rule), 1 if relax else 0,
                                                   _ptr(out, C.c_double)), "memd_eps_from_density")
         Nx, Ny, Nz = self.mesh
@@ -527,7 +527,7 @@ class Memd:
 
     def setup(self):
         Nx, Ny, Nz = self.mesh
-        ie = np.zeros((3, Nz, Ny, Nx))
+        ie = np.empty((3, Nz, Ny, Nx))
         G = np.zeros(8)
         M = np.zeros((3, 3))
         self._check(self._L.memd_get_setup(self._h, _ptr(ie, C.c_double), _ptr(G, C.c_double),
@@ -735,8 +735,8 @@ class Server:
 
     def result(self, rid):
         n = self.n_of[rid]
-        x, v, f = np.zeros((n, 3)), np.zeros((n, 3)), np.zeros((n, 3))
-        img = np.zeros((n, 3), dtype=np.int32)
+        x, v, f = np.empty((n, 3)), np.empty((n, 3)), np.empty((n, 3))
+        img = np.empty((n, 3), dtype=np.int32)
         e = EnergyTerms()
         self._err(self._L.memd_server_result(self._h, int(rid), _ptr(x, C.c_double),
                                              _ptr(v, C.c_double), _ptr(img, C.c_int32),
