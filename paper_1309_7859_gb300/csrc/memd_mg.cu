@@ -33,11 +33,10 @@
 // most kMgCtaSites vertices run in one CTA a right-hand side, which needs
 // CTA barriers only.  A whole system's setup (48^3, 2200 charges; 77^3, 10^4
 // charges): 8.7 and 27.1 ms with one launch a half sweep, host checks between
-// iterations, and aggregation with Jacobi on odd levels; 3.8 and 8.7 ms so.
+// iterations, and aggregation with Jacobi on odd levels; 3.6 and 8.2 ms so.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <mutex>
 #include <vector>
 
 #include "memd_ctx.cuh"
@@ -47,6 +46,9 @@ namespace memd {
 
 namespace {
 
+// 512 threads with all the registers they take: held to 64 registers the
+// three-right-hand-side solve spills (48^3 and 77^3 setups 3.77 and 8.60 ms
+// against 3.63 and 8.19), 1024 threads only add to the barriers (4.25, 9.09).
 constexpr int kMgThreads = 512;
 constexpr int kMgMaxLevels = 32;  // an axis has less than 2^30 vertices
 // Levels up to this size run in one CTA a right-hand side, in shared memory:
@@ -437,10 +439,10 @@ __device__ __forceinline__ void share_sums(double* part, int slot, const double 
     if (lane == 0) sh[wp][q] = s;
   }
   __syncthreads();
-  static_assert(kMgThreads == 512, "sixteen warps");
+  constexpr int NW = kMgThreads / 32;
   if (wp < NQ) {
-    double s = lane < 16 ? sh[lane][wp] : 0.0;
-    for (int o = 8; o > 0; o >>= 1) s = add_(s, __shfl_down_sync(0xffffffffu, s, o));
+    double s = lane < NW ? sh[lane][wp] : 0.0;
+    for (int o = NW / 2; o > 0; o >>= 1) s = add_(s, __shfl_down_sync(0xffffffffu, s, o));
     if (lane == 0) part[((int64_t)slot * kMgQ + wp) * gridDim.x + blockIdx.x] = s;
   }
 }
@@ -522,7 +524,7 @@ __device__ void invert_level(const MgLv& L, double* A) {
 // its rounding floor and the residual grows again (to 100 times its least
 // value), when that least value was below 100 tol |f|.
 template <int NR, int MODE>
-__global__ void __launch_bounds__(kMgThreads, 2) k_mg_solve(const __grid_constant__ MgArgs a) {
+__global__ void __launch_bounds__(kMgThreads) k_mg_solve(const __grid_constant__ MgArgs a) {
   __shared__ double sh[kMgThreads / 32][kMgQ];
   __shared__ double tot[2][kMgQ];
   __shared__ int s_ok;
@@ -953,26 +955,13 @@ __global__ void __launch_bounds__(kMgThreads, 2) k_mg_solve(const __grid_constan
 }
 
 // ---------------------------------------------------------------- host
-// One of these launches is in flight on a device at a time, whatever streams
-// and threads they come from: each waits (on its stream) for the one before,
-// so two grids never hold SMs that the other's barriers wait for.  A grid
-// takes half an SM's registers, which leaves the room of a single-launch
-// step's CTA beside it.
-struct Gate {
-  std::mutex mu;
-  cudaEvent_t ev = nullptr;
-};
-constexpr int kMgDevices = 64;
-Gate g_gate[kMgDevices];
-
+// A cooperative grid starts when all of it fits, whatever else is resident or
+// queued on other streams (checked on GB300: two grids that each need every
+// SM, the second at a higher priority, while a third kernel holds half of
+// them: neither started in part), so concurrent solves and single-launch
+// steps never hold SMs that another's barriers wait for.
 template <int NR, int MODE>
-cudaError_t launch_solve(const MgArgs& a, int device, int grid, cudaStream_t st) {
-  if (device < 0 || device >= kMgDevices) return cudaErrorInvalidDevice;
-  Gate& g = g_gate[device];
-  std::lock_guard<std::mutex> lock(g.mu);
-  cudaError_t e = g.ev ? cudaStreamWaitEvent(st, g.ev, 0)
-                       : cudaEventCreateWithFlags(&g.ev, cudaEventDisableTiming);
-  if (e != cudaSuccess) return e;
+cudaError_t launch_solve(const MgArgs& a, int grid, cudaStream_t st) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)grid, 1, 1);
   cfg.blockDim = dim3(kMgThreads, 1, 1);
@@ -982,9 +971,7 @@ cudaError_t launch_solve(const MgArgs& a, int device, int grid, cudaStream_t st)
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, k_mg_solve<NR, MODE>, a);
-  if (e == cudaSuccess) e = cudaEventRecord(g.ev, st);
-  return e;
+  return cudaLaunchKernelEx(&cfg, k_mg_solve<NR, MODE>, a);
 }
 
 // The levels and their scratch for NR right-hand sides, one block of memory.
@@ -1063,7 +1050,7 @@ struct MgPlan {
   memd_status run(memd_ctx* c, MgOut& h) {
     const cudaStream_t st = c->stream;
     if (cudaMemsetAsync(block, 0, zero_bytes, st) != cudaSuccess ||
-        launch_solve<NR, MODE>(a, c->device, grid, st) != cudaSuccess ||
+        launch_solve<NR, MODE>(a, grid, st) != cudaSuccess ||
         cudaMemcpyAsync(&h, a.out, sizeof(h), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
       return MEMD_ERR_CUDA;
