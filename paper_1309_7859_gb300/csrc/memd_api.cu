@@ -1071,9 +1071,11 @@ memd_status memd_init_field(memd_ctx* c, int64_t n, const double* pos, const int
       launch_cast(c->prec, c->D(), D64, 3 * m.V, st);
       CK(cudaMemsetAsync(c->B(), 0, 3 * m.V * esz(c), st));
       CK(clear_transfers(c, c->Tb, st));
-      if (c->Tb2) CK(cudaMemsetAsync(c->Tb2, 0, kLT * 3 * m.V * sizeof(long long), st));
+      if (c->Tb2) CK(cudaMemsetAsync(c->Tb2, 0, kCoopSlots * 3 * m.V * sizeof(long long), st));
       c->pending = false;
+      c->tslot = 0;
       CK(cudaMemsetAsync(&c->ds->ticket, 0, sizeof(unsigned int), st));
+      CK(cudaMemsetAsync(c->ds->Pc, 0, sizeof(c->ds->Pc), st));
       const StepParams sp = step_params(c, 0, 0.0, 0.0);
       launch_particle_constants(sp, c->P, st);
       launch_gather(m, c->prec, sp, c->P, c->D(), c->ie, c->ie64, c->ds, 0, 1, st);
@@ -1130,23 +1132,33 @@ static memd_status record_step(memd_ctx* c, const StepParams& sp, int par, bool 
   return MEMD_OK;
 }
 
-// transfer buffer of buffer parity q of the single-launch step, which leaves
-// the transfers of its move, not yet applied, in the buffer of the parity it
-// wrote: transfer words only, component major (tw_index with cmV = V), the
-// two buffers one after the other in Tb2 (the graph step uses the pairs of
-// Tb, and applies them at once)
-static long long* tbuf(memd_ctx* c, int q) { return c->Tb2 + q * 3 * c->mesh.V; }
+// transfer slot w of the single-launch step, which leaves the transfers of
+// its last move, not yet applied, in slot tslot: transfer words only,
+// component major (tw_index with cmV = V), the slots one after the other in
+// Tb2 (the graph step uses the pairs of Tb, and applies them at once)
+static long long* tbuf(memd_ctx* c, int w) { return c->Tb2 + w * 3 * c->mesh.V; }
 
-// the whole step as one cooperative launch (same kernels' device functions)
-static memd_status record_step_coop(memd_ctx* c, const StepParams& sp, int par, bool timed) {
+// nsteps steps as one cooperative launch; io: the host block that its last step fills (and its first
+// one reads, io_load)
+static memd_status run_steps_coop(memd_ctx* c, const StepParams& sp, bool timed, int nsteps,
+                                  void* io = nullptr, int io_load = 0) {
   const cudaStream_t st = c->stream;
+  CoopBufs buf;
+  for (int q = 0; q < 2; ++q) {
+    buf.D[q] = c->Dbuf[q];
+    buf.B[q] = c->Bbuf[q];
+  }
+  for (int w = 0; w < kCoopSlots; ++w) buf.T[w] = tbuf(c, w);
   if (timed) CK(record_timing_event(c->ev0, st));
-  const cudaError_t e = launch_step_coop(
-      c->mesh, c->prec, sp, c->P, c->Dbuf[par], c->Bbuf[par], c->ie, c->Dbuf[par ^ 1],
-      c->Bbuf[par ^ 1], c->ie64, tbuf(c, par), tbuf(c, par ^ 1), c->Lg, c->ds, c->coop_grid,
-      coop_zchunk(c->mesh, c->coop_grid), st);
+  const cudaError_t e =
+      launch_step_coop(c->mesh, c->prec, sp, c->P, buf, c->ie, c->ie64, c->Lg, c->ds, c->coop_grid,
+                       c->cur, c->tslot, nsteps, io, io_load, st);
   if (e != cudaSuccess) return fail(c, MEMD_ERR_CUDA, cudaGetErrorString(e));
   if (timed) CK(record_timing_event(c->ev1, st));
+  c->timing_pending = timed;
+  c->cur ^= nsteps & 1;
+  c->tslot = (c->tslot + nsteps) % kCoopSlots;
+  c->pending = true;
   return MEMD_OK;
 }
 
@@ -1157,7 +1169,7 @@ static memd_status record_step_coop(memd_ctx* c, const StepParams& sp, int par, 
 // the state.  (C++ linkage: used by the batch, not part of the C ABI.)
 memd_status memd_flush(memd_ctx* c) {
   if (!c->pending) return MEMD_OK;
-  launch_apply(c->mesh, c->prec, c->P, tbuf(c, c->cur), c->Lg, c->D(),
+  launch_apply(c->mesh, c->prec, c->P, tbuf(c, c->tslot), c->Lg, c->D(),
                std::ldexp(1.0, -48) / (c->mesh.a * c->mesh.a), c->stream, c->mesh.V);
   c->pending = false;
   if (cudaGetLastError() != cudaSuccess) return fail(c, MEMD_ERR_CUDA, "applying pending transfers");
@@ -1167,11 +1179,18 @@ memd_status memd_flush(memd_ctx* c) {
 extern "C" {
 
 // single launch or graph of four kernels for this system (decided when the
-// step graphs are built, once the particle count is known)
+// step graphs are built, once the particle count is known).  Left to choose,
+// the single launch runs where it was the faster of the two: FP32 32^3
+// 7.2-7.7 us a step against 16-19 (200 to 4800 charges), 48^3 14-17.6 against
+// 16.5-22.6 (200 to 9000), 56^3 18-24 against 16.5-21.6; FP64 40^3 21-30
+// against 30-37, 48^3 26-36.5 against 30-37, 56^3 37-49 against 38-45; and
+// from 16000 charges (four passes of its particle warps) 26-51 against
+// 25-47.
 static bool want_coop(const memd_ctx* c) {
   if (c->coop_grid <= 0 || c->step_engine == MEMD_STEP_GRAPH) return false;
   if (c->step_engine == MEMD_STEP_SINGLE) return true;
-  return c->mesh.V <= (int64_t(1) << 17) && c->P.n <= (int64_t)16 * c->coop_grid;
+  return c->mesh.V <= (c->prec == MEMD_FP32 ? 125000 : 110000) &&
+         c->P.n <= (int64_t)60 * c->coop_grid;
 }
 
 // Errors raised by kernels of earlier batches, without blocking: the flag is
@@ -1200,10 +1219,10 @@ static memd_status step_prepare(memd_ctx* c, const memd_thermostat* th, StepPara
   }
   if (!c->graph[0] && !c->graph[1]) c->coop = want_coop(c);
   if (c->coop && !c->Tb2) {
-    // the single-launch step's two transfer buffers (3 V words each)
-    c->Tb2 = (long long*)dalloc(c, kLT * 3 * c->mesh.V * sizeof(long long));
-    if (!c->Tb2) return fail(c, MEMD_ERR_OOM, "second transfer buffer");
-    CK(cudaMemsetAsync(c->Tb2, 0, kLT * 3 * c->mesh.V * sizeof(long long), c->stream));
+    // the single-launch step's transfer slots (3 V words each)
+    c->Tb2 = (long long*)dalloc(c, kCoopSlots * 3 * c->mesh.V * sizeof(long long));
+    if (!c->Tb2) return fail(c, MEMD_ERR_OOM, "transfer slots");
+    CK(cudaMemsetAsync(c->Tb2, 0, kCoopSlots * 3 * c->mesh.V * sizeof(long long), c->stream));
   }
   if (!c->coop) {
     const memd_status e = memd_flush(c);
@@ -1231,37 +1250,33 @@ memd_status memd_step(memd_ctx* c, int64_t nsteps, const memd_thermostat* th) {
     if (e != MEMD_OK) return e;
   }
   const bool timed = c->time_kernels != 0;
-  auto record = [&](int par) {
-    return c->coop ? record_step_coop(c, sp, par, timed) : record_step(c, sp, par, timed);
-  };
+  if (c->coop) {
+    // the single launch takes up to kCoopSteps steps at a time (one when each
+    // is timed)
+    for (int64_t s = 0; s < nsteps;) {
+      const int k = timed ? 1 : (int)std::min<int64_t>(nsteps - s, kCoopSteps);
+      harvest_timing(c);
+      const memd_status r = run_steps_coop(c, sp, timed, k);
+      if (r != MEMD_OK) return r;
+      s += k;
+    }
+    return poll_err(c, false);
+  }
   for (int64_t s = 0; s < nsteps; ++s) {
     const int par = c->cur;
     harvest_timing(c);
-    if (!c->use_graphs || (c->coop && !c->coop_graph_ok)) {
-      memd_status r = record(par);
+    if (!c->use_graphs) {
+      const memd_status r = record_step(c, sp, par, timed);
       if (r != MEMD_OK) return r;
     } else {
       if (!c->graph[par]) {
         cudaGraph_t g = nullptr;
         CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-        memd_status r = record(par);
-        cudaError_t e = cudaStreamEndCapture(c->stream, &g);
+        const memd_status r = record_step(c, sp, par, timed);
+        const cudaError_t e = cudaStreamEndCapture(c->stream, &g);
         cudaError_t ie = cudaErrorUnknown;
         if (r == MEMD_OK && e == cudaSuccess) ie = cudaGraphInstantiate(&c->graph[par], g, 0);
         if (g) cudaGraphDestroy(g);
-        if (ie != cudaSuccess && c->coop) {
-          // a cooperative launch that cannot be captured or replayed: launch
-          // it directly from now on
-          cudaGetLastError();
-          c->graph[par] = nullptr;
-          c->coop_graph_ok = false;
-          memd_status r2 = record(par);
-          if (r2 != MEMD_OK) return r2;
-          c->timing_pending = timed;
-          c->cur = par ^ 1;
-          c->pending = true;
-          continue;
-        }
         if (r != MEMD_OK) return r;
         if (e != cudaSuccess) return fail(c, MEMD_ERR_CUDA, "graph capture");
         if (ie != cudaSuccess) return fail(c, MEMD_ERR_CUDA, "graph instantiate");
@@ -1273,7 +1288,6 @@ memd_status memd_step(memd_ctx* c, int64_t nsteps, const memd_thermostat* th) {
     }
     c->timing_pending = timed;
     c->cur = par ^ 1;
-    if (c->coop) c->pending = true;
   }
   return poll_err(c, false);
 }
@@ -1551,24 +1565,42 @@ memd_status memd_step_io(memd_ctx* c, int32_t load, int64_t nsteps, const memd_t
   if (s != MEMD_OK) return s;
   const IoLayout L = io_layout(c->P.n);
   const cudaStream_t st = c->stream;
-  if (load && nsteps == 1 && c->P.n > 0 && c->use_graphs && c->io_graph_ok) {
-    // the usual host loop: one graph launch a call
+  // few charges: the kernels use the host block itself
+  const bool direct = c->P.n <= kIoDirectMax;
+  auto io_in = [&] {
+    if (!direct) cudaMemcpyAsync(c->io_dev, c->io_host, (size_t)L.f, cudaMemcpyHostToDevice, st);
+    launch_io_unpack(c->mesh, c->P, direct ? c->io_host : c->io_dev, &c->ds->err, st);
+  };
+  auto io_out = [&] {
+    launch_io_pack(c->P, direct ? c->io_host : c->io_dev, &c->ds->err, st);
+    if (!direct)
+      cudaMemcpyAsync(c->io_host, c->io_dev, (size_t)L.bytes, cudaMemcpyDeviceToHost, st);
+  };
+  auto finish = [&]() -> memd_status {
+    CK(cudaStreamSynchronize(st));
+    if (*(const unsigned int*)(c->io_host + L.err)) return check_err(c);
+    return MEMD_OK;
+  };
+  if (load && nsteps == 1 && c->P.n > 0) {
+    // the usual host loop: one launch a call
     StepParams sp;
     s = step_prepare(c, th, sp);
     if (s != MEMD_OK) return s;
-    if (!c->coop || c->coop_graph_ok) {
-      const bool timed = c->time_kernels != 0;
-      const int par = c->cur;
+    const bool timed = c->time_kernels != 0;
+    const int par = c->cur;
+    if (c->coop && direct) {
+      harvest_timing(c);
+      s = run_steps_coop(c, sp, timed, 1, c->io_host, 1);
+      return s == MEMD_OK ? finish() : s;
+    }
+    if (!c->coop && c->use_graphs && c->io_graph_ok) {
       harvest_timing(c);
       if (!c->io_graph[par]) {
         cudaGraph_t g = nullptr;
         CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        cudaMemcpyAsync(c->io_dev, c->io_host, (size_t)L.f, cudaMemcpyHostToDevice, st);
-        launch_io_unpack(c->mesh, c->P, c->io_dev, &c->ds->err, st);
-        const memd_status r = c->coop ? record_step_coop(c, sp, par, timed)
-                                      : record_step(c, sp, par, timed);
-        launch_io_pack(c->P, c->io_dev, &c->ds->err, st);
-        cudaMemcpyAsync(c->io_host, c->io_dev, (size_t)L.bytes, cudaMemcpyDeviceToHost, st);
+        io_in();
+        const memd_status r = record_step(c, sp, par, timed);
+        io_out();
         const cudaError_t e = cudaStreamEndCapture(st, &g);
         cudaError_t ie = cudaErrorUnknown;
         if (r == MEMD_OK && e == cudaSuccess) ie = cudaGraphInstantiate(&c->io_graph[par], g, 0);
@@ -1583,27 +1615,20 @@ memd_status memd_step_io(memd_ctx* c, int32_t load, int64_t nsteps, const memd_t
         CK(cudaGraphLaunch(c->io_graph[par], st));
         c->timing_pending = timed;
         c->cur = par ^ 1;
-        if (c->coop) c->pending = true;
-        CK(cudaStreamSynchronize(st));
-        if (*(const unsigned int*)(c->io_host + L.err)) return check_err(c);
-        return MEMD_OK;
+        return finish();
       }
     }
   }
   if (load && c->P.n > 0) {
     // positions, velocities and image counters: the first 60 n bytes
-    CK(cudaMemcpyAsync(c->io_dev, c->io_host, (size_t)L.f, cudaMemcpyHostToDevice, st));
-    launch_io_unpack(c->mesh, c->P, c->io_dev, &c->ds->err, st);
+    io_in();
     CKL();
   }
   s = memd_step(c, nsteps, th);
   if (s != MEMD_OK) return s;
-  launch_io_pack(c->P, c->io_dev, &c->ds->err, st);
+  io_out();
   CKL();
-  CK(cudaMemcpyAsync(c->io_host, c->io_dev, (size_t)L.bytes, cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  if (*(const unsigned int*)(c->io_host + L.err)) return check_err(c);
-  return MEMD_OK;
+  return finish();
 }
 
 memd_status memd_move(memd_ctx* c, const double* pos, const int32_t* img) {
@@ -1856,13 +1881,14 @@ memd_status memd_load_state(memd_ctx* c, const void* buf, int64_t bytes) {
     if (ok && clear_transfers(c, c->Tb, st) != cudaSuccess) ok = false;
   }
   if (ok && c->Tb2 &&
-      cudaMemsetAsync(c->Tb2, 0, kLT * 3 * c->mesh.V * sizeof(long long), st) != cudaSuccess)
+      cudaMemsetAsync(c->Tb2, 0, kCoopSlots * 3 * c->mesh.V * sizeof(long long), st) != cudaSuccess)
     ok = false;
   launch_state_counters(c->ds, h.step, reinterpret_cast<const long long*>(h.Plast), st);
   if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) ok = false;
   dfree(c, pack);
   if (!ok) return fail(c, MEMD_ERR_CUDA, "state copy");
   c->pending = false;
+  c->tslot = 0;
   c->bg = bg;
   c->sig_ready = false;
   c->gen += 1;

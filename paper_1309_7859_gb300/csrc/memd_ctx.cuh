@@ -46,7 +46,8 @@ struct memd_ctx {
   double eps_eff_inv[9] = {0};  // exact inverse of the effective permittivity (Minv symmetrised)
   double* psi = nullptr;        // cell-problem potentials of the scalar solver (3V), or null
   double* pin = nullptr;        // memd_set_particles staging (3n doubles + 3n ints)
-  long long* Tb2 = nullptr;     // second transfer buffer of the single-launch step
+  long long* Tb2 = nullptr;     // transfer slots of the single-launch step
+  int tslot = 0;                // its slot of the last step
   long long bg = 0;             // neutralising background a vertex (units of e 2^-48)
   bool pending = false;         // transfers of the last single-launch step not yet applied
   // particles
@@ -75,7 +76,6 @@ struct memd_ctx {
   int apply_mode = 0;    // MEMD_APPLY_*
   int coop_grid = 0;     // CTAs of the single-launch step (0: unsupported)
   bool coop = false;     // the steps run as one cooperative launch
-  bool coop_graph_ok = true;  // its launch can be captured in a graph
   int graph_thermo = -1;
   double graph_gamma = 0, graph_kT = 0;
   cudaStream_t side = nullptr;

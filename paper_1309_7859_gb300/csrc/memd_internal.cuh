@@ -82,6 +82,7 @@ struct DevState {
                                     // since init (grows by the grid size a barrier)
   long long lsum[3];           // scratch: sum of the ledger per component
   double scal[16];             // scratch scalars for the relaxation
+  unsigned long long Pc[3][3]; // the single-launch step's dipole sums, one slot a step in turn
 };
 
 __host__ __device__ inline int64_t vindex(const Mesh& m, int i, int j, int k) {
@@ -272,13 +273,29 @@ constexpr unsigned long long kBarrierWaitNs = 200000000ull;  // 0.2 s
 // single-launch step (memd_particles.cu): the whole time step in one
 // cooperative launch, for systems small enough that launch gaps dominate
 constexpr int kCoopFieldWarps = 11;                  // 34 x 10 site tile of 8 rows
-constexpr int kCoopThreads = 32 * (kCoopFieldWarps + 1);
+constexpr int kCoopParticleWarps = 4;                // one a scheduler: 8 charges each a pass
+constexpr int kCoopThreads = 32 * (kCoopFieldWarps + kCoopParticleWarps);
 int coop_grid(int prec, int device);                 // CTAs of one cooperative launch, 0 if none
-int coop_zchunk(const Mesh& m, int grid);
+// nsteps steps from buffer parity par and transfer slot `slot` (which holds
+// the transfers not yet applied).  io (page-locked host memory of io_layout,
+// or null): the first step takes positions, image counters and velocities
+// from it when io_load is set, the last one writes the state, the forces and
+// the error word into it
+constexpr int kCoopSlots = 3;
+struct CoopBufs {
+  void* D[2];
+  void* B[2];
+  long long* T[kCoopSlots];
+};
+// the field tiles: sites a row, rows and planes a tile
+struct CoopShape {
+  int width, rows, planes;
+};
+constexpr int kCoopSteps = 32;  // most steps a launch
 cudaError_t launch_step_coop(const Mesh& m, int prec, const StepParams& sp, Particles p,
-                             const void* Din, const void* Bin, const void* ie, void* Dout,
-                             void* Bout, const double* ie64, long long* Tprev, long long* Tcur,
-                             long long* Lg, DevState* ds, int grid, int zchunk, cudaStream_t st);
+                             const CoopBufs& buf, const void* ie, const double* ie64,
+                             long long* Lg, DevState* ds, int grid, int par, int slot,
+                             int nsteps, void* io, int io_load, cudaStream_t st);
 // a state's host copies (memd_setup.cu): the ledger's component-major words
 // (3 V) and the particle arrays in a saved state's order (120 bytes a charge)
 void launch_ledger_pack(const Mesh& m, const long long* Lg, long long* out, cudaStream_t st);
@@ -310,6 +327,11 @@ __host__ __device__ inline IoLayout io_layout(int64_t n) {
 // what a pack writes: everything, the moved part (positions, image
 // counters) or the rest (velocities, forces, error words)
 enum : int { kIoAll = 0, kIoMoved = 1, kIoRest = 2 };
+// Up to this many charges the kernels read and write the page-locked host
+// block in place, beyond it the copy engine moves it to and from a device
+// block: a host-loop step of 2512 charges takes 38 us in place and 50 by
+// copies, of 8000 57 and 63, of 16000 84 and 81, of 32768 149 and 131.
+constexpr int64_t kIoDirectMax = 8192;
 void launch_io_unpack(const Mesh& m, Particles p, const void* io, unsigned int* err,
                       cudaStream_t st);
 void launch_io_pack(Particles p, void* io, const unsigned int* err, cudaStream_t st);

@@ -1403,18 +1403,28 @@ __global__ void __launch_bounds__(kBatchStepThreads, 2)
 }
 
 // ---------------------------------------------------- single-launch step
-// The whole time step of one system in one cooperative launch of G CTAs,
-// with one grid barrier.  The transfers of a step are applied lazily: they
-// stay in the transfer buffer Tcur, the gather reads D + Tcur scale (rounded
-// as their application rounds), and the next step's field tiles read their
-// D the same way from that buffer (then Tprev) before updating it; after
-// that step's barrier the field warps move Tprev into the ledger and clear
-// it.  Phase 1: warps 0-10 of every CTA run field tiles (B' then D',
-// one-thread-per-site tiles of 8 rows) while warp 11 runs the kick, drift
-// and deposition into Tcur; grid barrier; phase 2: warp 11 gathers the
-// forces (Langevin, half kick) while the field warps commit Tprev; the last
-// CTA closes the step.  The values are those of the four launches of the
-// graph step, bit for bit.
+// Time steps of one system in one cooperative launch of G CTAs, with one grid
+// barrier a step.  The transfers of a step are applied lazily: they stay in
+// the step's transfer slot, the gather reads D + T scale (rounded as their
+// application rounds), and the next step's field tiles read their D the same
+// way before updating it.  Warps 0-10 of every CTA run field tiles (B' then
+// D', one-thread-per-site tiles), warps 11-14 the particles.  Between the
+// barriers of steps s and s + 1 (the barrier of a step follows its field
+// tiles and its deposition):
+//   field warps: the field tiles of step s + 1 (they need D, B and the
+//   transfers of step s only), then the transfers of step s - 1 into the
+//   ledger and their slot cleared
+//   particle warps: the gather of step s, then kick, drift and deposition of
+//   step s + 1
+// Every word is written at least one barrier after its last reader: D and B
+// alternate between two buffers, transfers and dipole sums go round three
+// slots (written in one interval, read in the next, cleared in the third).
+// The values are those of the four launches of the graph step, bit for bit.
+//
+// What bounds it: latency.  With a barrier between deposition and gather and
+// a launch a step (or a second barrier), both chains of a step were in turn
+// and the field tiles waited on every plane's pending transfers in turn:
+// 32^3 with 1000 charges 12.9 us a step, 8^3 FP64 18.8; now 7.3 and 9.5.
 
 // Grid-wide barrier of a cooperative launch over a monotonic 64-bit count
 // of CTA arrivals: each CTA adds one with release and acquire semantics and
@@ -1428,9 +1438,21 @@ __global__ void __launch_bounds__(kBatchStepThreads, 2)
 // by the global timer (0.2 s); a wait that runs out sets kErrTimeout and
 // goes on, the step is then void and the host resets the count when it
 // reports the error.
-__device__ inline void grid_barrier(DevState* ds, unsigned nctas, unsigned long long wait_ns) {
-  __syncthreads();
+//
+// In two halves, so that a warp with work of its own to do need not wait for
+// the others: barrier_arrive (field warps wait there for the CTA's arrival,
+// the particle warp passes), then barrier_wait.
+__device__ __forceinline__ void barrier_arrive(bool pass) {
+  if (pass)
+    asm volatile("bar.arrive 3, %0;" ::"n"(kCoopThreads) : "memory");
+  else
+    asm volatile("bar.sync 3, %0;" ::"n"(kCoopThreads) : "memory");
+}
+__device__ __forceinline__ bool barrier_wait(DevState* ds, unsigned nctas,
+                                             unsigned long long wait_ns) {
+  __shared__ int s_late;
   if (threadIdx.x == 0) {
+    s_late = 0;  // every thread has read the last barrier's (it has arrived)
     unsigned long long a;
     asm volatile("atom.acq_rel.gpu.global.add.u64 %0, [%1], 1;"
                  : "=l"(a)
@@ -1450,6 +1472,7 @@ __device__ inline void grid_barrier(DevState* ds, unsigned nctas, unsigned long 
           asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
           if (t - t0 > wait_ns) {
             atomicOr(&ds->err, kErrTimeout);
+            s_late = 1;
             break;
           }
         }
@@ -1458,6 +1481,7 @@ __device__ inline void grid_barrier(DevState* ds, unsigned nctas, unsigned long 
     }
   }
   __syncthreads();
+  return s_late == 0;
 }
 
 // barrier of the field warps of a CTA (named barrier 1)
@@ -1467,13 +1491,13 @@ struct FieldWarpsSync {
   }
 };
 
-// ledger += Tprev, Tprev = 0 on the sites a field thread updates
+// ledger += Tp, Tp = 0 on the sites a field thread updates
 __device__ __forceinline__ void commit_tile(const Mesh& m, int txi, int tyi, int tz, int zchunk,
-                                            int tx, int ty, bool live, long long* __restrict__ Tp,
-                                            long long* __restrict__ Lg) {
+                                            int rows, int wx, int tx, int ty, bool live,
+                                            long long* Tp, long long* __restrict__ Lg) {
   const int nx = m.n[0], ny = m.n[1];
-  const int x = txi * 32 - 1 + tx, y = tyi * 8 - 1 + ty;
-  if (!live || tx < 1 || tx > 32 || ty < 1 || ty > 8 || x >= nx || y >= ny) return;
+  const int x = txi * wx - 1 + tx, y = tyi * rows - 1 + ty;
+  if (!live || tx < 1 || tx > wx || ty < 1 || ty > rows || x >= nx || y >= ny) return;
   const int z0 = tz * zchunk, z1 = min(z0 + zchunk, m.n[2]);
   const int64_t P = (int64_t)nx * ny;
   for (int k = z0; k < z1; ++k)
@@ -1481,7 +1505,7 @@ __device__ __forceinline__ void commit_tile(const Mesh& m, int txi, int tyi, int
     for (int c = 0; c < 3; ++c) {
       const int64_t v = (int64_t)k * P + (int64_t)y * nx + x;
       const int64_t w = tw_index(c, v, m.V);  // the step's own buffer: component major
-      const long long t = Tp[w];
+      const long long t = __ldcg(Tp + w);
       if (t != 0) {
         Lg[kLT * tl_pair(c, v)] += t;
         Tp[w] = 0;
@@ -1489,83 +1513,367 @@ __device__ __forceinline__ void commit_tile(const Mesh& m, int txi, int tyi, int
     }
 }
 
+// io: the host's block, read by the first step's particle lanes and written
+// by the last one's (each lane its own component), so that a host loop's
+// round trip is this one launch.
+__device__ __forceinline__ void io_take(const Mesh& m, const Particles& P,
+                                        const unsigned char* io, int64_t p, int d,
+                                        unsigned int* err) {
+  const IoLayout L = io_layout(P.n);
+  const int64_t c = 3 * p + d;
+  double x = reinterpret_cast<const double*>(io + L.pos)[c];
+  int k = reinterpret_cast<const int*>(io + L.img)[c];
+  const double v = reinterpret_cast<const double*>(io + L.vel)[c];
+  if (!(fabs(x) <= 4.0 * m.L[d])) {
+    atomicOr(err, kErrNonFinite);
+    x = 0.0;
+  }
+  fold(m.L[d], x, k);
+  P.x[c] = x;
+  P.img[c] = k;
+  P.v[c] = v;
+}
+__device__ __forceinline__ void io_give(const Particles& P, unsigned char* io, int64_t p, int d) {
+  const IoLayout L = io_layout(P.n);
+  const int64_t c = 3 * p + d;
+  reinterpret_cast<double*>(io + L.pos)[c] = P.x[c];
+  reinterpret_cast<int*>(io + L.img)[c] = P.img[c];
+  reinterpret_cast<double*>(io + L.vel)[c] = P.v[c];
+  reinterpret_cast<double*>(io + L.f)[c] = P.F[c];
+}
+
+// A quad lane's charge held in registers from step to step (one pass over the
+// charges a step, at most 8 a particle warp): the move and the gather of
+// deposit_body, quad_move and gather_body with the same expressions.  What
+// the gather can form before the step's barrier completes (the cell's 1/eps,
+// weights, self energy, noise) is formed while the barrier is under way.
+template <typename T>
+struct HeldCharge {
+  double x, v, Ft, F, h, sig, gm;
+  int img, q, c, f;     // own axis: image counter, cell, sub-cell step (c, f of the present x)
+  int c0;               // cell before the last move
+  int C[3], W[3];       // the quad's cells and sub-cell steps after the move
+  int64_t link[3];      // the lane's corner: field index of its three links
+  T wie[3];             // their 1/eps and weight
+  T w[3];
+  T self;               // self-energy force of the own component
+  double fn, fr;        // Langevin noise and friction
+
+  __device__ __forceinline__ void take(const Mesh& m, const Particles& P, int64_t p, int d,
+                                       bool active, int thermo) {
+    x = v = Ft = F = h = sig = gm = 0.0;
+    img = q = c = f = c0 = 0;
+    if (!active) return;
+    q = P.q[p];
+    if (d < 3) {
+      x = P.x[3 * p + d];
+      v = P.v[3 * p + d];
+      Ft = P.Ft[3 * p + d];
+      img = P.img[3 * p + d];
+      h = P.h[p];
+      if (thermo) {
+        sig = P.sig[p];
+        gm = P.gm[p];
+      }
+      quantize(m, d, x, c, f);
+    }
+  }
+  // half kick, drift, charge transfer; the lane's dipole term
+  __device__ __forceinline__ long long move(const Mesh& m, const StepParams& sp, int d,
+                                            bool active, unsigned long long* Tb, DevState* ds,
+                                            int64_t V) {
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31, base = lane & ~3;
+    const bool own = active && d < 3;
+    double xn = x;
+    int kn = img, c1 = 0, f1 = 0, dc = 0;
+    bool ok = true;
+    if (own) {
+      v = __dadd_rn(v, __dmul_rn(h, Ft));
+      const double step = __dmul_rn(sp.dt, v);
+      if (fabs(step) <= 2.0 * m.a) {
+        xn = __dadd_rn(x, step);
+        fold(m.L[d], xn, kn);
+      } else {
+        ok = false;
+      }
+      quantize(m, d, xn, c1, f1);
+      dc = c1 + (kn - img) * m.n[d] - c;
+      if (dc < -1 || dc > 1) ok = false;
+    }
+    const bool all_ok = ((__ballot_sync(full, ok) >> base) & 0xfu) == 0xfu;
+    int C0[3], F0[3], C1[3], F1[3];
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      C0[e] = __shfl_sync(full, c, base + e);
+      F0[e] = __shfl_sync(full, f, base + e);
+      C1[e] = __shfl_sync(full, c1, base + e);
+      F1[e] = __shfl_sync(full, f1, base + e);
+      C[e] = all_ok ? C1[e] : C0[e];
+      W[e] = all_ok ? F1[e] : F0[e];
+    }
+    long long U = 0;
+    if (own) {
+      c0 = c;
+      if (all_ok) {
+        int cc[3], cf[3];
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+          cc[e] = (e < d) ? C1[e] : C0[e];
+          cf[e] = (e < d) ? F1[e] : F0[e];
+        }
+        deposit_axis(m, d, q, c, f, f1, dc, cc, cf, Tb, V);
+        x = xn;
+        img = kn;
+        c = c1;
+        f = f1;
+      } else if (d == 0) {
+        atomicOr(&ds->err, kErrCellJump);
+      }
+      U = (((long long)img * m.n[d] + c) * kS + f) * (long long)q;
+    }
+    return U;
+  }
+  // the gather's part that needs no field
+  __device__ __forceinline__ void before(const Mesh& m, const StepParams& sp, int thermo,
+                                         const T* __restrict__ ie,
+                                         const double* __restrict__ ie64, int64_t p, int d,
+                                         bool active, long long step) {
+    const unsigned full = 0xffffffffu;
+    const int a1 = d & 1, a2 = d >> 1;
+    T iw[3] = {T(0), T(0), T(0)}, itot = T(0);
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      link[e] = 0;
+      wie[e] = w[e] = T(0);
+    }
+    if (active) {
+      T iv[3];
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        const int e1 = (e + 1) % 3, e2 = (e + 2) % 3;
+        int at[3] = {C[0], C[1], C[2]};
+        at[e1] += a1;
+        at[e2] += a2;
+        link[e] = (int64_t)e * m.V + link_vertex(m, at[0], at[1], at[2]);
+        wie[e] = ie[link[e]];
+        iv[e] = sizeof(T) == 8 && sp.self_mode != 0 ? (T)ie64[link[e]] : wie[e];
+      }
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        const int e1 = (e + 1) % 3, e2 = (e + 2) % 3;
+        w[e] = ((T)wgt(W[e1], a1) / (T)kS) * ((T)wgt(W[e2], a2) / (T)kS);
+        if (sp.self_mode != 0) itot += iv[e];
+        if (sp.self_mode == 2) iw[e] = iv[e] * w[e];
+      }
+    }
+    if (sp.self_mode == 2) {
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        iw[e] = iw[e] + __shfl_xor_sync(full, iw[e], 1);
+        iw[e] = iw[e] + __shfl_xor_sync(full, iw[e], 2);
+      }
+    }
+    if (sp.self_mode != 0) {
+      itot = itot + __shfl_xor_sync(full, itot, 1);
+      itot = itot + __shfl_xor_sync(full, itot, 2);
+    }
+    self = T(0);
+    fn = fr = 0.0;
+    if (active && d < 3) {
+      if (sp.self_mode != 0) {
+        const T qr = (T)q;
+        const T ie_cell = itot * (T(1) / T(12));
+        const T iwd = d == 0 ? iw[0] : (d == 1 ? iw[1] : iw[2]);
+        const T ie_d = (sp.self_mode == 2) ? iwd : ie_cell;
+        const SelfC<T> sc = self_coeffs<T>(W);
+        self = (qr * qr * sp_self_pre<T>(sp)) * ie_d * self_sum<T>(sp, sc, d);
+      }
+      if (thermo) {
+        unsigned ctr[4] = {(unsigned)p, (unsigned)((unsigned long long)p >> 32), (unsigned)step,
+                           (unsigned)((unsigned long long)step >> 32)};
+        philox4x32_10(ctr, (unsigned)sp.seed, (unsigned)(sp.seed >> 32));
+        fr = gm * v;  // (-gamma m) v
+        fn = sig * unit_noise(d == 0 ? ctr[0] : (d == 1 ? ctr[1] : ctr[2]));
+      }
+    }
+  }
+  // the rest: field, dipole, second half kick
+  __device__ __forceinline__ void after(const Mesh& m, const StepParams& sp, int thermo,
+                                        const T* D, const long long* Tp, bool exact32,
+                                        const unsigned long long* Pc, int d, bool active) {
+    const unsigned full = 0xffffffffu;
+    T E[3] = {T(0), T(0), T(0)};
+    long long Pl[3] = {0, 0, 0};
+    if (active) {
+      T Dv[3];
+      long long t[3];
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        Dv[e] = __ldcg(D + link[e]);
+        t[e] = __ldcg(Tp + link[e]);  // the slot is component major: the field's index
+      }
+      if (sp.dipole_corr && d < 3)
+#pragma unroll
+        for (int e = 0; e < 3; ++e) Pl[e] = (long long)__ldcg(Pc + e);
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        if (t[e] != 0) Dv[e] = Dv[e] + pending_inc<T>(t[e], sp.scale, exact32);
+        E[e] = Dv[e] * wie[e] * w[e];
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      E[e] = E[e] + __shfl_xor_sync(full, E[e], 1);
+      E[e] = E[e] + __shfl_xor_sync(full, E[e], 2);
+    }
+    if (active && d < 3) {
+      const T qr = (T)q;
+      T Fr = qr * (d == 0 ? E[0] : (d == 1 ? E[1] : E[2]));
+      if (sp.self_mode != 0) Fr = Fr + self;
+      if (sp.dipole_corr) {
+        const T MP = sp_Mdip<T>(sp, 3 * d) * (T)Pl[0] + sp_Mdip<T>(sp, 3 * d + 1) * (T)Pl[1] +
+                     sp_Mdip<T>(sp, 3 * d + 2) * (T)Pl[2];
+        Fr = Fr + qr * MP;
+      }
+      F = (double)Fr;
+      Ft = F;
+      if (thermo) Ft = F + (fr + fn);
+      v = __dadd_rn(v, __dmul_rn(h, Ft));
+    }
+  }
+  // the arrays as the kernels of the other engines leave them
+  __device__ __forceinline__ void give(const Particles& P, int64_t p, int d) const {
+    const int64_t k = 3 * p + d;
+    P.x[k] = x;
+    P.v[k] = v;
+    P.img[k] = img;
+    P.F[k] = F;
+    P.Ft[k] = Ft;
+    int* mv = P.mv + kMoveInts * p;
+    mv[d] = c0;
+    mv[3 + d] = c;
+    mv[6 + d] = f;
+  }
+};
+
 template <typename T>
 __global__ void __launch_bounds__(kCoopThreads)
     k_step_coop(const __grid_constant__ Mesh m, const __grid_constant__ StepParams sp, Particles P,
-                const T* __restrict__ Din, const T* __restrict__ Bin, const T* __restrict__ ie,
-                T* __restrict__ Dout, T* __restrict__ Bout, const double* __restrict__ ie64,
-                long long* __restrict__ Tprev, unsigned long long* __restrict__ Tcur,
-                long long* __restrict__ Lg, DevState* ds, int zchunk) {
+                const __grid_constant__ CoopBufs buf, const T* __restrict__ ie,
+                const double* __restrict__ ie64, long long* __restrict__ Lg, DevState* ds,
+                CoopShape shape, int par, int slot, int nsteps, unsigned char* io, int io_load) {
   const bool exact32 = m.a_pow2 != 0;  // power-of-two scale (FP32 fields use it)
   const int tid = threadIdx.x;
-  const bool pwarp = (tid >> 5) == kCoopFieldWarps;
+  const int pw = (tid >> 5) - kCoopFieldWarps;  // particle warp, < 0 for field warps
+  const bool pwarp = pw >= 0;
   const unsigned G = gridDim.x;
   const int lane = tid & 31;
   const int64_t nq = 4 * P.n;  // quad lanes of all particles
-  const int64_t stride = (int64_t)G * 32;
-  const int tiles_x = (m.n[0] + 31) / 32, tiles_y = (m.n[1] + 7) / 8;
+  // few charges go to the first particle warp of every CTA
+  const int64_t first = ((int64_t)max(pw, 0) * G + blockIdx.x) * 32;
+  const int64_t stride = (int64_t)G * 32 * kCoopParticleWarps;
+  const int rows = shape.rows, zchunk = shape.planes, wx = shape.width;
+  const int tiles_x = (m.n[0] + wx - 1) / wx, tiles_y = (m.n[1] + rows - 1) / rows;
   const int tiles_z = (m.n[2] + zchunk - 1) / zchunk;
   const int ntiles = tiles_x * tiles_y * tiles_z;
-  const bool live = tid < 34 * 10;
-  const int tx = live ? tid % 34 : 0, ty = live ? tid / 34 : 0;
-  if (!pwarp) {
+  const bool live = tid < (wx + 2) * (rows + 2);
+  const int ty = live ? tid / (wx + 2) : 0, tx = live ? tid - ty * (wx + 2) : 0;
+  const long long step0 = __ldcg(&ds->step);  // before the first barrier: unchanged until the last
+
+  // the field tiles of the step from parity q, its pending transfers in Tp
+  auto field = [&](int q, const long long* Tp) {
     for (int t = blockIdx.x; t < ntiles; t += (int)G) {
       const int tz = t / (tiles_x * tiles_y), r = t - tz * (tiles_x * tiles_y);
       const int tyi = r / tiles_x, txi = r - tyi * tiles_x;
-      site_tile<T, 8, 1>(m, Din, Bin, ie, Dout, Bout, (T)sp.coefB, (T)sp.coefD, txi, tyi, tz,
-                         zchunk, tx, ty, live, FieldWarpsSync{}, Tprev, sp.scale, exact32);
+      site_tile<T, 8, 1, FieldWarpsSync, 32, true>(
+          m, (const T*)buf.D[q], (const T*)buf.B[q], ie, (T*)buf.D[q ^ 1], (T*)buf.B[q ^ 1],
+          (T)sp.coefB, (T)sp.coefD, txi, tyi, tz, zchunk, tx, ty, live, FieldWarpsSync{}, Tp,
+          sp.scale, exact32, wx, rows);
     }
-  } else {
-    for (int64_t b = (int64_t)blockIdx.x * 32; b < nq; b += stride)
-      quad_dipole_add(ds->Pacc, deposit_body(m, sp, P, Tcur, ds, b + lane, (const char*)ie,
-                                             (int)sizeof(T), m.V));
-  }
-  grid_barrier(ds, G, sp.wait_ns);
+  };
+  // kick, drift and deposition into transfer slot w
+  auto deposit = [&](int w, bool take) {
+    for (int64_t b = first; b < nq; b += stride) {
+      if (take && b + lane < nq && (lane & 3) < 3)
+        io_take(m, P, io, (b + lane) >> 2, lane & 3, &ds->err);
+      quad_dipole_add(ds->Pc[w], deposit_body(m, sp, P, (unsigned long long*)buf.T[w], ds,
+                                              b + lane, (const char*)ie, (int)sizeof(T), m.V));
+    }
+  };
+  auto next = [](int w) { return w == 2 ? 0 : w + 1; };
+
+  int q = par, w = next(slot);  // the step's parity and transfer slot
+  // every charge in one pass: held in registers by the particle lanes
+  const bool held = nq <= stride;
+  HeldCharge<T> ch;
+  const int64_t hp = (first + lane) >> 2;
+  const int hd = lane & 3;
+  const bool mine = hp < P.n;
   if (pwarp) {
-    // the dipole sum of this move and the step counter, read once; the
-    // particle warp then signals field warp 0 (named barrier 2), which takes
-    // the CTA's ticket while the gather runs, so the last CTA closes the step
-    // (P of this state reported, the sum cleared, the counter advanced) off
-    // the gather's path.  Every CTA's reads are complete before its signal:
-    // the signal consumes them.
-    long long pre[4];
-    pre[0] = (long long)__ldcg(&ds->Pacc[0]);
-    pre[1] = (long long)__ldcg(&ds->Pacc[1]);
-    pre[2] = (long long)__ldcg(&ds->Pacc[2]);
-    pre[3] = __ldcg(&ds->step);
-    const long long used = ((pre[0] ^ pre[1]) ^ pre[2]) ^ pre[3];
-    asm volatile("bar.arrive 2, 64;" ::"l"(used) : "memory");
-    for (int64_t b = (int64_t)blockIdx.x * 32; b < nq; b += stride)
-      gather_body<T>(m, sp, sp.thermo, sp.gamma, sp.kT, P, Dout, ie, ie64, ds, 1, 0, G, b + lane,
-                     (const long long*)Tcur, exact32, pre, true);
-  } else {
-    for (int t = blockIdx.x; t < ntiles; t += (int)G) {
-      const int tz = t / (tiles_x * tiles_y), r = t - tz * (tiles_x * tiles_y);
-      const int tyi = r / tiles_x, txi = r - tyi * tiles_x;
-      commit_tile(m, txi, tyi, tz, zchunk, tx, ty, live, Tprev, Lg);
+    if (held && first < nq) {
+      if (io_load && mine && hd < 3) io_take(m, P, io, hp, hd, &ds->err);
+      ch.take(m, P, hp, hd, mine, sp.thermo);
+      quad_dipole_add(ds->Pc[w],
+                      ch.move(m, sp, hd, mine, (unsigned long long*)buf.T[w], ds, m.V));
+    } else if (!held) {
+      deposit(w, io_load != 0);
     }
-    if (tid < 32) {
-      asm volatile("bar.sync 2, 64;" ::: "memory");
-      if (tid == 0) {
-        unsigned t;
-        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;"
-                     : "=r"(t)
-                     : "l"(&ds->ticket)
-                     : "memory");
-        if (t == G - 1) {
-          const unsigned long long p0 = __ldcg(&ds->Pacc[0]), p1 = __ldcg(&ds->Pacc[1]),
-                                   p2 = __ldcg(&ds->Pacc[2]);
-          const long long st = __ldcg(&ds->step);
-          ds->Plast[0] = (long long)p0;
-          ds->Plast[1] = (long long)p1;
-          ds->Plast[2] = (long long)p2;
-          ds->Pacc[0] = 0ull;
-          ds->Pacc[1] = 0ull;
-          ds->Pacc[2] = 0ull;
-          ds->step = st + 1;
-          ds->ticket = 0u;
-        }
+  } else {
+    field(q, buf.T[slot]);
+  }
+  for (int s = 1;; ++s) {
+    const bool last = s == nsteps;
+    barrier_arrive(pwarp);
+    if (pwarp && held && first < nq) ch.before(m, sp, sp.thermo, ie, ie64, hp, hd, mine, step0 + (s - 1));
+    const bool ok = barrier_wait(ds, G, sp.wait_ns);
+    const int w1 = next(w), w0 = next(w1);  // the next step's slot, the step before's
+    if (pwarp && held && first < nq) {
+      ch.after(m, sp, sp.thermo, (const T*)buf.D[q ^ 1], buf.T[w], exact32, ds->Pc[w], hd, mine);
+      if (!last && ok) {
+        quad_dipole_add(ds->Pc[w1],
+                        ch.move(m, sp, hd, mine, (unsigned long long*)buf.T[w1], ds, m.V));
+      } else if (mine && hd < 3) {
+        ch.give(P, hp, hd);
+        if (io) io_give(P, io, hp, hd);
       }
+    } else if (pwarp && !held) {
+      const long long pre[4] = {(long long)__ldcg(&ds->Pc[w][0]), (long long)__ldcg(&ds->Pc[w][1]),
+                                (long long)__ldcg(&ds->Pc[w][2]), step0 + (s - 1)};
+      for (int64_t b = first; b < nq; b += stride) {
+        gather_body<T>(m, sp, sp.thermo, sp.gamma, sp.kT, P, (const T*)buf.D[q ^ 1], ie, ie64, ds,
+                       1, 0, G, b + lane, buf.T[w], exact32, pre, true);
+        if (last && io && b + lane < nq && (lane & 3) < 3)
+          io_give(P, io, (b + lane) >> 2, lane & 3);
+      }
+      if (!last && ok) deposit(w1, false);
+    } else if (!pwarp) {
+      if (!last && ok) field(q ^ 1, buf.T[w]);
+      for (int t = blockIdx.x; t < ntiles; t += (int)G) {
+        const int tz = t / (tiles_x * tiles_y), r = t - tz * (tiles_x * tiles_y);
+        const int tyi = r / tiles_x, txi = r - tyi * tiles_x;
+        commit_tile(m, txi, tyi, tz, zchunk, rows, wx, tx, ty, live, buf.T[w0], Lg);
+      }
+      if (blockIdx.x == 0 && tid < 3) {
+        ds->Pc[w0][tid] = 0ull;
+        if (last) ds->Plast[tid] = (long long)__ldcg(&ds->Pc[w][tid]);
+        if (last && tid == 0) ds->step = step0 + nsteps;
+      }
+    }
+    if (last || !ok) break;
+    q ^= 1;
+    w = w1;
+  }
+  if (io && tid == 0) {
+    // the last CTA through its barriers reports their errors
+    unsigned t;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;"
+                 : "=r"(t)
+                 : "l"(&ds->ticket)
+                 : "memory");
+    if (t == G - 1) {
+      ds->ticket = 0u;
+      *reinterpret_cast<unsigned int*>(io + io_layout(P.n).err) = __ldcg(&ds->err);
     }
   }
 }
@@ -1872,17 +2180,30 @@ int coop_grid(int prec, int device) {
   return sms;  // one CTA per SM
 }
 
-int coop_zchunk(const Mesh& m, int grid) {
-  const int tiles_xy = ((m.n[0] + 31) / 32) * ((m.n[1] + 7) / 8);
+// Field tiles of the single launch.  Small meshes take one plane and as few
+// rows a tile as still give at most one tile a CTA: the tile's chain of
+// loads, FP64 (or FP32) updates and barriers is what a step waits for, and
+// GB300's FP64 pipe serves few warps at a time.  Larger ones take 8 rows and
+// as many planes as that needs.
+static CoopShape coop_shape(const Mesh& m, int grid) {
+  const int tx = (m.n[0] + 31) / 32;
+  const int width = (m.n[0] + tx - 1) / tx;  // equal tiles: 45 sites as 23 and 22
+  for (int rows = 1; rows <= 8; rows *= 2)
+    if ((int64_t)tx * ((m.n[1] + rows - 1) / rows) * m.n[2] <= grid)
+      return CoopShape{width, rows, 1};
+  const int ty = (m.n[1] + 7) / 8;
+  const int rows = (m.n[1] + ty - 1) / ty;
+  const int64_t xy = (int64_t)tx * ty;
   int zc = 1;
-  while (zc < m.n[2] && (int64_t)tiles_xy * ((m.n[2] + zc - 1) / zc) > grid) zc *= 2;
-  return zc < m.n[2] ? zc : m.n[2];
+  while (zc < m.n[2] && xy * ((m.n[2] + zc - 1) / zc) > grid) ++zc;
+  return CoopShape{width, rows, zc};
 }
 
 cudaError_t launch_step_coop(const Mesh& m, int prec, const StepParams& sp, Particles p,
-                             const void* Din, const void* Bin, const void* ie, void* Dout,
-                             void* Bout, const double* ie64, long long* Tprev, long long* Tcur,
-                             long long* Lg, DevState* ds, int grid, int zchunk, cudaStream_t st) {
+                             const CoopBufs& buf, const void* ie, const double* ie64,
+                             long long* Lg, DevState* ds, int grid, int par, int slot,
+                             int nsteps, void* io, int io_load, cudaStream_t st) {
+  const CoopShape shape = coop_shape(m, grid);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)grid, 1, 1);
   cfg.blockDim = dim3(kCoopThreads, 1, 1);
@@ -1893,14 +2214,12 @@ cudaError_t launch_step_coop(const Mesh& m, int prec, const StepParams& sp, Part
   at[0].val.cooperative = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  unsigned long long* tc = (unsigned long long*)Tcur;
+  unsigned char* iob = (unsigned char*)io;
   if (prec == 1)
-    return cudaLaunchKernelEx(&cfg, k_step_coop<float>, m, sp, p, (const float*)Din,
-                              (const float*)Bin, (const float*)ie, (float*)Dout, (float*)Bout, ie64,
-                              Tprev, tc, Lg, ds, zchunk);
-  return cudaLaunchKernelEx(&cfg, k_step_coop<double>, m, sp, p, (const double*)Din,
-                            (const double*)Bin, (const double*)ie, (double*)Dout, (double*)Bout,
-                            ie64, Tprev, tc, Lg, ds, zchunk);
+    return cudaLaunchKernelEx(&cfg, k_step_coop<float>, m, sp, p, buf, (const float*)ie, ie64, Lg,
+                              ds, shape, par, slot, nsteps, iob, io_load);
+  return cudaLaunchKernelEx(&cfg, k_step_coop<double>, m, sp, p, buf, (const double*)ie, ie64, Lg,
+                            ds, shape, par, slot, nsteps, iob, io_load);
 }
 
 void launch_gather(const Mesh& m, int prec, const StepParams& sp, Particles p, const void* D,

@@ -427,7 +427,10 @@ __global__ void k_state_counters(DevState* ds, long long step, long long P0, lon
   ds->Plast[0] = P0;
   ds->Plast[1] = P1;
   ds->Plast[2] = P2;
-  for (int d = 0; d < 3; ++d) ds->Pacc[d] = 0ull;
+  for (int d = 0; d < 3; ++d) {
+    ds->Pacc[d] = 0ull;
+    for (int s = 0; s < 3; ++s) ds->Pc[s][d] = 0ull;
+  }
   ds->ticket = 0u;
 }
 

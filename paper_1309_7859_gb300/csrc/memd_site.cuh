@@ -49,14 +49,22 @@ __device__ __forceinline__ float fma_t<float>(float a, float b, float c) { retur
 template <>
 __device__ __forceinline__ double fma_t<double>(double a, double b, double c) { return __fma_rn(a, b, c); }
 
-template <typename T, int TY, int PF, class Sync, int TX = 32>
+// wx, wy: sites of the tile in use (a narrow mesh, or lower tiles so that a
+// small one spreads over more SMs): the threads form wx + 2 columns and wy + 2
+// rows.
+//
+// COH: the field and transfer words may have been written earlier in the same
+// launch by other CTAs: read at L2 (a thread reads each word once, so L1
+// would hold nothing for it anyway).
+template <typename T, int TY, int PF, class Sync, int TX = 32, bool COH = false>
 __device__ __forceinline__ void site_tile(const Mesh& m, const T* __restrict__ Din,
                                           const T* __restrict__ Bin, const T* __restrict__ ie,
                                           T* __restrict__ Dout, T* __restrict__ Bout, T cB, T cD,
                                           int tile_x, int tile_y, int tile_z, int zchunk, int tx,
                                           int ty, bool live, Sync sync,
                                           const long long* __restrict__ Tp = nullptr,
-                                          double tscale = 0.0, bool exact32 = false) {
+                                          double tscale = 0.0, bool exact32 = false,
+                                          int wx = TX, int wy = TY) {
   static_assert(PF >= 1 && PF <= 2, "prefetch depth");
   static_assert(TX == 16 || TX == 32, "tile width");
   constexpr int EX = TX + 2, EY = TY + 2;
@@ -65,12 +73,12 @@ __device__ __forceinline__ void site_tile(const Mesh& m, const T* __restrict__ D
   const int nx = m.n[0], ny = m.n[1], nz = m.n[2];
   const int64_t V = m.V;
   const int64_t P = (int64_t)nx * ny;
-  const int x0 = tile_x * TX, y0 = tile_y * TY;
+  const int x0 = tile_x * wx, y0 = tile_y * wy;
   const int z0 = tile_z * zchunk;
   const int z1 = min(z0 + zchunk, nz);
   int x = x0 - 1 + tx, y = y0 - 1 + ty;
-  const bool inside = live && tx >= 1 && tx <= TX && ty >= 1 && ty <= TY && x < nx && y < ny;
-  const bool bel = live && tx <= TX && ty <= TY;  // B' computed here (tile and low halo)
+  const bool inside = live && tx >= 1 && tx <= wx && ty >= 1 && ty <= wy && x < nx && y < ny;
+  const bool bel = live && tx <= wx && ty <= wy;  // B' computed here (tile and low halo)
   x = (x < 0) ? x + nx : (x >= nx ? x - nx : x);
   y = (y < 0) ? y + ny : (y >= ny ? y - ny : y);
   if (x >= nx) x = nx - 1;  // tiles wider than the mesh (unused values)
@@ -81,19 +89,25 @@ __device__ __forceinline__ void site_tile(const Mesh& m, const T* __restrict__ D
   auto ld3 = [&](const T* a, int k, T (&r)[3]) {
     if (!live) return;
     const T* p = a + (int64_t)k * P + off;
-    r[0] = p[0];
-    r[1] = p[V];
-    r[2] = p[2 * V];
+    r[0] = COH ? __ldcg(p) : p[0];
+    r[1] = COH ? __ldcg(p + V) : p[V];
+    r[2] = COH ? __ldcg(p + 2 * V) : p[2 * V];
   };
-  auto ldD = [&](int k, T (&r)[3]) {
-    ld3(Din, k, r);
-    if (!live || !Tp) return;
+  // pending transfers: the words of a plane are loaded beside its D, and
+  // added once every load of the moment has been issued
+  auto ldT = [&](int k, long long (&t)[3]) {
+    if (!Tp) return;
+    t[0] = t[1] = t[2] = 0;
+    if (!live) return;
     const long long* q = Tp + tw_index(0, (int64_t)k * P + off, V);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const long long t = q[c * V];
-      if (t != 0) r[c] = r[c] + pending_inc<T>(t, tscale, exact32);
-    }
+    for (int c = 0; c < 3; ++c) t[c] = COH ? __ldcg(q + c * V) : q[c * V];
+  };
+  auto addT = [&](T (&r)[3], const long long (&t)[3]) {
+    if (!Tp) return;
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      if (t[c] != 0) r[c] = r[c] + pending_inc<T>(t[c], tscale, exact32);
   };
   auto putE = [&](int slot, const T (&d)[3], const T (&i)[3]) {
     if (!live) return;
@@ -132,24 +146,33 @@ __device__ __forceinline__ void site_tile(const Mesh& m, const T* __restrict__ D
   for (int j = 0; j < PF + 1; ++j) bq[j][0] = bq[j][1] = bq[j][2] = T(0);
   {
     T dm[3] = {}, im[3] = {}, bm[3] = {}, i0[3] = {}, i1[3] = {};
+    long long tm[3], t0[3], t1[3], t2[3];
     const int zm = wrapz(z0 - 1), zp = wrapz(z0 + 1);
-    ldD(zm, dm);
+    ld3(Din, zm, dm);
+    ldT(zm, tm);
     ld3(ie, zm, im);
     ld3(Bin, zm, bm);
-    ldD(z0, dq[0]);
+    ld3(Din, z0, dq[0]);
+    ldT(z0, t0);
     ld3(ie, z0, i0);
     ld3(Bin, z0, bq[0]);
-    ldD(zp, dq[1]);
+    ld3(Din, zp, dq[1]);
+    ldT(zp, t1);
     ld3(ie, zp, i1);
 #pragma unroll
     for (int j = 0; j + 1 < PF; ++j)  // planes z0+2 .. z0+PF
       if (z0 + 2 + j <= z1) {
-        ldD(wrapz(z0 + 2 + j), dq[2 + j]);
+        ld3(Din, wrapz(z0 + 2 + j), dq[2 + j]);
+        ldT(wrapz(z0 + 2 + j), t2);
         ld3(ie, wrapz(z0 + 2 + j), iq[j]);
       }
 #pragma unroll
     for (int j = 1; j < PF; ++j)  // planes z0+1 .. z0+PF-1
       if (z0 + j < z1) ld3(Bin, wrapz(z0 + j), bq[j]);
+    addT(dm, tm);
+    addT(dq[0], t0);
+    addT(dq[1], t1);
+    if (PF > 1 && z0 + 2 <= z1) addT(dq[2], t2);
     putE(0, dm, im);
     putE(1, dq[0], i0);
     putE(2, dq[1], i1);
@@ -159,8 +182,11 @@ __device__ __forceinline__ void site_tile(const Mesh& m, const T* __restrict__ D
   int ec = 1, en = 2, ef = 0, bp = 0, bcs = 1;
   for (int k = z0; k < z1; ++k) {
     // issue plane k+PF+1 of D and 1/eps, plane k+PF of B
-    if (k + PF + 1 <= z1) {
-      ldD(wrapz(k + PF + 1), dq[PF + 1]);
+    long long tn[3];
+    const bool more = k + PF + 1 <= z1;
+    if (more) {
+      ld3(Din, wrapz(k + PF + 1), dq[PF + 1]);
+      ldT(wrapz(k + PF + 1), tn);
       ld3(ie, wrapz(k + PF + 1), iq[PF - 1]);
     }
     if (k + PF < z1) ld3(Bin, wrapz(k + PF), bq[PF]);
@@ -175,6 +201,7 @@ __device__ __forceinline__ void site_tile(const Mesh& m, const T* __restrict__ D
       p[2 * V] = fma_t<T>(cD, ((By - sB[bcs][1][ty][tx - 1]) - Bx) + sB[bcs][0][ty - 1][tx],
                           dq[0][2]);
     }
+    if (more) addT(dq[PF + 1], tn);
     if (k + 1 < z1) putE(ef, dq[2], iq[0]);  // E(k+2), read from the next iteration on
 #pragma unroll
     for (int j = 0; j < PF + 1; ++j)
