@@ -525,7 +525,8 @@ static memd_status autotune_fused(memd_ctx* c) {
   // asked for alone and not fitting, the site kernel's shapes stand in
   if (fk == MEMD_FIELD_AUTO || fk == MEMD_FIELD_ROWS) {
     const bool fits = rows_setup(c, 256);
-    for (int nt = 256; nt <= 512 && fits; nt *= 2) {
+    for (const int nt : {256, 512, kRowsWide}) {
+      if (!fits) break;
       FusedCfg r = fused_default(c->mesh);
       r.tma = 0;
       r.site = 0;

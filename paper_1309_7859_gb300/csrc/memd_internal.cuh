@@ -401,6 +401,9 @@ struct RowSeg {
   int rep, y0, rows, za, zb;
 };
 // row kernel: sites a thread (16 bytes of the field type), CTAs an SM, launch
+// threads a CTA: 256, 512, or kRowsWide, the most whose staged planes fit
+// shared memory (seven tile rows and two halo rows of 256 FP32 sites)
+constexpr int kRowsWide = 576;
 size_t rows_smem_bytes(int nt, size_t esz);
 int rows_sites_per_thread(int prec);
 int rows_occupancy(int prec, int nt);

@@ -106,6 +106,7 @@ size_t rows_smem_bytes(int nt, size_t esz) {
 int rows_sites_per_thread(int prec) { return prec == 1 ? 4 : 2; }
 
 int rows_occupancy(int prec, int nt) {
+  if (nt == kRowsWide) return prec == 1 ? rows_occ<float, kRowsWide>() : rows_occ<double, kRowsWide>();
   if (prec == 1) return nt == 256 ? rows_occ<float, 256>() : rows_occ<float, 512>();
   return nt == 256 ? rows_occ<double, 256>() : rows_occ<double, 512>();
 }
@@ -114,6 +115,9 @@ cudaError_t launch_rows_batch(int prec, const RepDesc* desc, const RowSeg* segs,
                               const int* seg_first, int nctas, int nt, int par, cudaStream_t st) {
   if (nctas <= 0) return cudaSuccess;
   const RowsArgs a{desc, segs, seg_first, par};
+  if (nt == kRowsWide)
+    return prec == 1 ? rows_launch<float, kRowsWide>(a, nctas, st)
+                     : rows_launch<double, kRowsWide>(a, nctas, st);
   if (prec == 1) return nt == 256 ? rows_launch<float, 256>(a, nctas, st) : rows_launch<float, 512>(a, nctas, st);
   return nt == 256 ? rows_launch<double, 256>(a, nctas, st) : rows_launch<double, 512>(a, nctas, st);
 }
@@ -124,6 +128,54 @@ cudaError_t launch_rows_batch(int prec, const RepDesc* desc, const RowSeg* segs,
 // planes
 constexpr long long kRowsFloor = 256;
 constexpr long long kRowsPro = 2;
+constexpr double kRowsL2Bytes = 150e6;  // fields beyond it leave L2 (129 MB) within a pass
+constexpr double kRowsSlack = 1.25;
+
+// Work split of one mesh whose fields do not fit L2: every tile cut at the
+// same planes, one segment a CTA.  All CTAs then walk through the planes
+// together, and a tile's halo rows, which its neighbours load as their own at
+// about the same time, come from L2; in the balanced cut neighbouring tiles
+// are at different planes and every halo row is read from DRAM again
+// (160^3: 192 MB read for 147 MB of fields, 160 MB so).  A pass over 192^3
+// takes 70.3 us against 78.2, over 256^3 164.7 (576 threads; 170.3 with 512)
+// against 199.8, which is 0.90 of the measured copy rate for its 60 bytes a
+// site, over 320^3 364 against 392; 128^3, 126 MB of fields, took 26.5
+// against 24.9 and keeps the balanced cut.  Taken when its longest segment is
+// at most `slack` of the balanced cut's load (320^3: 1.18 of it).
+static bool rows_plan_aligned(const memd_ctx* c, int maxrows, int nctas, double slack,
+                              std::vector<RowSeg>& segs, std::vector<int>& first) {
+  const int ny = c->mesh.n[1], nz = c->mesh.n[2];
+  const int ntmin = (ny + maxrows - 3) / (maxrows - 2);
+  int bt = 0, bc = 0;
+  double best = 1e300;
+  for (int cuts = 1; cuts * ntmin <= nctas && cuts <= nz; ++cuts) {
+    const int nt = std::min(nctas / cuts, ny);
+    const int rows = (ny + nt - 1) / nt, planes = (nz + cuts - 1) / cuts;
+    const double cost = (double)(rows + 2) * (planes + kRowsPro);
+    if (cost < best) {
+      best = cost;
+      bt = nt;
+      bc = cuts;
+    }
+  }
+  if (bt == 0) return false;
+  const int rt = (ny + ntmin - 1) / ntmin;
+  const double even = (double)ntmin * (rt + 2) * nz / nctas + kRowsPro * (rt + 2);
+  if (best > slack * even) return false;
+  segs.clear();
+  first.assign(nctas + 1, 0);
+  int cta = 0;
+  for (int k = 0; k < bc; ++k)
+    for (int t = 0; t < bt; ++t) {
+      const int y0 = (int)((int64_t)ny * t / bt), y1 = (int)((int64_t)ny * (t + 1) / bt);
+      const int za = (int)((int64_t)nz * k / bc), zb = (int)((int64_t)nz * (k + 1) / bc);
+      segs.push_back(RowSeg{0, y0, y1 - y0, za, zb});
+      first[++cta] = (int)segs.size();
+    }
+  while (cta < nctas) first[++cta] = (int)segs.size();
+  return true;
+}
+
 bool rows_plan(const std::vector<memd_ctx*>& m, int prec, int nt, int nctas,
                std::vector<RowSeg>& segs, std::vector<int>& first) {
   const int W = rows_sites_per_thread(prec);
@@ -152,6 +204,9 @@ bool rows_plan(const std::vector<memd_ctx*>& m, int prec, int nt, int nctas,
       tiles.push_back(Tile{(int)r, y0, rows, nz, w});
     }
   }
+  if (m.size() == 1 && 15.0 * memd_esz(m[0]) * m[0]->mesh.V > kRowsL2Bytes &&
+      rows_plan_aligned(m[0], nt / (m[0]->mesh.n[0] / W), nctas, kRowsSlack, segs, first))
+    return true;
   // Greedy cut in order with a capacity per CTA: a segment's first plane
   // also pays its prologue (the plane below and the wait for the first
   // planes), `pro` planes' worth.  The capacity is the least for which the
