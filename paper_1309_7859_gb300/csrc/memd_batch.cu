@@ -53,6 +53,8 @@ struct memd_batch {
   int2* d_apply_chunk = nullptr;
   int n_apply_chunk = 0;
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
+  cudaGraphExec_t run_graph[2] = {nullptr, nullptr};  // kRunSteps steps
+  int64_t run_steps = 0;  // steps since the step graphs were dropped
   // single-launch step (k_batch_step): the engine asked for, whether it runs,
   // its grid, the CTAs that start with field work, planes per field item, the
   // four work queues and the scheduling state
@@ -110,11 +112,17 @@ void drop(memd_batch* b) {
       cudaGraphExecDestroy(g);
       g = nullptr;
     }
+  for (cudaGraphExec_t& g : b->run_graph)
+    if (g) {
+      cudaGraphExecDestroy(g);
+      g = nullptr;
+    }
   for (cudaGraphExec_t& g : b->io_graph)
     if (g) {
       cudaGraphExecDestroy(g);
       g = nullptr;
     }
+  b->run_steps = 0;
 }
 
 void* balloc(memd_batch* b, size_t bytes) {
@@ -369,12 +377,12 @@ memd_status build_tables(memd_batch* b, bool sync = true) {
 }
 
 // the batch's field update: row kernel or site tiles
-cudaError_t launch_field(memd_batch* b, int par, cudaStream_t st) {
+cudaError_t launch_field(memd_batch* b, int par, cudaStream_t st, bool early = false) {
   if (b->f_rows > 0)
     return launch_rows_batch(b->prec, b->d_desc, b->d_segs, b->d_seg_first, b->n_rows_ctas,
-                             b->f_rows, par, st);
+                             b->f_rows, par, st, early);
   launch_fused_batch(b->prec, b->d_desc, b->d_field_rep, b->n_field, par, b->f_ty, b->f_pf,
-                     b->f_w, st);
+                     b->f_w, st, early);
   return cudaGetLastError();
 }
 
@@ -583,18 +591,17 @@ memd_status record(memd_batch* b, int par, int thermo, double gamma, double kT, 
   // writes): it is latency bound, the pass bandwidth bound, and the pass's
   // evict_first accesses leave the deposition's evict_last transfer words in
   // L2 for the application (64 replicas: 113.9 -> 109.8 us a step against
-  // the two in turn).  Moving the gather that closes a step beside the next
+  // the two in turn).  The pass is launched early behind the deposition: as
+  // two roots of a graph they started in either order, and a deposition that
+  // finds the SMs full of the pass's CTAs ends late, piled up on the first
+  // SMs that drain.  Moving the gather that closes a step beside the next
   // field pass, ahead of the deposition, was slower (116.9 us): the two
   // particle kernels in turn then outlast the pass.  Without overlap (the
   // request server, whose admission work runs on other streams meanwhile)
   // the two run in turn.
-  if (b->overlap) {
-    BCK(cudaEventRecord(b->fork, st));
-    BCK(cudaStreamWaitEvent(b->side, b->fork, 0));
-    deposit(b->side);
-    BCK(cudaEventRecord(b->join, b->side));
-    BCK(launch_field(b, par, st));
-    BCK(cudaStreamWaitEvent(st, b->join, 0));
+  if (b->overlap && (b->wide ? b->n_part_w : b->n_part) > 0) {
+    deposit(st);
+    BCK(launch_field(b, par, st, true));
   } else {
     BCK(launch_field(b, par, st));
     deposit(st);
@@ -849,22 +856,29 @@ memd_status memd_batch_step(memd_batch* b, int64_t nsteps, const memd_thermostat
   const double gamma = th ? th->gamma : 0.0, kT = th ? th->kT : 0.0;
   set_thermostat(b, thermo, gamma, kT);
   const bool timed = batch_timed(b);
-  for (int64_t s = 0; s < nsteps; ++s) {
+  for (int64_t s = 0; s < nsteps;) {
     const int par = b->bpar;
     harvest(b);
+    const int k = !b->single && !timed && nsteps - s >= kRunSteps &&
+                          (b->run_graph[par] || b->run_steps + nsteps - s >= kRunAfter)
+                      ? kRunSteps
+                      : 1;
     if (b->single && !b->single_graph_ok) {
       // the cooperative launch could not be captured here: launched directly
       const memd_status r = record(b, par, thermo, gamma, kT, timed);
       if (r != MEMD_OK) return r;
       b->timing_pending = timed;
       b->bpar ^= 1;
+      ++s;
       continue;
     }
-    cudaGraphExec_t& gx = b->graph[par];
+    cudaGraphExec_t& gx = k > 1 ? b->run_graph[par] : b->graph[par];
     if (!gx) {
       cudaGraph_t g = nullptr;
       BCK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
-      memd_status r = record(b, par, thermo, gamma, kT, timed);
+      memd_status r = MEMD_OK;
+      for (int j = 0; j < k && r == MEMD_OK; ++j)
+        r = record(b, par ^ (j & 1), thermo, gamma, kT, timed);
       cudaError_t e = cudaStreamEndCapture(b->stream, &g);
       if (r != MEMD_OK) {
         if (g) cudaGraphDestroy(g);
@@ -877,13 +891,14 @@ memd_status memd_batch_step(memd_batch* b, int64_t nsteps, const memd_thermostat
         if (!b->single) return bfail(b, MEMD_ERR_CUDA, "graph capture");
         cudaGetLastError();
         b->single_graph_ok = false;
-        --s;  // this step again, launched directly
-        continue;
+        continue;  // this step again, launched directly
       }
     }
     BCK(cudaGraphLaunch(gx, b->stream));
     b->timing_pending = timed;
-    b->bpar ^= 1;
+    b->bpar ^= k & 1;
+    b->run_steps += k;
+    s += k;
   }
   for (size_t r = 0; r < b->m.size(); ++r) b->m[r]->cur = (b->base[r] + b->bpar) & 1;
   return MEMD_OK;

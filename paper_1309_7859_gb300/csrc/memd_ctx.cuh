@@ -68,6 +68,8 @@ struct memd_ctx {
   int rows_nt = 0;       // a permittivity is mapped (memd_set_eps restores it on failure)
   // step graphs, one per buffer parity
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
+  cudaGraphExec_t run_graph[2] = {nullptr, nullptr};  // kRunSteps steps
+  int64_t run_steps = 0;  // steps since the step graphs were dropped
   // memd_step_io's whole round trip (copy in, unpack, step, pack, copy out)
   // as one graph per buffer parity; io_graph_ok false once capture failed
   cudaGraphExec_t io_graph[2] = {nullptr, nullptr};

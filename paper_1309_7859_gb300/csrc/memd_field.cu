@@ -329,6 +329,7 @@ __global__ void __launch_bounds__(34 * (TY + 2))
                  T cD, int zchunk) {
   site_tile<T, TY, PF>(m, Din, Bin, ie, Dout, Bout, cB, cD, blockIdx.x, blockIdx.y, blockIdx.z,
                        zchunk, threadIdx.x, threadIdx.y, true, CtaSync{});
+  wait_for_previous();
 }
 
 // Many independent systems in one launch: CTA b works on a site tile of
@@ -345,6 +346,7 @@ __global__ void __launch_bounds__((TX + 2) * (TY + 2))
                                     (T*)r.D[par ^ 1], (T*)r.B[par ^ 1], (T)r.sp.coefB,
                                     (T)r.sp.coefD, tx, ty, tz, r.f_zchunk, threadIdx.x,
                                     threadIdx.y, true, CtaSync{});
+  wait_for_previous();
 }
 
 template <typename T, int TX, int TY>
@@ -354,6 +356,7 @@ __global__ void __launch_bounds__(TX* TY)
                  T cD, int zchunk) {
   fused_tile<T, TX, TY>(m, Din, Bin, ie, Dout, Bout, cB, cD, blockIdx.x, blockIdx.y, blockIdx.z,
                         zchunk);
+  wait_for_previous();
 }
 
 
@@ -602,66 +605,69 @@ void launch_curl_D(const Mesh& m, int prec, void* D, const void* B, double coef,
 namespace {
 template <typename T, int TY>
 void fused_launch_t(const Mesh& m, const void* Din, const void* Bin, const void* ie, void* Dout,
-                    void* Bout, double cB, double cD, int zchunk, cudaStream_t st) {
+                    void* Bout, double cB, double cD, int zchunk, cudaStream_t st,
+                   bool early) {
   constexpr int TX = 32;
   const dim3 grid((m.n[0] + TX - 1) / TX, (m.n[1] + TY - 1) / TY, (m.n[2] + zchunk - 1) / zchunk);
-  k_fused_curl<T, TX, TY><<<grid, dim3(TX, TY, 1), 0, st>>>(
-      m, (const T*)Din, (const T*)Bin, (const T*)ie, (T*)Dout, (T*)Bout, (T)cB, (T)cD, zchunk);
+  launch_early(k_fused_curl<T, TX, TY>, grid, dim3(TX, TY, 1), 0, st, early, m, (const T*)Din,
+               (const T*)Bin, (const T*)ie, (T*)Dout, (T*)Bout, (T)cB, (T)cD, zchunk);
 }
 }  // namespace
 
 namespace {
 template <typename T, int TY, int PF>
 void site_launch_t(const Mesh& m, const void* Din, const void* Bin, const void* ie, void* Dout,
-                   void* Bout, double cB, double cD, int zchunk, cudaStream_t st) {
+                   void* Bout, double cB, double cD, int zchunk, cudaStream_t st,
+                   bool early) {
   const dim3 grid((m.n[0] + 31) / 32, (m.n[1] + TY - 1) / TY, (m.n[2] + zchunk - 1) / zchunk);
-  k_fused_site<T, TY, PF><<<grid, dim3(34, TY + 2, 1), 0, st>>>(
-      m, (const T*)Din, (const T*)Bin, (const T*)ie, (T*)Dout, (T*)Bout, (T)cB, (T)cD, zchunk);
+  launch_early(k_fused_site<T, TY, PF>, grid, dim3(34, TY + 2, 1), 0, st, early, m,
+               (const T*)Din, (const T*)Bin, (const T*)ie, (T*)Dout, (T*)Bout, (T)cB, (T)cD, zchunk);
 }
 template <typename T, int TY>
 void site_launch_pf(int pf, const Mesh& m, const void* Din, const void* Bin, const void* ie,
-                    void* Dout, void* Bout, double cB, double cD, int zchunk, cudaStream_t st) {
+                    void* Dout, void* Bout, double cB, double cD, int zchunk, cudaStream_t st,
+                   bool early) {
   if (pf >= 2)
-    site_launch_t<T, TY, 2>(m, Din, Bin, ie, Dout, Bout, cB, cD, zchunk, st);
+    site_launch_t<T, TY, 2>(m, Din, Bin, ie, Dout, Bout, cB, cD, zchunk, st, early);
   else
-    site_launch_t<T, TY, 1>(m, Din, Bin, ie, Dout, Bout, cB, cD, zchunk, st);
+    site_launch_t<T, TY, 1>(m, Din, Bin, ie, Dout, Bout, cB, cD, zchunk, st, early);
 }
 }  // namespace
 
 void launch_fused_curl(const Mesh& m, int prec, const void* Din, const void* Bin, const void* ie,
                        void* Dout, void* Bout, double cB, double cD, FusedCfg cfg,
-                       cudaStream_t st) {
+                       cudaStream_t st, bool early) {
   if (cfg.zchunk < 1) cfg = fused_default(m);
   if (cfg.zchunk > m.n[2]) cfg.zchunk = m.n[2];
   if (cfg.site) {
     const int pf = cfg.site;
     if (prec == 1) {
       if (cfg.ty == 4)
-        site_launch_pf<float, 4>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
+        site_launch_pf<float, 4>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
       else if (cfg.ty == 16)
-        site_launch_pf<float, 16>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
+        site_launch_pf<float, 16>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
       else
-        site_launch_pf<float, 8>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
+        site_launch_pf<float, 8>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
     } else {
       if (cfg.ty == 4)
-        site_launch_pf<double, 4>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
+        site_launch_pf<double, 4>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
       else
-        site_launch_pf<double, 8>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
+        site_launch_pf<double, 8>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
     }
     return;
   }
   if (prec == 1) {
     switch (cfg.ty) {
-      case 4: fused_launch_t<float, 4>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st); break;
-      case 16: fused_launch_t<float, 16>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st); break;
-      default: fused_launch_t<float, 8>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
+      case 4: fused_launch_t<float, 4>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early); break;
+      case 16: fused_launch_t<float, 16>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early); break;
+      default: fused_launch_t<float, 8>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
     }
   } else {
     // FP64 tiles stop at 8 rows: 16 would exceed the 48 KB of static shared memory
     if (cfg.ty == 4)
-      fused_launch_t<double, 4>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
+      fused_launch_t<double, 4>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
     else
-      fused_launch_t<double, 8>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
+      fused_launch_t<double, 8>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
   }
 }
 
@@ -682,41 +688,43 @@ FusedCfg fused_default(const Mesh& m) {
 namespace {
 template <typename T, int TY, int PF>
 void batch_launch_t(const RepDesc* desc, const int* cta_rep, int nctas, int par, int tw,
-                    cudaStream_t st) {
+                    cudaStream_t st, bool early) {
   if (tw == 16)
-    k_fused_site_batch<T, TY, PF, 16><<<nctas, dim3(18, TY + 2, 1), 0, st>>>(desc, cta_rep, par);
+    launch_early(k_fused_site_batch<T, TY, PF, 16>, nctas, dim3(18, TY + 2, 1), 0, st, early, desc,
+                 cta_rep, par);
   else
-    k_fused_site_batch<T, TY, PF, 32><<<nctas, dim3(34, TY + 2, 1), 0, st>>>(desc, cta_rep, par);
+    launch_early(k_fused_site_batch<T, TY, PF, 32>, nctas, dim3(34, TY + 2, 1), 0, st, early, desc,
+                 cta_rep, par);
 }
 template <typename T>
 void batch_launch_ty(const RepDesc* desc, const int* cta_rep, int nctas, int par, int ty, int pf,
-                     int tw, cudaStream_t st) {
+                     int tw, cudaStream_t st, bool early) {
   if (ty == 4) {
     if (pf >= 2)
-      batch_launch_t<T, 4, 2>(desc, cta_rep, nctas, par, tw, st);
+      batch_launch_t<T, 4, 2>(desc, cta_rep, nctas, par, tw, st, early);
     else
-      batch_launch_t<T, 4, 1>(desc, cta_rep, nctas, par, tw, st);
+      batch_launch_t<T, 4, 1>(desc, cta_rep, nctas, par, tw, st, early);
   } else if (ty == 16 && sizeof(T) == 4) {
     if (pf >= 2)
-      batch_launch_t<float, 16, 2>(desc, cta_rep, nctas, par, tw, st);
+      batch_launch_t<float, 16, 2>(desc, cta_rep, nctas, par, tw, st, early);
     else
-      batch_launch_t<float, 16, 1>(desc, cta_rep, nctas, par, tw, st);
+      batch_launch_t<float, 16, 1>(desc, cta_rep, nctas, par, tw, st, early);
   } else {
     if (pf >= 2)
-      batch_launch_t<T, 8, 2>(desc, cta_rep, nctas, par, tw, st);
+      batch_launch_t<T, 8, 2>(desc, cta_rep, nctas, par, tw, st, early);
     else
-      batch_launch_t<T, 8, 1>(desc, cta_rep, nctas, par, tw, st);
+      batch_launch_t<T, 8, 1>(desc, cta_rep, nctas, par, tw, st, early);
   }
 }
 }  // namespace
 
 void launch_fused_batch(int prec, const RepDesc* desc, const int* cta_rep, int nctas, int par,
-                        int ty, int pf, int tw, cudaStream_t st) {
+                        int ty, int pf, int tw, cudaStream_t st, bool early) {
   if (nctas <= 0) return;
   if (prec == 1)
-    batch_launch_ty<float>(desc, cta_rep, nctas, par, ty, pf, tw, st);
+    batch_launch_ty<float>(desc, cta_rep, nctas, par, ty, pf, tw, st, early);
   else
-    batch_launch_ty<double>(desc, cta_rep, nctas, par, ty, pf, tw, st);
+    batch_launch_ty<double>(desc, cta_rep, nctas, par, ty, pf, tw, st, early);
 }
 
 int fused_candidates(const Mesh& m, int prec, FusedCfg* out, int cap) {

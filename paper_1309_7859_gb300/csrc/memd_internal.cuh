@@ -35,6 +35,8 @@ struct Mesh {
   double inv_a;  // 1 / a; used instead of the division when a is a power of two
   int a_pow2;    // (x * inv_a == x / a exactly then)
   double inv_aS; // S / a (exact when a is a power of two)
+  int wexp;      // its exponent then: S / a = 2^wexp
+  long long step_max;  // bits of 2 a, the longest move accepted (a double)
 };
 
 // The transfer buffer and the ledger of a system share one allocation of
@@ -128,6 +130,46 @@ __device__ __forceinline__ unsigned long long exch_hint(unsigned long long* a, u
   return r;
 }
 
+// Steps of the graph engine recorded as one graph: between two graph launches
+// the device idles 2.8-4.5 us, between two nodes about 1 (64^3 with 32768
+// charges 36.0 -> 33.1 us a step of a 20-step call).  Recorded once
+// a caller has asked for kRunAfter steps of the same set-up; shorter runs do
+// not repay the recording of eight steps.
+constexpr int kRunSteps = 8;
+constexpr int64_t kRunAfter = 32;
+
+// Programmatic dependent launch.  A kernel launched early (launch_early with
+// early set) may start once every CTA of the kernel before it in its stream
+// has called let_next_start (or left); wait_for_previous then returns when
+// that kernel has completed and its writes are visible.  Without the early
+// launch both calls are no-ops.  The field kernels are the only ones launched
+// early, behind the charge transfer, whose data they do not touch: they wait
+// as their last statement, so that what follows them follows both.  (The
+// application and the gather are not: their CTAs, placed while the kernel
+// before them still held SMs, piled up unevenly, and 256^3 with 100k charges
+// took 370 us a step for 300.)
+__device__ __forceinline__ void wait_for_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void let_next_start() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... K, typename... A>
+inline cudaError_t launch_early(void (*kernel)(K...), dim3 grid, dim3 block, size_t smem,
+                                cudaStream_t st, bool early, A&&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // ------------------------------------------------------------ field kernels
 // (memd_field.cu)
 void launch_curl_B(const Mesh& m, int prec, void* B, const void* D, const void* ie,
@@ -146,7 +188,7 @@ struct FusedCfg {
 };
 void launch_fused_curl(const Mesh& m, int prec, const void* Din, const void* Bin, const void* ie,
                        void* Dout, void* Bout, double cB, double cD, FusedCfg cfg,
-                       cudaStream_t st);
+                       cudaStream_t st, bool early = false);
 FusedCfg fused_default(const Mesh& m);
 // candidate shapes for the autotuner; returns how many were written
 int fused_candidates(const Mesh& m, int prec, FusedCfg* out, int cap);
@@ -408,7 +450,8 @@ size_t rows_smem_bytes(int nt, size_t esz);
 int rows_sites_per_thread(int prec);
 int rows_occupancy(int prec, int nt);
 cudaError_t launch_rows_batch(int prec, const RepDesc* desc, const RowSeg* segs,
-                              const int* seg_first, int nctas, int nt, int par, cudaStream_t st);
+                              const int* seg_first, int nctas, int nt, int par, cudaStream_t st,
+                              bool early = false);
 // ------------------------------------------- single-launch batch step
 // (memd_particles.cu) The whole step of every replica in one cooperative
 // launch of persistent CTAs that claim work: field segments (a row tile over
@@ -469,7 +512,7 @@ int batch_step_occupancy(int prec);
 cudaError_t launch_batch_step(int prec, const BatchStepArgs& a, int grid, cudaStream_t st);
 // field update of every replica (memd_field.cu)
 void launch_fused_batch(int prec, const RepDesc* desc, const int* cta_rep, int nctas, int par,
-                        int ty, int pf, int tw, cudaStream_t st);
+                        int ty, int pf, int tw, cudaStream_t st, bool early = false);
 // the batch's host I/O block (memd_batch_step_io): the members' particles in
 // order, member r from entry off[r] of ntot = off[count]; io_layout(ntot),
 // with count error words at its err offset

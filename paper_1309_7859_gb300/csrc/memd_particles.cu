@@ -43,9 +43,21 @@ inline int quad_threads(int64_t n) {
 }
 
 // ------------------------------------------------------------ fixed point
+// GB300's FP64 pipe takes 64 to 77 cycles a warp instruction, with no overlap
+// inside a warp, so what the bits of a double decide is decided there, by
+// integers: the order of non-negative doubles is that of their bits, and a
+// negative one (or a NaN) reads as larger than every finite bound.
+__device__ __forceinline__ bool in_box(double x, double L) {  // 0 <= x < L
+  return (unsigned long long)__double_as_longlong(x) < (unsigned long long)__double_as_longlong(L);
+}
+__device__ __forceinline__ bool short_step(const Mesh& m, double s) {  // |s| <= 2 a
+  return (__double_as_longlong(s) & 0x7fffffffffffffffll) <= m.step_max;
+}
+
 // Sec. V periodic stitching: shift by whole box lengths into [0, L); a sum
 // that rounds up to L starts the next image.  Callers bound |x| by a few L.
 __device__ inline void fold(double L, double& x, int& img) {
+  if (in_box(x, L)) return;
   double y = x;
   int k = 0;
   while (y >= L) {
@@ -64,12 +76,25 @@ __device__ inline void fold(double L, double& x, int& img) {
   img += k;
 }
 
+// floor(x S / a) for a power-of-two spacing and 0 <= x, from the bits of x:
+// the product is exact, so its integer part is the mantissa shifted by the
+// exponents (the FP64 product and conversion give the same).  False for what
+// the shift does not cover (negative, NaN, 2^48 and beyond).
+__device__ __forceinline__ bool lattice_steps(const Mesh& m, double x, long long& W) {
+  const long long b = __double_as_longlong(x);
+  const int e = (int)(b >> 52) - 1023 + m.wexp;  // binary exponent of x S / a
+  if (b < 0 || e > 47) return false;
+  W = e < 0 ? 0 : ((b & 0xfffffffffffffll) | 0x10000000000000ll) >> (52 - e);
+  return true;
+}
+
 // cell c = floor(x / a) and sub-cell step f = floor((x/a - c) S).  When a is
 // a power of two, x / a, x / a - c and the scaling by S are all exact, so
 // floor(x S / a) = c S + f holds both in one rounding-free product.
 __device__ inline void quantize(const Mesh& m, int d, double x, int& c, int& f) {
   if (m.a_pow2) {
-    const long long W = __double2ll_rd(__dmul_rn(x, m.inv_aS));
+    long long W;
+    if (!lattice_steps(m, x, W)) W = __double2ll_rd(__dmul_rn(x, m.inv_aS));
     const long long cw = W >> kWBits;  // floor(W / S)
     if (cw >= (long long)m.n[d]) {
       c = m.n[d] - 1;
@@ -105,13 +130,47 @@ __device__ inline long long wgt(int f, int a) { return a ? (long long)f : (long 
 // look one cell beyond a quantised cell, so no integer division is needed
 __device__ inline int wrap1(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 
-// the vertex a link leaves (its cell coordinates wrapped once)
-__device__ inline int64_t link_vertex(const Mesh& m, int ci, int cj, int ck) {
-  return vindex(m, wrap1(ci, m.n[0]), wrap1(cj, m.n[1]), wrap1(ck, m.n[2]));
+// The step kernels index vertices, links and transfer words by 32 bits: a
+// mesh has less than 2^31 links, so less than 2^32 transfer and ledger words.
+// One warp instruction a charge's 32-bit sum costs takes several in 64 bits,
+// and these kernels wait on their instruction count (1200 a warp of 32
+// charges in the deposition, 760 in the gather, at under two warps a
+// scheduler: 64^3, 32768 charges).
+__device__ inline unsigned link_vertex(const Mesh& m, int ci, int cj, int ck) {
+  return (unsigned)wrap1(ci, m.n[0]) +
+         (unsigned)m.n[0] * ((unsigned)wrap1(cj, m.n[1]) +
+                             (unsigned)m.n[1] * (unsigned)wrap1(ck, m.n[2]));
 }
 
-__device__ inline int64_t link_index(const Mesh& m, int d, int ci, int cj, int ck) {
-  return (int64_t)d * m.V + link_vertex(m, ci, cj, ck);
+__device__ inline unsigned link_index(const Mesh& m, int d, int ci, int cj, int ck) {
+  return (unsigned)d * (unsigned)m.V + link_vertex(m, ci, cj, ck);
+}
+
+// the flat index shares of a cell's coordinate and of the next one along
+// each axis: vertex (a, b, c) of the cell is x[a] + y[b] + z[c]
+struct CellShares {
+  unsigned x[2], y[2], z[2];
+};
+__device__ __forceinline__ CellShares cell_shares(const Mesh& m, const int c[3]) {
+  const unsigned nx = (unsigned)m.n[0], P = nx * (unsigned)m.n[1];
+  CellShares s;
+  s.x[0] = (unsigned)c[0];
+  s.y[0] = (unsigned)c[1] * nx;
+  s.z[0] = (unsigned)c[2] * P;
+  s.x[1] = c[0] + 1 == m.n[0] ? 0u : s.x[0] + 1u;
+  s.y[1] = c[1] + 1 == m.n[1] ? 0u : s.y[0] + nx;
+  s.z[1] = c[2] + 1 == m.n[2] ? 0u : s.z[0] + P;
+  return s;
+}
+// vertex at corner (a1, a2) of the axes after d, cyclically
+__device__ __forceinline__ unsigned corner_vertex(const CellShares& s, int d, int a1, int a2) {
+  if (d == 0) return s.x[0] + (a1 ? s.y[1] : s.y[0]) + (a2 ? s.z[1] : s.z[0]);
+  if (d == 1) return (a2 ? s.x[1] : s.x[0]) + s.y[0] + (a1 ? s.z[1] : s.z[0]);
+  return (a1 ? s.x[1] : s.x[0]) + (a2 ? s.y[1] : s.y[0]) + s.z[0];
+}
+// tw_index in 32 bits
+__device__ __forceinline__ unsigned tw_word(int d, unsigned v, unsigned cmV) {
+  return cmV ? (unsigned)d * cmV + v : (unsigned)kLT * (3u * v + (unsigned)d);
 }
 
 // warp-aggregated int64 atomic add into a device word
@@ -206,47 +265,43 @@ __device__ inline double unit_noise(unsigned r) {
 __device__ inline int sel3(int d, int a, int b, int c) { return d == 0 ? a : (d == 1 ? b : c); }
 
 // cmV: the layout of Tb (tw_index)
-__device__ inline void deposit_axis(const Mesh& m, int d, int q, int c0, int f0, int f1, int dc,
-                                    const int cc[3], const int cf[3],
-                                    unsigned long long* __restrict__ Tb, int64_t cmV = 0) {
-  // axis d is the lane's own (a run-time value): select sizes, strides and
-  // perpendicular coordinates instead of indexing arrays with it
+__device__ __forceinline__ void deposit_axis(const Mesh& m, int d, int q, int c0, int f0, int f1,
+                                             int dc, const int cc[3], const int cf[3],
+                                             unsigned long long* __restrict__ Tb,
+                                             unsigned cmV = 0) {
+  // axis d may be the lane's own (a run-time value): select sizes, strides
+  // and perpendicular coordinates instead of indexing arrays with it
   const int e1 = d == 2 ? 0 : d + 1, e2 = d == 0 ? 2 : d - 1;
-  const int64_t st[3] = {1, (int64_t)m.n[0], (int64_t)m.n[0] * m.n[1]};
+  const unsigned s1x = (unsigned)m.n[0], s2x = s1x * (unsigned)m.n[1];
   const int nd = sel3(d, m.n[0], m.n[1], m.n[2]);
   const int n1 = sel3(e1, m.n[0], m.n[1], m.n[2]), n2 = sel3(e2, m.n[0], m.n[1], m.n[2]);
-  const int64_t sd = d == 0 ? st[0] : (d == 1 ? st[1] : st[2]);
-  const int64_t s1 = e1 == 0 ? st[0] : (e1 == 1 ? st[1] : st[2]);
-  const int64_t s2 = e2 == 0 ? st[0] : (e2 == 1 ? st[1] : st[2]);
+  const unsigned sd = d == 0 ? 1u : (d == 1 ? s1x : s2x);
+  const unsigned s1 = e1 == 0 ? 1u : (e1 == 1 ? s1x : s2x);
+  const unsigned s2 = e2 == 0 ? 1u : (e2 == 1 ? s1x : s2x);
   const int v0 = sel3(e1, cc[0], cc[1], cc[2]), w0 = sel3(e2, cc[0], cc[1], cc[2]);
-  const int fv = sel3(e1, cf[0], cf[1], cf[2]), fw = sel3(e2, cf[0], cf[1], cf[2]);
-  // vertex indices of the old and new cell along d (the link's pair is
-  // tl_pair(d, vertex))
-  const int64_t u0 = (int64_t)wrap1(c0, nd) * sd;
-  const int64_t u1 = (int64_t)wrap1(c0 + dc, nd) * sd;
+  const unsigned fv = (unsigned)sel3(e1, cf[0], cf[1], cf[2]);
+  const unsigned fw = (unsigned)sel3(e2, cf[0], cf[1], cf[2]);
+  // index shares of the old and new cell along d and of the corners
+  const unsigned u0 = (unsigned)c0 * sd, u1 = (unsigned)wrap1(c0 + dc, nd) * sd;
+  const unsigned p0 = (unsigned)v0 * s1, p1 = v0 + 1 == n1 ? 0u : p0 + s1;
+  const unsigned r0 = (unsigned)w0 * s2, r1 = w0 + 1 == n2 ? 0u : r0 + s2;
+  // signed sub-cell steps made in the old and in the new cell
+  const int old = dc == 0 ? f1 - f0 : (dc > 0 ? (int)kS - f0 : -f0);
+  const int fresh = dc == 0 ? 0 : (dc > 0 ? f1 : f1 - (int)kS);
+  const long long A0 = -(long long)q * old, A1 = -(long long)q * fresh;
+  const unsigned long long pol = l2_policy_last();
 #pragma unroll
   for (int a2 = 0; a2 < 2; ++a2)
 #pragma unroll
     for (int a1 = 0; a1 < 2; ++a1) {
-      const long long wp = wgt(fv, a1) * wgt(fw, a2);
-      if (wp == 0) continue;
-      const int64_t perp = (int64_t)wrap1(v0 + a1, n1) * s1 + (int64_t)wrap1(w0 + a2, n2) * s2;
-      const int64_t l0 = u0 + perp;
-      if (dc == 0) {
-        const long long t = -(long long)q * (long long)(f1 - f0) * wp;
-        if (t) red_add_hint(&Tb[tw_index(d, l0, cmV)], (unsigned long long)t, l2_policy_last());
-      } else if (dc == 1) {
-        const int64_t l1 = u1 + perp;
-        const long long t0 = -(long long)q * (long long)(kS - f0) * wp;
-        const long long t1 = -(long long)q * (long long)f1 * wp;
-        if (t0) red_add_hint(&Tb[tw_index(d, l0, cmV)], (unsigned long long)t0, l2_policy_last());
-        if (t1) red_add_hint(&Tb[tw_index(d, l1, cmV)], (unsigned long long)t1, l2_policy_last());
-      } else {
-        const int64_t l1 = u1 + perp;
-        const long long t0 = (long long)q * (long long)f0 * wp;
-        const long long t1 = (long long)q * (long long)(kS - f1) * wp;
-        if (t0) red_add_hint(&Tb[tw_index(d, l0, cmV)], (unsigned long long)t0, l2_policy_last());
-        if (t1) red_add_hint(&Tb[tw_index(d, l1, cmV)], (unsigned long long)t1, l2_policy_last());
+      const long long wp =
+          (long long)((unsigned long long)(a1 ? fv : (unsigned)kS - fv) * (a2 ? fw : (unsigned)kS - fw));
+      const unsigned perp = (a1 ? p1 : p0) + (a2 ? r1 : r0);
+      const long long t0 = A0 * wp;
+      if (t0) red_add_hint(&Tb[tw_word(d, u0 + perp, cmV)], (unsigned long long)t0, pol);
+      if (dc != 0) {
+        const long long t1 = A1 * wp;
+        if (t1) red_add_hint(&Tb[tw_word(d, u1 + perp, cmV)], (unsigned long long)t1, pol);
       }
     }
 }
@@ -291,14 +346,12 @@ __device__ inline long long quad_move(const Mesh& m, Particles P, int64_t p, int
   }
   if (pf_ie && active) {
     // quad lane d holds corner (d & 1, d >> 1): its three links of the final cell
-    const int a1 = d & 1, a2 = d >> 1;
+    const int at[3] = {all_ok ? C1[0] : C0[0], all_ok ? C1[1] : C0[1], all_ok ? C1[2] : C0[2]};
+    const CellShares cs = cell_shares(m, at);
 #pragma unroll
     for (int e = 0; e < 3; ++e) {
-      const int e1 = (e + 1) % 3, e2 = (e + 2) % 3;
-      int at[3] = {all_ok ? C1[0] : C0[0], all_ok ? C1[1] : C0[1], all_ok ? C1[2] : C0[2]};
-      at[e1] += a1;
-      at[e2] += a2;
-      const char* a = pf_ie + link_index(m, e, at[0], at[1], at[2]) * pf_es;
+      const char* a =
+          pf_ie + (size_t)((unsigned)e * (unsigned)m.V + corner_vertex(cs, e, d & 1, d >> 1)) * pf_es;
       asm volatile("prefetch.global.L2 [%0];" ::"l"(a));
     }
     if (d == 0) {
@@ -317,7 +370,7 @@ __device__ inline long long quad_move(const Mesh& m, Particles P, int64_t p, int
         cc[e] = (e < d) ? C1[e] : C0[e];
         cf[e] = (e < d) ? F1[e] : F0[e];
       }
-      deposit_axis(m, d, P.q[p], c0, f0, f1, dc, cc, cf, Tb, cmV);
+      deposit_axis(m, d, P.q[p], c0, f0, f1, dc, cc, cf, Tb, (unsigned)cmV);
       P.x[3 * p + d] = xn;
       P.img[3 * p + d] = kn;
       mv[d] = c0;
@@ -439,7 +492,7 @@ __device__ __forceinline__ long long deposit_body(const Mesh& m, const StepParam
     ko = P.img[3 * p + d];
     kn = ko;
     xn = x;
-    if (fabs(step) <= 2.0 * m.a) {
+    if (short_step(m, step)) {
       xn = __dadd_rn(x, step);
       fold(m.L[d], xn, kn);
     } else {
@@ -474,7 +527,7 @@ __device__ __forceinline__ void deposit_wide(const Mesh& m, const StepParams& sp
     ko[d] = P.img[3 * p + d];
     kn[d] = ko[d];
     xn[d] = x[d];
-    if (fabs(step) <= 2.0 * m.a) {
+    if (short_step(m, step)) {
       xn[d] = __dadd_rn(x[d], step);
     } else {
       ok = false;
@@ -484,24 +537,8 @@ __device__ __forceinline__ void deposit_wide(const Mesh& m, const StepParams& sp
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     quantize(m, d, x[d], c0[d], f0[d]);
-    // With a power-of-two spacing the product x S / a is exact, so xn lies in
-    // [0, L) exactly when 0 <= floor(xn S / a) < n S: the quantised value then
-    // is the cell and step of the folded position, and the fold's FP64
-    // comparisons are skipped (GB300's FP64 pipe is narrow).  Otherwise fold
-    // and quantise as the other kernels do; the results are the same.
-    bool inside = false;
-    if (m.a_pow2) {
-      const long long W = __double2ll_rd(__dmul_rn(xn[d], m.inv_aS));
-      if (W >= 0 && W < (long long)m.n[d] * kS) {
-        inside = true;
-        c1[d] = (int)(W >> kWBits);
-        f1[d] = (int)(W & (kS - 1));
-      }
-    }
-    if (!inside) {
-      fold(m.L[d], xn[d], kn[d]);
-      quantize(m, d, xn[d], c1[d], f1[d]);
-    }
+    fold(m.L[d], xn[d], kn[d]);
+    quantize(m, d, xn[d], c1[d], f1[d]);
     dc[d] = c1[d] + (kn[d] - ko[d]) * m.n[d] - c0[d];
     if (dc[d] < -1 || dc[d] > 1) ok = false;
   }
@@ -539,6 +576,7 @@ __device__ __forceinline__ void deposit_wide(const Mesh& m, const StepParams& sp
 __global__ void __launch_bounds__(kWideThreads)
     k_deposit_wide(const __grid_constant__ Mesh m, const __grid_constant__ StepParams sp,
                    Particles P, unsigned long long* __restrict__ Tb, DevState* ds) {
+  let_next_start();
   long long U[3];
   deposit_wide(m, sp, P, Tb, ds, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, U);
   cta_dipole_add3(ds->Pacc, U);
@@ -548,6 +586,7 @@ __global__ void __launch_bounds__(kQuadThreads)
     k_kick_drift_deposit(const __grid_constant__ Mesh m, const __grid_constant__ StepParams sp,
                          Particles P, unsigned long long* __restrict__ Tb,
                          DevState* ds) {
+  let_next_start();
   cta_dipole_add(ds->Pacc,
                  deposit_body(m, sp, P, Tb, ds, blockIdx.x * (int64_t)blockDim.x + threadIdx.x));
 }
@@ -596,24 +635,28 @@ __device__ __forceinline__ void apply_body(const Mesh& m, Particles P,
   const int c0[3] = {__ldcg(mv), __ldcg(mv + 1), __ldcg(mv + 2)};
   const int c1[3] = {__ldcg(mv + 3), __ldcg(mv + 4), __ldcg(mv + 5)};
   // slot 2d: the d-link at the old cell along d; slot 2d+1: at the new
-  // cell, when the move crossed a face; v: the vertex the link leaves
-  int64_t v[6];
+  // cell, when the move crossed a face; v: the vertex the link leaves.  The
+  // perpendicular cells are those at the time of the move along d: axes
+  // before d have moved, axes after d have not.
+  const unsigned st[3] = {1u, (unsigned)m.n[0], (unsigned)m.n[0] * (unsigned)m.n[1]};
+  unsigned o0[3], o1[3], n0[3], n1[3];  // index shares: old and new cell, and the next one of each
+#pragma unroll
+  for (int e = 0; e < 3; ++e) {
+    o0[e] = (unsigned)c0[e] * st[e];
+    n0[e] = (unsigned)c1[e] * st[e];
+    o1[e] = c0[e] + 1 == m.n[e] ? 0u : o0[e] + st[e];
+    n1[e] = c1[e] + 1 == m.n[e] ? 0u : n0[e] + st[e];
+  }
+  unsigned v[6];
   bool has[6];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const int e1 = (d + 1) % 3, e2 = (d + 2) % 3;
-    // perpendicular cells at the time of the move along d: axes before d
-    // have moved, axes after d have not
-    const int p1 = (e1 < d) ? c1[e1] : c0[e1];
-    const int p2 = (e2 < d) ? c1[e2] : c0[e2];
-    int at[3];
-    at[e1] = p1 + a1;
-    at[e2] = p2 + a2;
-    at[d] = c0[d];
-    v[2 * d] = link_vertex(m, at[0], at[1], at[2]);
+    const unsigned q1 = e1 < d ? (a1 ? n1[e1] : n0[e1]) : (a1 ? o1[e1] : o0[e1]);
+    const unsigned q2 = e2 < d ? (a2 ? n1[e2] : n0[e2]) : (a2 ? o1[e2] : o0[e2]);
+    v[2 * d] = o0[d] + q1 + q2;
     has[2 * d] = true;
-    at[d] = c1[d];
-    v[2 * d + 1] = link_vertex(m, at[0], at[1], at[2]);
+    v[2 * d + 1] = n0[d] + q1 + q2;
     has[2 * d + 1] = c1[d] != c0[d];
   }
   // the transfer and ledger words stay in L2 for the gather's ledger reads
@@ -621,16 +664,17 @@ __device__ __forceinline__ void apply_body(const Mesh& m, Particles P,
   long long t[6];
 #pragma unroll
   for (int s = 0; s < 6; ++s)
-    t[s] = has[s] ? (long long)exch_hint(&Tb[tw_index(s >> 1, v[s], cmV)], 0ull, pol) : 0ll;
+    t[s] = has[s] ? (long long)exch_hint(&Tb[tw_word(s >> 1, v[s], (unsigned)cmV)], 0ull, pol)
+                  : 0ll;
   // only the lane that took a link's transfer adds it, so each reduction
   // below is the one addition to its word in this kernel: exact for the
   // ledger, D + x rounded once for the field
 #pragma unroll
   for (int s = 0; s < 6; ++s)
     if (t[s] != 0) {
-      red_add_hint((unsigned long long*)&Lg[kLT * tl_pair(s >> 1, v[s])], (unsigned long long)t[s],
+      red_add_hint((unsigned long long*)&Lg[tw_word(s >> 1, v[s], 0)], (unsigned long long)t[s],
                    pol);
-      atomicAdd(&D[(int64_t)(s >> 1) * m.V + v[s]], (T)((double)t[s] * scale));
+      atomicAdd(&D[(unsigned)(s >> 1) * (unsigned)m.V + v[s]], (T)((double)t[s] * scale));
     }
 }
 
@@ -901,19 +945,16 @@ __device__ __forceinline__ void gather_body(const Mesh& m, const StepParams& sp,
   if (active) {
     T Dv[3], Iv[3];
     double I64[3] = {0.0, 0.0, 0.0};
+    const CellShares cs = cell_shares(m, c);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      const int e1 = (d + 1) % 3, e2 = (d + 2) % 3;
-      int at[3] = {c[0], c[1], c[2]};
-      at[e1] += a1;
-      at[e2] += a2;
-      const int64_t vtx = link_vertex(m, at[0], at[1], at[2]);
-      const int64_t l = (int64_t)d * m.V + vtx;
+      const unsigned vtx = corner_vertex(cs, d, a1, a2);
+      const unsigned l = (unsigned)d * (unsigned)m.V + vtx;
       Dv[d] = __ldcg(D + l);  // D was updated in this launch by other CTAs (single launch)
       Iv[d] = ie[l];
       if (sp.self_mode != 0 && sizeof(T) == 8) I64[d] = ie64[l];
       if (Tpend) {  // transfers of this step not yet applied: as their application rounds
-        const long long t = __ldcg(Tpend + tw_index(d, vtx, m.V));  // the step's own buffer
+        const long long t = __ldcg(Tpend + l);  // the step's own slot: component major
         if (t != 0) Dv[d] = Dv[d] + pending_inc<T>(t, sp.scale, exact32);
       }
     }
@@ -1041,29 +1082,32 @@ __device__ __forceinline__ void gather_wide(const Mesh& m, const StepParams& sp,
     philox4x32_10(ctr, (unsigned)sp.seed, (unsigned)(sp.seed >> 32));
   }
   T Ek[4][3], iwk[4][3], itk[4];
+  const CellShares cs = cell_shares(m, c);
+  // every load of the cell's links before the first use
+  T Dv[4][3], Iv[4][3];
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      const unsigned l = (unsigned)d * (unsigned)m.V + corner_vertex(cs, d, k & 1, k >> 1);
+      Dv[k][d] = __ldcg(D + l);
+      Iv[k][d] = ie[l];
+    }
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int a1 = k & 1, a2 = k >> 1;
-    T Dv[3], Iv[3];
     double I64[3] = {0.0, 0.0, 0.0};
+    if (sp.self_mode != 0 && sizeof(T) == 8)
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const int e1 = (d + 1) % 3, e2 = (d + 2) % 3;
-      int at[3] = {c[0], c[1], c[2]};
-      at[e1] += a1;
-      at[e2] += a2;
-      const int64_t l = link_index(m, d, at[0], at[1], at[2]);
-      Dv[d] = __ldcg(D + l);
-      Iv[d] = ie[l];
-      if (sp.self_mode != 0 && sizeof(T) == 8) I64[d] = ie64[l];
-    }
+      for (int d = 0; d < 3; ++d)
+        I64[d] = ie64[(unsigned)d * (unsigned)m.V + corner_vertex(cs, d, a1, a2)];
     itk[k] = T(0);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const int e1 = (d + 1) % 3, e2 = (d + 2) % 3;
       const T w = ((T)wgt(f[e1], a1) / (T)kS) * ((T)wgt(f[e2], a2) / (T)kS);
-      Ek[k][d] = Dv[d] * Iv[d] * w;
-      const T iv = sizeof(T) == 8 ? (T)I64[d] : Iv[d];
+      Ek[k][d] = Dv[k][d] * Iv[k][d] * w;
+      const T iv = sizeof(T) == 8 ? (T)I64[d] : Iv[k][d];
       itk[k] += iv;
       iwk[k][d] = iv * w;
     }
@@ -1127,6 +1171,7 @@ __device__ inline int64_t batch_local(const RepDesc& r) {
 __global__ void __launch_bounds__(kBatchQuadThreads)
     k_deposit_batch(const RepDesc* __restrict__ desc, const int* __restrict__ cta_rep, int thermo,
                     double gamma, double kT) {
+  let_next_start();
   const RepDesc& r = desc[cta_rep[blockIdx.x]];
   cta_dipole_add(r.ds->Pacc,
                  deposit_body(r.m, r.sp, r.P, (unsigned long long*)r.Tb, r.ds, batch_local(r)));
@@ -1165,12 +1210,12 @@ __device__ inline int64_t batch_local_w(const RepDesc& r) {
   return (int64_t)(blockIdx.x - r.pw_first) * blockDim.x + threadIdx.x;
 }
 
-// Seven CTAs an SM (at most 72 registers, a few words spilled to L1) hold
-// a 64-replica batch's ~1000 CTAs in one wave; at the 88 registers the
-// kernel takes unbounded, five fit and a second wave trails (42.4 -> 38.5 us
-// a launch on 124k charges).
+// Seven CTAs an SM (at most 72 registers) hold a 64-replica batch's ~1000
+// CTAs in one wave; five and a trailing second wave took 42.4 us a launch for
+// 38.5 on 124k charges beside the field pass (now ahead of it: 25).
 __global__ void __launch_bounds__(kWideThreads, 7)
     k_deposit_batch_wide(const RepDesc* __restrict__ desc, const int* __restrict__ cta_rep) {
+  let_next_start();
   const RepDesc& r = desc[cta_rep[blockIdx.x]];
   long long U[3];
   deposit_wide(r.m, r.sp, r.P, (unsigned long long*)r.Tb, r.ds, batch_local_w(r), U);
@@ -1553,7 +1598,7 @@ struct HeldCharge {
   int img, q, c, f;     // own axis: image counter, cell, sub-cell step (c, f of the present x)
   int c0;               // cell before the last move
   int C[3], W[3];       // the quad's cells and sub-cell steps after the move
-  int64_t link[3];      // the lane's corner: field index of its three links
+  unsigned link[3];     // the lane's corner: field index of its three links
   T wie[3];             // their 1/eps and weight
   T w[3];
   T self;               // self-energy force of the own component
@@ -1591,7 +1636,7 @@ struct HeldCharge {
     if (own) {
       v = __dadd_rn(v, __dmul_rn(h, Ft));
       const double step = __dmul_rn(sp.dt, v);
-      if (fabs(step) <= 2.0 * m.a) {
+      if (short_step(m, step)) {
         xn = __dadd_rn(x, step);
         fold(m.L[d], xn, kn);
       } else {
@@ -1622,7 +1667,7 @@ struct HeldCharge {
           cc[e] = (e < d) ? C1[e] : C0[e];
           cf[e] = (e < d) ? F1[e] : F0[e];
         }
-        deposit_axis(m, d, q, c, f, f1, dc, cc, cf, Tb, V);
+        deposit_axis(m, d, q, c, f, f1, dc, cc, cf, Tb, (unsigned)V);
         x = xn;
         img = kn;
         c = c1;
@@ -1649,13 +1694,10 @@ struct HeldCharge {
     }
     if (active) {
       T iv[3];
+      const CellShares cs = cell_shares(m, C);
 #pragma unroll
       for (int e = 0; e < 3; ++e) {
-        const int e1 = (e + 1) % 3, e2 = (e + 2) % 3;
-        int at[3] = {C[0], C[1], C[2]};
-        at[e1] += a1;
-        at[e2] += a2;
-        link[e] = (int64_t)e * m.V + link_vertex(m, at[0], at[1], at[2]);
+        link[e] = (unsigned)e * (unsigned)m.V + corner_vertex(cs, e, a1, a2);
         wie[e] = ie[link[e]];
         iv[e] = sizeof(T) == 8 && sp.self_mode != 0 ? (T)ie64[link[e]] : wie[e];
       }

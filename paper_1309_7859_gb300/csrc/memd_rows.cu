@@ -59,6 +59,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : 2) k_rows_batch(const __gr
                         (T*)r.D[a.par ^ 1], (T*)r.B[a.par ^ 1], (T)r.sp.coefB, (T)r.sp.coefD,
                         g.y0, g.rows, g.za, g.zb, sE, sB, stg);
   }
+  wait_for_previous();
 }
 
 // the kernel's dynamic shared memory exceeds the 48 KB default: raise its
@@ -73,11 +74,10 @@ cudaError_t rows_attr() {
 }
 
 template <typename T, int NT>
-cudaError_t rows_launch(const RowsArgs& a, int nctas, cudaStream_t st) {
+cudaError_t rows_launch(const RowsArgs& a, int nctas, cudaStream_t st, bool early) {
   const cudaError_t e = rows_attr<T, NT>();
   if (e != cudaSuccess) return e;
-  k_rows_batch<T, NT><<<nctas, NT, rows_smem_bytes(NT, sizeof(T)), st>>>(a);
-  return cudaGetLastError();
+  return launch_early(k_rows_batch<T, NT>, nctas, NT, rows_smem_bytes(NT, sizeof(T)), st, early, a);
 }
 
 template <typename T, int NT>
@@ -112,14 +112,15 @@ int rows_occupancy(int prec, int nt) {
 }
 
 cudaError_t launch_rows_batch(int prec, const RepDesc* desc, const RowSeg* segs,
-                              const int* seg_first, int nctas, int nt, int par, cudaStream_t st) {
+                              const int* seg_first, int nctas, int nt, int par, cudaStream_t st,
+                              bool early) {
   if (nctas <= 0) return cudaSuccess;
   const RowsArgs a{desc, segs, seg_first, par};
   if (nt == kRowsWide)
-    return prec == 1 ? rows_launch<float, kRowsWide>(a, nctas, st)
-                     : rows_launch<double, kRowsWide>(a, nctas, st);
-  if (prec == 1) return nt == 256 ? rows_launch<float, 256>(a, nctas, st) : rows_launch<float, 512>(a, nctas, st);
-  return nt == 256 ? rows_launch<double, 256>(a, nctas, st) : rows_launch<double, 512>(a, nctas, st);
+    return prec == 1 ? rows_launch<float, kRowsWide>(a, nctas, st, early)
+                     : rows_launch<double, kRowsWide>(a, nctas, st, early);
+  if (prec == 1) return nt == 256 ? rows_launch<float, 256>(a, nctas, st, early) : rows_launch<float, 512>(a, nctas, st, early);
+  return nt == 256 ? rows_launch<double, 256>(a, nctas, st, early) : rows_launch<double, 512>(a, nctas, st, early);
 }
 
 // cost model of the row plan (measured on 64 mixed replicas): a tile-plane
