@@ -171,16 +171,12 @@ void drop_graphs(memd_ctx* c) {
       cudaGraphExecDestroy(c->graph[t]);
       c->graph[t] = nullptr;
     }
-    if (c->run_graph[t]) {
-      cudaGraphExecDestroy(c->run_graph[t]);
-      c->run_graph[t] = nullptr;
-    }
     if (c->io_graph[t]) {
       cudaGraphExecDestroy(c->io_graph[t]);
       c->io_graph[t] = nullptr;
     }
   }
-  c->run_steps = 0;
+  drop_runs(c->run);
 }
 
 double* scal(memd_ctx* c) { return c->red + 4 * reduce_blocks(); }
@@ -433,6 +429,7 @@ static bool rows_setup(memd_ctx* c, int nt) {
   return true;
 }
 
+// early: of the row kernel only
 static void launch_field(memd_ctx* c, int par, double cB, double cD, FusedCfg cfg,
                          bool early = false) {
   if (cfg.rows)
@@ -443,7 +440,7 @@ static void launch_field(memd_ctx* c, int par, double cB, double cD, FusedCfg cf
                      c->Dbuf[par ^ 1], c->Bbuf[par ^ 1], cB, cD, cfg, &c->ds->err, c->stream);
   else
     launch_fused_curl(c->mesh, c->prec, c->Dbuf[par], c->Bbuf[par], c->ie, c->Dbuf[par ^ 1],
-                      c->Bbuf[par ^ 1], cB, cD, cfg, c->stream, early);
+                      c->Bbuf[par ^ 1], cB, cD, cfg, c->stream);
 }
 
 // ------------------------------------------------------------------ autotuner
@@ -643,8 +640,6 @@ void memd_destroy(memd_ctx* c) {
   if (c->ev0) cudaEventDestroy(c->ev0);
   if (c->ev1) cudaEventDestroy(c->ev1);
   if (c->fork) cudaEventDestroy(c->fork);
-  if (c->join) cudaEventDestroy(c->join);
-  if (c->side) cudaStreamDestroy(c->side);
   if (c->err_host) cudaFreeHost(c->err_host);
   if (c->io_host) cudaFreeHost(c->io_host);
   while (!c->blocks.empty()) dfree(c, c->blocks.back().first);
@@ -936,9 +931,7 @@ memd_status memd_create(const int32_t mesh[3], const double box[3], const memd_e
     if (s != MEMD_OK) goto done;
   }
   if (cudaEventCreate(&c->ev0) != cudaSuccess || cudaEventCreate(&c->ev1) != cudaSuccess ||
-      cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&c->join, cudaEventDisableTiming) != cudaSuccess ||
-      cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking) != cudaSuccess) {
+      cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming) != cudaSuccess) {
     s = fail(c, MEMD_ERR_CUDA, "events");
     goto done;
   }
@@ -1106,11 +1099,13 @@ memd_status memd_init_field(memd_ctx* c, int64_t n, const double* pos, const int
 // The charge transfer of the drift runs beside the fused field update
 // (neither reads what the other writes; with timing on, after it); the
 // transfers are applied to the new D, then the gather closes the step.  The
-// field update is launched early behind the transfer, so the transfer always
-// takes its SMs first: as two roots of a graph they started in either order,
-// and 32768 charges on 64^3 took 7.4 us when first, 13-17 us piled up on the
-// first SMs that the field pass left when second (the two together 11.5
-// against 13-17).
+// second of the two is launched early behind the first, so that they take
+// their SMs in a known order: as two roots of a graph they started in either
+// one, and the transfer of 32768 charges on 64^3 took 7.4 us ahead of the row
+// kernel, 13-17 us piled up on the first SMs that it left when behind (the
+// two together 11.5 against 13-17).  Inside a run (first, last: this step's
+// place in it) the gather waits for the next step's transfer, one kernel with
+// it.
 // a timing event inside a captured graph is an external event node; outside
 // capture it is recorded as usual
 static cudaError_t record_timing_event(cudaEvent_t ev, cudaStream_t st) {
@@ -1120,34 +1115,42 @@ static cudaError_t record_timing_event(cudaEvent_t ev, cudaStream_t st) {
                                              : cudaEventRecord(ev, st);
 }
 
-static memd_status record_step(memd_ctx* c, const StepParams& sp, int par, bool timed) {
+static memd_status record_step(memd_ctx* c, const StepParams& sp, int par, bool timed,
+                               bool first = true, bool last = true) {
   const Mesh& m = c->mesh;
   const cudaStream_t st = c->stream;
-  // the TMA kernel leaves early on an expired wait, so it does not end behind
-  // the deposition; without charges nothing stands between two field passes
-  const bool early = (c->fcfg.rows || !c->fcfg.tma) && c->P.n > 0;
+  const bool early = !timed && c->P.n > 0;
+  // the charge transfer, in a run behind the gather of the step before, whose
+  // D is this step's
+  auto transfer = [&](bool behind_field) {
+    if (first || !early)
+      launch_kick_drift_deposit(m, sp, c->P, c->Tb, c->ds, st, behind_field);
+    else
+      launch_turn(m, c->prec, sp, c->P, c->Tb, c->Dbuf[par], c->ie, c->ie64, c->ds, st,
+                  behind_field);
+  };
   if (timed) {
     // instrumented: the field update alone between its event pair
     CK(record_timing_event(c->ev0, st));
     launch_field(c, par, sp.coefB, sp.coefD, c->fcfg);
     CK(record_timing_event(c->ev1, st));
-    launch_kick_drift_deposit(m, sp, c->P, c->Tb, c->ds, st);
-  } else if (early) {
-    launch_kick_drift_deposit(m, sp, c->P, c->Tb, c->ds, st);
+    transfer(false);
+  } else if (early && c->fcfg.rows) {
+    transfer(false);
     launch_field(c, par, sp.coefB, sp.coefD, c->fcfg, true);
   } else {
-    CK(cudaEventRecord(c->fork, st));
-    CK(cudaStreamWaitEvent(c->side, c->fork, 0));
-    launch_kick_drift_deposit(m, sp, c->P, c->Tb, c->ds, c->side);
-    CK(cudaEventRecord(c->join, c->side));
     launch_field(c, par, sp.coefB, sp.coefD, c->fcfg);
-    CK(cudaStreamWaitEvent(st, c->join, 0));
+    CK(cudaEventRecord(c->fork, st));
+    transfer(early);
+    CK(cudaStreamWaitEvent(st, c->fork, 0));
   }
+  const int turn = early ? (first ? 0 : kTurnCount) | (last ? 0 : kTurnClose) : 0;
   if (apply_dense(c->apply_mode))
-    launch_apply_dense(c->prec, 3 * m.V, c->Tb, c->Lg, c->Dbuf[par ^ 1], sp.scale, st);
+    launch_apply_dense(c->prec, 3 * m.V, c->Tb, c->Lg, c->Dbuf[par ^ 1], sp.scale, st, c->ds, turn);
   else
-    launch_apply(m, c->prec, c->P, c->Tb, c->Lg, c->Dbuf[par ^ 1], sp.scale, st);
-  launch_gather(m, c->prec, sp, c->P, c->Dbuf[par ^ 1], c->ie, c->ie64, c->ds, 1, 2, st);
+    launch_apply(m, c->prec, c->P, c->Tb, c->Lg, c->Dbuf[par ^ 1], sp.scale, st, 0, c->ds, turn);
+  if (last || !early)
+    launch_gather(m, c->prec, sp, c->P, c->Dbuf[par ^ 1], c->ie, c->ie64, c->ds, 1, 2, st);
   CKL();
   return MEMD_OK;
 }
@@ -1237,8 +1240,7 @@ static memd_status step_prepare(memd_ctx* c, const memd_thermostat* th, StepPara
     c->graph_gamma = gamma;
     c->graph_kT = kT;
   }
-  if (!c->graph[0] && !c->graph[1] && !c->run_graph[0] && !c->run_graph[1])
-    c->coop = want_coop(c);
+  if (!c->graph[0] && !c->graph[1] && !c->run.any) c->coop = want_coop(c);
   if (c->coop && !c->Tb2) {
     // the single-launch step's transfer slots (3 V words each)
     c->Tb2 = (long long*)dalloc(c, kCoopSlots * 3 * c->mesh.V * sizeof(long long));
@@ -1283,24 +1285,22 @@ memd_status memd_step(memd_ctx* c, int64_t nsteps, const memd_thermostat* th) {
     }
     return poll_err(c, false);
   }
+  int64_t single = 0;
   for (int64_t s = 0; s < nsteps;) {
     const int par = c->cur;
     harvest_timing(c);
-    const int k = c->use_graphs && !timed && nsteps - s >= kRunSteps &&
-                          (c->run_graph[par] || c->run_steps + nsteps - s >= kRunAfter)
-                      ? kRunSteps
-                      : 1;
+    const int k = c->use_graphs && !timed ? run_length(c->run, par, nsteps - s, &single) : 1;
     if (!c->use_graphs) {
       const memd_status r = record_step(c, sp, par, timed);
       if (r != MEMD_OK) return r;
     } else {
-      cudaGraphExec_t& gx = k > 1 ? c->run_graph[par] : c->graph[par];
+      cudaGraphExec_t& gx = k > 1 ? c->run.graph[par][k] : c->graph[par];
       if (!gx) {
         cudaGraph_t g = nullptr;
         CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
         memd_status r = MEMD_OK;
         for (int j = 0; j < k && r == MEMD_OK; ++j)
-          r = record_step(c, sp, par ^ (j & 1), timed);
+          r = record_step(c, sp, par ^ (j & 1), timed, j == 0, j == k - 1);
         const cudaError_t e = cudaStreamEndCapture(c->stream, &g);
         cudaError_t ie = cudaErrorUnknown;
         if (r == MEMD_OK && e == cudaSuccess) ie = cudaGraphInstantiate(&gx, g, 0);
@@ -1317,7 +1317,6 @@ memd_status memd_step(memd_ctx* c, int64_t nsteps, const memd_thermostat* th) {
     }
     c->timing_pending = timed;
     c->cur = par ^ (k & 1);
-    c->run_steps += k;
     s += k;
   }
   return poll_err(c, false);

@@ -4,9 +4,10 @@
 // parameters, field and particle pointers) and two CTA->replica maps, one
 // for the field tiles and one for the particle quads.  Each time step is one
 // CUDA graph of four launches covering every member: the charge transfer of
-// the drift on a side stream beside the fused field update, then the
-// transfer application, then the force gather, which also closes each
-// replica's step.  Small systems that would each leave most SMs idle fill
+// the drift beside the fused field update, then the transfer application,
+// then the force gather, which also closes each replica's step.  Calls of
+// several steps run up to sixteen as one graph, a step's gather and the next
+// one's charge transfer as one launch.  Small systems that would each leave most SMs idle fill
 // the GPU together, and the per-step launch cost is paid once for all.
 #include <algorithm>
 #include <cstring>
@@ -53,8 +54,7 @@ struct memd_batch {
   int2* d_apply_chunk = nullptr;
   int n_apply_chunk = 0;
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
-  cudaGraphExec_t run_graph[2] = {nullptr, nullptr};  // kRunSteps steps
-  int64_t run_steps = 0;  // steps since the step graphs were dropped
+  StepRuns run;
   // single-launch step (k_batch_step): the engine asked for, whether it runs,
   // its grid, the CTAs that start with field work, planes per field item, the
   // four work queues and the scheduling state
@@ -112,17 +112,12 @@ void drop(memd_batch* b) {
       cudaGraphExecDestroy(g);
       g = nullptr;
     }
-  for (cudaGraphExec_t& g : b->run_graph)
-    if (g) {
-      cudaGraphExecDestroy(g);
-      g = nullptr;
-    }
   for (cudaGraphExec_t& g : b->io_graph)
     if (g) {
       cudaGraphExecDestroy(g);
       g = nullptr;
     }
-  b->run_steps = 0;
+  drop_runs(b->run);
 }
 
 void* balloc(memd_batch* b, size_t bytes) {
@@ -377,12 +372,13 @@ memd_status build_tables(memd_batch* b, bool sync = true) {
 }
 
 // the batch's field update: row kernel or site tiles
+// (early: of the row kernel only)
 cudaError_t launch_field(memd_batch* b, int par, cudaStream_t st, bool early = false) {
   if (b->f_rows > 0)
     return launch_rows_batch(b->prec, b->d_desc, b->d_segs, b->d_seg_first, b->n_rows_ctas,
                              b->f_rows, par, st, early);
   launch_fused_batch(b->prec, b->d_desc, b->d_field_rep, b->n_field, par, b->f_ty, b->f_pf,
-                     b->f_w, st, early);
+                     b->f_w, st);
   return cudaGetLastError();
 }
 
@@ -506,19 +502,33 @@ cudaError_t gather_batch(memd_batch* b, int par, int thermo, double gamma, doubl
 }
 
 // the kick, drift and charge transfer of every replica
-void deposit_batch(memd_batch* b, int thermo, double gamma, double kT, cudaStream_t s) {
+void deposit_batch(memd_batch* b, int thermo, double gamma, double kT, cudaStream_t s,
+                   bool early = false) {
   if (b->wide)
-    launch_deposit_batch_wide(b->d_desc, b->d_part_rep_w, b->n_part_w, s);
+    launch_deposit_batch_wide(b->d_desc, b->d_part_rep_w, b->n_part_w, s, early);
   else
-    launch_deposit_batch(b->d_desc, b->d_part_rep, b->n_part, thermo, gamma, kT, s);
+    launch_deposit_batch(b->d_desc, b->d_part_rep, b->n_part, thermo, gamma, kT, s, early);
+}
+
+// the gather of the step before (which wrote the D of parity par) with the
+// kick, drift and charge transfer of this one
+void turn_batch(memd_batch* b, int par, int thermo, double gamma, double kT, cudaStream_t s,
+                bool early) {
+  if (b->wide)
+    launch_turn_batch_wide(b->prec, b->d_desc, b->d_part_rep_w, b->n_part_w, par ^ 1, thermo, s,
+                           early);
+  else
+    launch_turn_batch(b->prec, b->d_desc, b->d_part_rep, b->n_part, par ^ 1, thermo, gamma, kT, s,
+                      early);
 }
 
 // the step's transfers into the ledgers and the new D of every replica
-void apply_batch(memd_batch* b, int par, cudaStream_t s) {
+void apply_batch(memd_batch* b, int par, cudaStream_t s, int turn = 0) {
   if (b->apply_dense)
-    launch_apply_dense_batch(b->prec, b->d_desc, b->d_apply_chunk, b->n_apply_chunk, par, s);
+    launch_apply_dense_batch(b->prec, b->d_desc, b->d_apply_chunk, b->n_apply_chunk, par, s,
+                             turn);
   else
-    launch_apply_batch(b->prec, b->d_desc, b->d_part_rep, b->n_part, par, s);
+    launch_apply_batch(b->prec, b->d_desc, b->d_part_rep, b->n_part, par, s, turn);
 }
 
 bool batch_timed(const memd_batch* b) {
@@ -539,7 +549,8 @@ void set_thermostat(memd_batch* b, int thermo, double gamma, double kT) {
   b->g_kT = kT;
 }
 
-memd_status record(memd_batch* b, int par, int thermo, double gamma, double kT, bool timed) {
+memd_status record(memd_batch* b, int par, int thermo, double gamma, double kT, bool timed,
+                   bool first = true, bool last = true) {
   const cudaStream_t st = b->stream;
   if (b->single) {
     // the whole step in one cooperative launch; with timing on, the event
@@ -591,23 +602,31 @@ memd_status record(memd_batch* b, int par, int thermo, double gamma, double kT, 
   // writes): it is latency bound, the pass bandwidth bound, and the pass's
   // evict_first accesses leave the deposition's evict_last transfer words in
   // L2 for the application (64 replicas: 113.9 -> 109.8 us a step against
-  // the two in turn).  The pass is launched early behind the deposition: as
-  // two roots of a graph they started in either order, and a deposition that
-  // finds the SMs full of the pass's CTAs ends late, piled up on the first
-  // SMs that drain.  Moving the gather that closes a step beside the next
-  // field pass, ahead of the deposition, was slower (116.9 us): the two
-  // particle kernels in turn then outlast the pass.  Without overlap (the
-  // request server, whose admission work runs on other streams meanwhile)
-  // the two run in turn.
-  if (b->overlap && (b->wide ? b->n_part_w : b->n_part) > 0) {
-    deposit(st);
+  // the two in turn).  The second of the two is launched early behind the
+  // first; as two roots of a graph they started in either order.  Inside a
+  // run the gather of the step before and the deposition are one kernel:
+  // 24 + 25 us a step on their own, 45 together, of which the row kernel now
+  // hides 21 instead of 8 (64 replicas, 10 steps: 1234 -> 1166 us).  Without
+  // overlap (the request server, whose admission work runs on other streams
+  // meanwhile) field pass, deposition and gather run in turn.
+  const bool early = b->overlap && (b->wide ? b->n_part_w : b->n_part) > 0;
+  auto transfer = [&](bool behind_field) {
+    if (first || !early)
+      deposit_batch(b, thermo, gamma, kT, st, behind_field);
+    else
+      turn_batch(b, par, thermo, gamma, kT, st, behind_field);
+  };
+  if (early && b->f_rows > 0) {
+    transfer(false);
     BCK(launch_field(b, par, st, true));
   } else {
     BCK(launch_field(b, par, st));
-    deposit(st);
+    BCK(cudaEventRecord(b->fork, st));
+    transfer(early);
+    BCK(cudaStreamWaitEvent(st, b->fork, 0));
   }
-  apply(st);
-  BCK(gather_batch(b, par, thermo, gamma, kT, st));
+  apply_batch(b, par, st, early ? (first ? 0 : kTurnCount) | (last ? 0 : kTurnClose) : 0);
+  if (last || !early) BCK(gather_batch(b, par, thermo, gamma, kT, st));
   BCK(cudaGetLastError());
   return MEMD_OK;
 }
@@ -856,13 +875,11 @@ memd_status memd_batch_step(memd_batch* b, int64_t nsteps, const memd_thermostat
   const double gamma = th ? th->gamma : 0.0, kT = th ? th->kT : 0.0;
   set_thermostat(b, thermo, gamma, kT);
   const bool timed = batch_timed(b);
+  int64_t single = 0;
   for (int64_t s = 0; s < nsteps;) {
     const int par = b->bpar;
     harvest(b);
-    const int k = !b->single && !timed && nsteps - s >= kRunSteps &&
-                          (b->run_graph[par] || b->run_steps + nsteps - s >= kRunAfter)
-                      ? kRunSteps
-                      : 1;
+    const int k = !b->single && !timed ? run_length(b->run, par, nsteps - s, &single) : 1;
     if (b->single && !b->single_graph_ok) {
       // the cooperative launch could not be captured here: launched directly
       const memd_status r = record(b, par, thermo, gamma, kT, timed);
@@ -872,13 +889,13 @@ memd_status memd_batch_step(memd_batch* b, int64_t nsteps, const memd_thermostat
       ++s;
       continue;
     }
-    cudaGraphExec_t& gx = k > 1 ? b->run_graph[par] : b->graph[par];
+    cudaGraphExec_t& gx = k > 1 ? b->run.graph[par][k] : b->graph[par];
     if (!gx) {
       cudaGraph_t g = nullptr;
       BCK(cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
       memd_status r = MEMD_OK;
       for (int j = 0; j < k && r == MEMD_OK; ++j)
-        r = record(b, par ^ (j & 1), thermo, gamma, kT, timed);
+        r = record(b, par ^ (j & 1), thermo, gamma, kT, timed, j == 0, j == k - 1);
       cudaError_t e = cudaStreamEndCapture(b->stream, &g);
       if (r != MEMD_OK) {
         if (g) cudaGraphDestroy(g);
@@ -897,7 +914,6 @@ memd_status memd_batch_step(memd_batch* b, int64_t nsteps, const memd_thermostat
     BCK(cudaGraphLaunch(gx, b->stream));
     b->timing_pending = timed;
     b->bpar ^= k & 1;
-    b->run_steps += k;
     s += k;
   }
   for (size_t r = 0; r < b->m.size(); ++r) b->m[r]->cur = (b->base[r] + b->bpar) & 1;

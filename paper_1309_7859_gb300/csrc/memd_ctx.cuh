@@ -68,8 +68,7 @@ struct memd_ctx {
   int rows_nt = 0;       // a permittivity is mapped (memd_set_eps restores it on failure)
   // step graphs, one per buffer parity
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
-  cudaGraphExec_t run_graph[2] = {nullptr, nullptr};  // kRunSteps steps
-  int64_t run_steps = 0;  // steps since the step graphs were dropped
+  memd::StepRuns run;
   // memd_step_io's whole round trip (copy in, unpack, step, pack, copy out)
   // as one graph per buffer parity; io_graph_ok false once capture failed
   cudaGraphExec_t io_graph[2] = {nullptr, nullptr};
@@ -80,8 +79,7 @@ struct memd_ctx {
   bool coop = false;     // the steps run as one cooperative launch
   int graph_thermo = -1;
   double graph_gamma = 0, graph_kT = 0;
-  cudaStream_t side = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr;
+  cudaEvent_t fork = nullptr;
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   bool timing_pending = false;
   double field_ms = 0;

@@ -327,9 +327,9 @@ __global__ void __launch_bounds__(34 * (TY + 2))
     k_fused_site(Mesh m, const T* __restrict__ Din, const T* __restrict__ Bin,
                  const T* __restrict__ ie, T* __restrict__ Dout, T* __restrict__ Bout, T cB,
                  T cD, int zchunk) {
+  let_next_start();
   site_tile<T, TY, PF>(m, Din, Bin, ie, Dout, Bout, cB, cD, blockIdx.x, blockIdx.y, blockIdx.z,
                        zchunk, threadIdx.x, threadIdx.y, true, CtaSync{});
-  wait_for_previous();
 }
 
 // Many independent systems in one launch: CTA b works on a site tile of
@@ -337,6 +337,7 @@ __global__ void __launch_bounds__(34 * (TY + 2))
 template <typename T, int TY, int PF, int TX>
 __global__ void __launch_bounds__((TX + 2) * (TY + 2))
     k_fused_site_batch(const RepDesc* __restrict__ desc, const int* __restrict__ cta_rep, int par) {
+  let_next_start();
   const RepDesc& r = desc[cta_rep[blockIdx.x]];
   const int local = blockIdx.x - r.f_first;
   const int per_z = r.f_tx * r.f_ty;
@@ -346,7 +347,6 @@ __global__ void __launch_bounds__((TX + 2) * (TY + 2))
                                     (T*)r.D[par ^ 1], (T*)r.B[par ^ 1], (T)r.sp.coefB,
                                     (T)r.sp.coefD, tx, ty, tz, r.f_zchunk, threadIdx.x,
                                     threadIdx.y, true, CtaSync{});
-  wait_for_previous();
 }
 
 template <typename T, int TX, int TY>
@@ -354,9 +354,9 @@ __global__ void __launch_bounds__(TX* TY)
     k_fused_curl(Mesh m, const T* __restrict__ Din, const T* __restrict__ Bin,
                  const T* __restrict__ ie, T* __restrict__ Dout, T* __restrict__ Bout, T cB,
                  T cD, int zchunk) {
+  let_next_start();
   fused_tile<T, TX, TY>(m, Din, Bin, ie, Dout, Bout, cB, cD, blockIdx.x, blockIdx.y, blockIdx.z,
                         zchunk);
-  wait_for_previous();
 }
 
 
@@ -605,69 +605,66 @@ void launch_curl_D(const Mesh& m, int prec, void* D, const void* B, double coef,
 namespace {
 template <typename T, int TY>
 void fused_launch_t(const Mesh& m, const void* Din, const void* Bin, const void* ie, void* Dout,
-                    void* Bout, double cB, double cD, int zchunk, cudaStream_t st,
-                   bool early) {
+                    void* Bout, double cB, double cD, int zchunk, cudaStream_t st) {
   constexpr int TX = 32;
   const dim3 grid((m.n[0] + TX - 1) / TX, (m.n[1] + TY - 1) / TY, (m.n[2] + zchunk - 1) / zchunk);
-  launch_early(k_fused_curl<T, TX, TY>, grid, dim3(TX, TY, 1), 0, st, early, m, (const T*)Din,
-               (const T*)Bin, (const T*)ie, (T*)Dout, (T*)Bout, (T)cB, (T)cD, zchunk);
+  k_fused_curl<T, TX, TY><<<grid, dim3(TX, TY, 1), 0, st>>>(
+      m, (const T*)Din, (const T*)Bin, (const T*)ie, (T*)Dout, (T*)Bout, (T)cB, (T)cD, zchunk);
 }
 }  // namespace
 
 namespace {
 template <typename T, int TY, int PF>
 void site_launch_t(const Mesh& m, const void* Din, const void* Bin, const void* ie, void* Dout,
-                   void* Bout, double cB, double cD, int zchunk, cudaStream_t st,
-                   bool early) {
+                   void* Bout, double cB, double cD, int zchunk, cudaStream_t st) {
   const dim3 grid((m.n[0] + 31) / 32, (m.n[1] + TY - 1) / TY, (m.n[2] + zchunk - 1) / zchunk);
-  launch_early(k_fused_site<T, TY, PF>, grid, dim3(34, TY + 2, 1), 0, st, early, m,
-               (const T*)Din, (const T*)Bin, (const T*)ie, (T*)Dout, (T*)Bout, (T)cB, (T)cD, zchunk);
+  k_fused_site<T, TY, PF><<<grid, dim3(34, TY + 2, 1), 0, st>>>(
+      m, (const T*)Din, (const T*)Bin, (const T*)ie, (T*)Dout, (T*)Bout, (T)cB, (T)cD, zchunk);
 }
 template <typename T, int TY>
 void site_launch_pf(int pf, const Mesh& m, const void* Din, const void* Bin, const void* ie,
-                    void* Dout, void* Bout, double cB, double cD, int zchunk, cudaStream_t st,
-                   bool early) {
+                    void* Dout, void* Bout, double cB, double cD, int zchunk, cudaStream_t st) {
   if (pf >= 2)
-    site_launch_t<T, TY, 2>(m, Din, Bin, ie, Dout, Bout, cB, cD, zchunk, st, early);
+    site_launch_t<T, TY, 2>(m, Din, Bin, ie, Dout, Bout, cB, cD, zchunk, st);
   else
-    site_launch_t<T, TY, 1>(m, Din, Bin, ie, Dout, Bout, cB, cD, zchunk, st, early);
+    site_launch_t<T, TY, 1>(m, Din, Bin, ie, Dout, Bout, cB, cD, zchunk, st);
 }
 }  // namespace
 
 void launch_fused_curl(const Mesh& m, int prec, const void* Din, const void* Bin, const void* ie,
                        void* Dout, void* Bout, double cB, double cD, FusedCfg cfg,
-                       cudaStream_t st, bool early) {
+                       cudaStream_t st) {
   if (cfg.zchunk < 1) cfg = fused_default(m);
   if (cfg.zchunk > m.n[2]) cfg.zchunk = m.n[2];
   if (cfg.site) {
     const int pf = cfg.site;
     if (prec == 1) {
       if (cfg.ty == 4)
-        site_launch_pf<float, 4>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
+        site_launch_pf<float, 4>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
       else if (cfg.ty == 16)
-        site_launch_pf<float, 16>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
+        site_launch_pf<float, 16>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
       else
-        site_launch_pf<float, 8>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
+        site_launch_pf<float, 8>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
     } else {
       if (cfg.ty == 4)
-        site_launch_pf<double, 4>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
+        site_launch_pf<double, 4>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
       else
-        site_launch_pf<double, 8>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
+        site_launch_pf<double, 8>(pf, m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
     }
     return;
   }
   if (prec == 1) {
     switch (cfg.ty) {
-      case 4: fused_launch_t<float, 4>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early); break;
-      case 16: fused_launch_t<float, 16>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early); break;
-      default: fused_launch_t<float, 8>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
+      case 4: fused_launch_t<float, 4>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st); break;
+      case 16: fused_launch_t<float, 16>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st); break;
+      default: fused_launch_t<float, 8>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
     }
   } else {
     // FP64 tiles stop at 8 rows: 16 would exceed the 48 KB of static shared memory
     if (cfg.ty == 4)
-      fused_launch_t<double, 4>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
+      fused_launch_t<double, 4>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
     else
-      fused_launch_t<double, 8>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st, early);
+      fused_launch_t<double, 8>(m, Din, Bin, ie, Dout, Bout, cB, cD, cfg.zchunk, st);
   }
 }
 
@@ -688,43 +685,41 @@ FusedCfg fused_default(const Mesh& m) {
 namespace {
 template <typename T, int TY, int PF>
 void batch_launch_t(const RepDesc* desc, const int* cta_rep, int nctas, int par, int tw,
-                    cudaStream_t st, bool early) {
+                    cudaStream_t st) {
   if (tw == 16)
-    launch_early(k_fused_site_batch<T, TY, PF, 16>, nctas, dim3(18, TY + 2, 1), 0, st, early, desc,
-                 cta_rep, par);
+    k_fused_site_batch<T, TY, PF, 16><<<nctas, dim3(18, TY + 2, 1), 0, st>>>(desc, cta_rep, par);
   else
-    launch_early(k_fused_site_batch<T, TY, PF, 32>, nctas, dim3(34, TY + 2, 1), 0, st, early, desc,
-                 cta_rep, par);
+    k_fused_site_batch<T, TY, PF, 32><<<nctas, dim3(34, TY + 2, 1), 0, st>>>(desc, cta_rep, par);
 }
 template <typename T>
 void batch_launch_ty(const RepDesc* desc, const int* cta_rep, int nctas, int par, int ty, int pf,
-                     int tw, cudaStream_t st, bool early) {
+                     int tw, cudaStream_t st) {
   if (ty == 4) {
     if (pf >= 2)
-      batch_launch_t<T, 4, 2>(desc, cta_rep, nctas, par, tw, st, early);
+      batch_launch_t<T, 4, 2>(desc, cta_rep, nctas, par, tw, st);
     else
-      batch_launch_t<T, 4, 1>(desc, cta_rep, nctas, par, tw, st, early);
+      batch_launch_t<T, 4, 1>(desc, cta_rep, nctas, par, tw, st);
   } else if (ty == 16 && sizeof(T) == 4) {
     if (pf >= 2)
-      batch_launch_t<float, 16, 2>(desc, cta_rep, nctas, par, tw, st, early);
+      batch_launch_t<float, 16, 2>(desc, cta_rep, nctas, par, tw, st);
     else
-      batch_launch_t<float, 16, 1>(desc, cta_rep, nctas, par, tw, st, early);
+      batch_launch_t<float, 16, 1>(desc, cta_rep, nctas, par, tw, st);
   } else {
     if (pf >= 2)
-      batch_launch_t<T, 8, 2>(desc, cta_rep, nctas, par, tw, st, early);
+      batch_launch_t<T, 8, 2>(desc, cta_rep, nctas, par, tw, st);
     else
-      batch_launch_t<T, 8, 1>(desc, cta_rep, nctas, par, tw, st, early);
+      batch_launch_t<T, 8, 1>(desc, cta_rep, nctas, par, tw, st);
   }
 }
 }  // namespace
 
 void launch_fused_batch(int prec, const RepDesc* desc, const int* cta_rep, int nctas, int par,
-                        int ty, int pf, int tw, cudaStream_t st, bool early) {
+                        int ty, int pf, int tw, cudaStream_t st) {
   if (nctas <= 0) return;
   if (prec == 1)
-    batch_launch_ty<float>(desc, cta_rep, nctas, par, ty, pf, tw, st, early);
+    batch_launch_ty<float>(desc, cta_rep, nctas, par, ty, pf, tw, st);
   else
-    batch_launch_ty<double>(desc, cta_rep, nctas, par, ty, pf, tw, st, early);
+    batch_launch_ty<double>(desc, cta_rep, nctas, par, ty, pf, tw, st);
 }
 
 int fused_candidates(const Mesh& m, int prec, FusedCfg* out, int cap) {

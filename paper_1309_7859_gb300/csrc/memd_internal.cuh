@@ -130,22 +130,51 @@ __device__ __forceinline__ unsigned long long exch_hint(unsigned long long* a, u
   return r;
 }
 
-// Steps of the graph engine recorded as one graph: between two graph launches
-// the device idles 2.8-4.5 us, between two nodes about 1 (64^3 with 32768
-// charges 36.0 -> 33.1 us a step of a 20-step call).  Recorded once
-// a caller has asked for kRunAfter steps of the same set-up; shorter runs do
-// not repay the recording of eight steps.
-constexpr int kRunSteps = 8;
-constexpr int64_t kRunAfter = 32;
+// Runs: up to kRunSteps steps of the graph engine recorded as one graph, one
+// for each length and buffer parity asked for.  Inside a run a step's gather
+// and the next one's deposition are one kernel, beside the next field pass.
+// A length is recorded the third time a caller asks for it with the same
+// set-up: a shorter use does not repay the recording (0.1-0.4 ms).
+constexpr int kRunSteps = 16;
+struct StepRuns {
+  cudaGraphExec_t graph[2][kRunSteps + 1] = {};
+  int asked[kRunSteps + 1] = {};
+  bool any = false;
+};
+// steps of the next launch when `left` remain; `single` (0 before the first)
+// counts down the rest of a run that is not recorded yet
+inline int run_length(StepRuns& r, int par, int64_t left, int64_t* single) {
+  const int k = left < kRunSteps ? (int)left : kRunSteps;
+  if (*single > 0) {
+    --*single;
+    return 1;
+  }
+  if (k < 2) return 1;
+  if (r.graph[par][k] || r.asked[k]++ >= 2) {
+    r.any = true;
+    return k;
+  }
+  *single = k - 1;
+  return 1;
+}
+inline void drop_runs(StepRuns& r) {
+  for (auto& p : r.graph)
+    for (cudaGraphExec_t& g : p)
+      if (g) cudaGraphExecDestroy(g);
+  r = StepRuns{};
+}
 
 // Programmatic dependent launch.  A kernel launched early (launch_early with
 // early set) may start once every CTA of the kernel before it in its stream
 // has called let_next_start (or left); wait_for_previous then returns when
 // that kernel has completed and its writes are visible.  Without the early
-// launch both calls are no-ops.  The field kernels are the only ones launched
-// early, behind the charge transfer, whose data they do not touch: they wait
-// as their last statement, so that what follows them follows both.  (The
-// application and the gather are not: their CTAs, placed while the kernel
+// launch both calls are no-ops.  Used for a step's field pass and the
+// particle kernel beside it, neither of which touches what the other writes:
+// it fixes which of the two takes its SMs first.  The row kernel's CTAs fill
+// an SM, so the particle kernel goes first (64^3, 32768 charges, 20 steps:
+// 549 us for 670); the smaller tiles leave room for it and go first (95^3,
+// 20000 charges, 10 steps: 316-343 us for 410-424).  (The application and a
+// gather by itself are never early: their CTAs, placed while the kernel
 // before them still held SMs, piled up unevenly, and 256^3 with 100k charges
 // took 370 us a step for 300.)
 __device__ __forceinline__ void wait_for_previous() {
@@ -188,7 +217,7 @@ struct FusedCfg {
 };
 void launch_fused_curl(const Mesh& m, int prec, const void* Din, const void* Bin, const void* ie,
                        void* Dout, void* Bout, double cB, double cD, FusedCfg cfg,
-                       cudaStream_t st, bool early = false);
+                       cudaStream_t st);
 FusedCfg fused_default(const Mesh& m);
 // candidate shapes for the autotuner; returns how many were written
 int fused_candidates(const Mesh& m, int prec, FusedCfg* out, int cap);
@@ -382,16 +411,18 @@ void launch_cic(const Mesh& m, Particles p, long long* Q, long long bg, cudaStre
 void launch_cic_abs(const Mesh& m, Particles p, long long* Q, cudaStream_t st);
 void launch_dipole(const Mesh& m, Particles p, DevState* ds, cudaStream_t st);
 void launch_kick_drift_deposit(const Mesh& m, const StepParams& sp, Particles p,
-                               long long* Tb, DevState* ds, cudaStream_t st);
+                               long long* Tb, DevState* ds, cudaStream_t st,
+                               bool early = false);
 void launch_move_deposit(const Mesh& m, Particles p, const double* pos_new,
                          const int* img_new, long long* Tb, DevState* ds, cudaStream_t st);
 // cmV: the layout of Tb (tw_index); the ledger Lg is always the pairs'
 void launch_apply(const Mesh& m, int prec, Particles p, long long* Tb, long long* Lg, void* D,
-                  double scale, cudaStream_t st, int64_t cmV = 0);
+                  double scale, cudaStream_t st, int64_t cmV = 0, DevState* ds = nullptr,
+                  int turn = 0);
 // the same over every one of nlinks transfer words (one pass, no particle
 // data); identical results.  Cheaper when the mesh has few links per charge.
 void launch_apply_dense(int prec, int64_t nlinks, long long* Tb, long long* Lg, void* D,
-                        double scale, cudaStream_t st);
+                        double scale, cudaStream_t st, DevState* ds = nullptr, int turn = 0);
 // MEMD_APPLY_AUTO is the sparse pass.  A dense pass reads 24 B a vertex and
 // rewrites the words that carry a transfer; the sparse pass costs ~0.25-0.3 ns
 // a charge on GB300 (12 atomic round trips per quad, issued together).
@@ -406,6 +437,14 @@ void launch_gather(const Mesh& m, int prec, const StepParams& sp, Particles p, c
                    const void* ie, const double* ie64, DevState* ds, int kick, int finish,
                    cudaStream_t st);
 void launch_step_end(DevState* ds, int advance, cudaStream_t st);
+// in a run of steps: the gather of a step with the kick, drift and deposition
+// of the next; the application before it closes the step's dipole sum
+// (kTurnClose), and counts the step before its own when that one ended in a
+// turn (kTurnCount)
+constexpr int kTurnClose = 1, kTurnCount = 2;
+void launch_turn(const Mesh& m, int prec, const StepParams& sp, Particles p, long long* Tb,
+                 const void* D, const void* ie, const double* ie64, DevState* ds,
+                 cudaStream_t st, bool early = false);
 
 // ------------------------------------------------------- batched replicas
 // One independent system of a batch, as the batched kernels see it.
@@ -512,7 +551,7 @@ int batch_step_occupancy(int prec);
 cudaError_t launch_batch_step(int prec, const BatchStepArgs& a, int grid, cudaStream_t st);
 // field update of every replica (memd_field.cu)
 void launch_fused_batch(int prec, const RepDesc* desc, const int* cta_rep, int nctas, int par,
-                        int ty, int pf, int tw, cudaStream_t st, bool early = false);
+                        int ty, int pf, int tw, cudaStream_t st);
 // the batch's host I/O block (memd_batch_step_io): the members' particles in
 // order, member r from entry off[r] of ntot = off[count]; io_layout(ntot),
 // with count error words at its err offset
@@ -525,12 +564,16 @@ void launch_io_pack_batch(const RepDesc* desc, const int64_t* off, int count, in
                           void* io, cudaStream_t st, int part = kIoAll);
 // particle kernels of every replica (memd_particles.cu); thermostat from the arguments
 void launch_deposit_batch(const RepDesc* desc, const int* cta_rep, int nctas, int thermo,
-                          double gamma, double kT, cudaStream_t st);
+                          double gamma, double kT, cudaStream_t st, bool early = false);
+void launch_turn_batch_wide(int prec, const RepDesc* desc, const int* cta_rep, int nctas, int par,
+                            int thermo, cudaStream_t st, bool early = false);
+void launch_turn_batch(int prec, const RepDesc* desc, const int* cta_rep, int nctas, int par,
+                       int thermo, double gamma, double kT, cudaStream_t st, bool early = false);
 void launch_apply_batch(int prec, const RepDesc* desc, const int* cta_rep, int nctas, int par,
-                        cudaStream_t st);
+                        cudaStream_t st, int turn = 0);
 // one thread per charge (cta_rep over kWideThreads charges a CTA)
 void launch_deposit_batch_wide(const RepDesc* desc, const int* cta_rep, int nctas,
-                               cudaStream_t st);
+                               cudaStream_t st, bool early = false);
 void launch_gather_batch_wide(int prec, const RepDesc* desc, const int* cta_rep, int nctas,
                               int par, int thermo, cudaStream_t st);
 // dense form: CTA b takes the kApplyChunk transfer words from chunk[b].y *
@@ -539,7 +582,7 @@ constexpr int kApplyThreads = 256;
 constexpr int kApplyPairs = 4;  // 16-byte word pairs a thread, all loaded before any store
 constexpr int64_t kApplyChunk = 2 * kApplyPairs * kApplyThreads;  // words a CTA
 void launch_apply_dense_batch(int prec, const RepDesc* desc, const int2* chunk, int nchunks,
-                              int par, cudaStream_t st);
+                              int par, cudaStream_t st, int turn = 0);
 void launch_gather_batch(int prec, const RepDesc* desc, const int* cta_rep, int nctas, int par,
                          int thermo, double gamma, double kT, cudaStream_t st);
 // per-particle constants: h = (dt/2)/m always; sig when thermo is set

@@ -508,22 +508,17 @@ __device__ __forceinline__ long long deposit_body(const Mesh& m, const StepParam
 // coordinate of each axis; 0 for a thread past the last charge).  For large
 // charge counts: a warp then moves 32 charges an instruction instead of 8,
 // with no exchange of cells between lanes.
-__device__ __forceinline__ void deposit_wide(const Mesh& m, const StepParams& sp, Particles P,
-                                             unsigned long long* __restrict__ Tb, DevState* ds,
-                                             int64_t p, long long U[3]) {
-  U[0] = U[1] = U[2] = 0;
-  if (p >= P.n) return;
-  const double h = P.h[p];
-  const int q = P.q[p];
-  double x[3], xn[3];
+__device__ __forceinline__ void drift_wide(const Mesh& m, const StepParams& sp, Particles P,
+                                           unsigned long long* __restrict__ Tb, DevState* ds,
+                                           int64_t p, int q, const double v[3], const double x[3],
+                                           const int c0[3], const int f0[3], long long U[3]) {
+  double xn[3];
   int ko[3], kn[3];
   bool ok = true;
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    const double v = __dadd_rn(P.v[3 * p + d], __dmul_rn(h, P.Ft[3 * p + d]));
-    P.v[3 * p + d] = v;
-    const double step = __dmul_rn(sp.dt, v);
-    x[d] = P.x[3 * p + d];
+    P.v[3 * p + d] = v[d];
+    const double step = __dmul_rn(sp.dt, v[d]);
     ko[d] = P.img[3 * p + d];
     kn[d] = ko[d];
     xn[d] = x[d];
@@ -533,10 +528,9 @@ __device__ __forceinline__ void deposit_wide(const Mesh& m, const StepParams& sp
       ok = false;
     }
   }
-  int c0[3], f0[3], c1[3], f1[3], dc[3];
+  int c1[3], f1[3], dc[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
-    quantize(m, d, x[d], c0[d], f0[d]);
     fold(m.L[d], xn[d], kn[d]);
     quantize(m, d, xn[d], c1[d], f1[d]);
     dc[d] = c1[d] + (kn[d] - ko[d]) * m.n[d] - c0[d];
@@ -571,6 +565,23 @@ __device__ __forceinline__ void deposit_wide(const Mesh& m, const StepParams& sp
     }
     atomicOr(&ds->err, kErrCellJump);
   }
+}
+
+__device__ __forceinline__ void deposit_wide(const Mesh& m, const StepParams& sp, Particles P,
+                                             unsigned long long* __restrict__ Tb, DevState* ds,
+                                             int64_t p, long long U[3]) {
+  U[0] = U[1] = U[2] = 0;
+  if (p >= P.n) return;
+  const double h = P.h[p];
+  double v[3], x[3];
+  int c0[3], f0[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    v[d] = __dadd_rn(P.v[3 * p + d], __dmul_rn(h, P.Ft[3 * p + d]));
+    x[d] = P.x[3 * p + d];
+    quantize(m, d, x[d], c0[d], f0[d]);
+  }
+  drift_wide(m, sp, P, Tb, ds, p, P.q[p], v, x, c0, f0, U);
 }
 
 __global__ void __launch_bounds__(kWideThreads)
@@ -678,10 +689,26 @@ __device__ __forceinline__ void apply_body(const Mesh& m, Particles P,
     }
 }
 
+// Inside a run of steps the application, which no other particle kernel of
+// its system runs beside, does what the gather's last CTA does at the end of
+// a step: it closes the dipole sum of the move (kTurnClose: the kernel that
+// follows gathers this step's forces and deposits the next move into a fresh
+// sum) and counts the step whose gather came before it (kTurnCount).
+__device__ __forceinline__ void turn_step(DevState* ds, int turn) {
+  if (turn & kTurnClose)
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      ds->Plast[d] = (long long)ds->Pacc[d];
+      ds->Pacc[d] = 0ull;
+    }
+  if (turn & kTurnCount) ds->step += 1;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kQuadThreads)
     k_apply(const __grid_constant__ Mesh m, Particles P, unsigned long long* __restrict__ Tb, long long* __restrict__ Lg,
-            T* __restrict__ D, double scale, int64_t cmV) {
+            T* __restrict__ D, double scale, int64_t cmV, DevState* ds, int turn) {
+  if (turn && blockIdx.x == 0 && threadIdx.x == 0) turn_step(ds, turn);
   apply_body<T>(m, P, Tb, Lg, D, scale, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, cmV);
 }
 
@@ -744,7 +771,8 @@ __device__ __forceinline__ void apply_dense_range(long long* __restrict__ Tb,
 template <typename T>
 __global__ void __launch_bounds__(kApplyThreads)
     k_apply_dense(int64_t nl, long long* __restrict__ Tb, long long* __restrict__ Lg,
-                  T* __restrict__ D, double scale) {
+                  T* __restrict__ D, double scale, DevState* ds, int turn) {
+  if (turn && blockIdx.x == 0 && threadIdx.x == 0) turn_step(ds, turn);
   const int64_t l0 = (int64_t)blockIdx.x * kApplyChunk;
   apply_dense_range<T>(Tb, Lg, D, scale, l0, l0 + kApplyChunk < nl ? l0 + kApplyChunk : nl,
                        nl / 3);
@@ -1048,15 +1076,16 @@ __global__ void __launch_bounds__(kQuadThreads)
 // One thread per charge: the gather of gather_body with the same
 // expressions and the same order of every sum (each corner's three links,
 // then the corners as ((c0 + c1) + (c2 + c3))), one Philox block a charge.
-template <typename T>
-__device__ __forceinline__ void gather_wide(const Mesh& m, const StepParams& sp, int thermo,
-                                            Particles P, const T* __restrict__ D,
-                                            const T* __restrict__ ie,
-                                            const double* __restrict__ ie64, DevState* ds,
-                                            int kick, int64_t p, bool use_mv) {
-  if (p >= P.n) return;
-  const int qi = P.q[p];
-  int c[3], f[3];
+// Turn: the force goes on to the next half kick in the same thread, so it and
+// the velocity it gives are returned (v, Ft) instead of stored, with the cell
+// and the lattice steps (c, f).
+template <typename T, bool Turn>
+__device__ __forceinline__ void force_wide(const Mesh& m, const StepParams& sp, int thermo,
+                                           Particles P, const T* __restrict__ D,
+                                           const T* __restrict__ ie,
+                                           const double* __restrict__ ie64, DevState* ds,
+                                           int kick, int64_t p, bool use_mv, int qi, int c[3],
+                                           int f[3], double v[3], double Ftot[3]) {
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     if (use_mv) {
@@ -1067,11 +1096,10 @@ __device__ __forceinline__ void gather_wide(const Mesh& m, const StepParams& sp,
     }
   }
   long long Pl[3] = {0, 0, 0};
-  if (sp.dipole_corr) {
-    Pl[0] = (long long)__ldcg(&ds->Pacc[0]);
-    Pl[1] = (long long)__ldcg(&ds->Pacc[1]);
-    Pl[2] = (long long)__ldcg(&ds->Pacc[2]);
-  }
+  if (sp.dipole_corr)
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+      Pl[d] = Turn ? __ldcg(&ds->Plast[d]) : (long long)__ldcg(&ds->Pacc[d]);
   unsigned ctr[4] = {0u, 0u, 0u, 0u};
   if (thermo) {
     const long long step = __ldcg(&ds->step);
@@ -1145,10 +1173,88 @@ __device__ __forceinline__ void gather_wide(const Mesh& m, const StepParams& sp,
       const double fn = sig * unit_noise(ctr[d]);
       Ft = Fd + (fr + fn);
     }
-    P.F[3 * p + d] = Fd;
-    P.Ft[3 * p + d] = Ft;
-    if (kick) P.v[3 * p + d] = __dadd_rn(vd, __dmul_rn(hh, Ft));
+    if (Turn) {
+      Ftot[d] = Ft;
+      v[d] = __dadd_rn(vd, __dmul_rn(hh, Ft));
+    } else {
+      P.F[3 * p + d] = Fd;
+      P.Ft[3 * p + d] = Ft;
+      if (kick) P.v[3 * p + d] = __dadd_rn(vd, __dmul_rn(hh, Ft));
+    }
   }
+}
+
+template <typename T>
+__device__ __forceinline__ void gather_wide(const Mesh& m, const StepParams& sp, int thermo,
+                                            Particles P, const T* __restrict__ D,
+                                            const T* __restrict__ ie,
+                                            const double* __restrict__ ie64, DevState* ds,
+                                            int kick, int64_t p, bool use_mv) {
+  if (p >= P.n) return;
+  int c[3], f[3];
+  double v[3], Ft[3];
+  force_wide<T, false>(m, sp, thermo, P, D, ie, ie64, ds, kick, p, use_mv, P.q[p], c, f, v, Ft);
+}
+
+// The gather that closes a step and the kick, drift and deposition of the
+// next one, for a charge in one thread (a quad in one quad): same values as
+// the two kernels.
+template <typename T>
+__device__ __forceinline__ void turn_wide(const Mesh& m, const StepParams& sp, int thermo,
+                                          Particles P, unsigned long long* __restrict__ Tb,
+                                          const T* __restrict__ D, const T* __restrict__ ie,
+                                          const double* __restrict__ ie64, DevState* ds,
+                                          int64_t p, long long U[3]) {
+  U[0] = U[1] = U[2] = 0;
+  if (p >= P.n) return;
+  const int q = P.q[p];
+  int c[3], f[3];
+  double v[3], Ft[3], x[3];
+  force_wide<T, true>(m, sp, thermo, P, D, ie, ie64, ds, 1, p, true, q, c, f, v, Ft);
+  const double h = P.h[p];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    v[d] = __dadd_rn(v[d], __dmul_rn(h, Ft[d]));
+    x[d] = P.x[3 * p + d];
+  }
+  drift_wide(m, sp, P, Tb, ds, p, q, v, x, c, f, U);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kWideThreads)
+    k_turn_wide(const __grid_constant__ Mesh m, const __grid_constant__ StepParams sp,
+                Particles P, unsigned long long* __restrict__ Tb, const T* __restrict__ D,
+                const T* __restrict__ ie, const double* __restrict__ ie64, DevState* ds) {
+  let_next_start();
+  long long U[3];
+  turn_wide<T>(m, sp, sp.thermo, P, Tb, D, ie, ie64, ds,
+               blockIdx.x * (int64_t)blockDim.x + threadIdx.x, U);
+  cta_dipole_add3(ds->Pacc, U);
+}
+
+// quads: velocity and force go through memory, from a lane to itself
+template <typename T>
+__device__ __forceinline__ long long turn_body(const Mesh& m, const StepParams& sp, int thermo,
+                                               double gamma, double kT, Particles P,
+                                               unsigned long long* __restrict__ Tb,
+                                               const T* __restrict__ D, const T* __restrict__ ie,
+                                               const double* __restrict__ ie64, DevState* ds,
+                                               int64_t g) {
+  const long long pre[4] = {__ldcg(&ds->Plast[0]), __ldcg(&ds->Plast[1]), __ldcg(&ds->Plast[2]),
+                            __ldcg(&ds->step)};
+  gather_body<T>(m, sp, thermo, gamma, kT, P, D, ie, ie64, ds, 1, 0, 0u, g, nullptr, false, pre,
+                 true);
+  return deposit_body(m, sp, P, Tb, ds, g);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kQuadThreads)
+    k_turn(const __grid_constant__ Mesh m, const __grid_constant__ StepParams sp, Particles P,
+           unsigned long long* __restrict__ Tb, const T* __restrict__ D, const T* __restrict__ ie,
+           const double* __restrict__ ie64, DevState* ds) {
+  let_next_start();
+  cta_dipole_add(ds->Pacc, turn_body<T>(m, sp, sp.thermo, sp.gamma, sp.kT, P, Tb, D, ie, ie64, ds,
+                                        blockIdx.x * (int64_t)blockDim.x + threadIdx.x));
 }
 
 template <typename T>
@@ -1179,8 +1285,10 @@ __global__ void __launch_bounds__(kBatchQuadThreads)
 
 template <typename T>
 __global__ void __launch_bounds__(kBatchQuadThreads)
-    k_apply_batch(const RepDesc* __restrict__ desc, const int* __restrict__ cta_rep, int par) {
+    k_apply_batch(const RepDesc* __restrict__ desc, const int* __restrict__ cta_rep, int par,
+                  int turn) {
   const RepDesc& r = desc[cta_rep[blockIdx.x]];
+  if (turn && (int)blockIdx.x == r.p_first && threadIdx.x == 0) turn_step(r.ds, turn);
   apply_body<T>(r.m, r.P, (unsigned long long*)r.Tb, r.Lg, (T*)r.D[par ^ 1], r.sp.scale,
                 batch_local(r));
 }
@@ -1188,9 +1296,10 @@ __global__ void __launch_bounds__(kBatchQuadThreads)
 template <typename T>
 __global__ void __launch_bounds__(kApplyThreads)
     k_apply_dense_batch(const RepDesc* __restrict__ desc, const int2* __restrict__ chunk,
-                        int par) {
+                        int par, int turn) {
   const int2 c = chunk[blockIdx.x];
   const RepDesc& r = desc[c.x];
+  if (turn && c.y == 0 && threadIdx.x == 0) turn_step(r.ds, turn);
   const int64_t nl = 3 * r.m.V, l0 = (int64_t)c.y * kApplyChunk;
   apply_dense_range<T>(r.Tb, r.Lg, (T*)r.D[par ^ 1], r.sp.scale, l0,
                        l0 + kApplyChunk < nl ? l0 + kApplyChunk : nl, r.m.V);
@@ -1230,6 +1339,32 @@ __global__ void __launch_bounds__(kWideThreads)
   gather_wide<T>(r.m, r.sp, thermo, r.P, (const T*)r.D[par ^ 1], (const T*)r.ie, r.ie64, r.ds, 1,
                  batch_local_w(r), true);
   finish_update(r.ds, 2, (unsigned)r.pw_ctas);
+}
+
+// as in k_deposit_batch_wide: seven CTAs an SM with FP32 fields (at the 89
+// registers it takes unbounded, five: 64 replicas, 10 steps 1205 -> 1166 us;
+// FP64 takes 128 and would spill)
+template <typename T>
+__global__ void __launch_bounds__(kWideThreads, sizeof(T) == 4 ? 7 : 1)
+    k_turn_batch_wide(const RepDesc* __restrict__ desc, const int* __restrict__ cta_rep, int par,
+                      int thermo) {
+  let_next_start();
+  const RepDesc& r = desc[cta_rep[blockIdx.x]];
+  long long U[3];
+  turn_wide<T>(r.m, r.sp, thermo, r.P, (unsigned long long*)r.Tb, (const T*)r.D[par ^ 1],
+               (const T*)r.ie, r.ie64, r.ds, batch_local_w(r), U);
+  cta_dipole_add3(r.ds->Pacc, U);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kBatchQuadThreads)
+    k_turn_batch(const RepDesc* __restrict__ desc, const int* __restrict__ cta_rep, int par,
+                 int thermo, double gamma, double kT) {
+  let_next_start();
+  const RepDesc& r = desc[cta_rep[blockIdx.x]];
+  cta_dipole_add(r.ds->Pacc, turn_body<T>(r.m, r.sp, thermo, gamma, kT, r.P,
+                                          (unsigned long long*)r.Tb, (const T*)r.D[par ^ 1],
+                                          (const T*)r.ie, r.ie64, r.ds, batch_local(r)));
 }
 
 // ------------------------------------------- single-launch batch step
@@ -2119,13 +2254,11 @@ void launch_particle_constants(const StepParams& sp, Particles p, cudaStream_t s
 }
 
 void launch_kick_drift_deposit(const Mesh& m, const StepParams& sp, Particles p, long long* Tb,
-                               DevState* ds, cudaStream_t st) {
+                               DevState* ds, cudaStream_t st, bool early) {
   if (p.n >= kWideMinCharges)
-    k_deposit_wide<<<blocks_for(p.n, kWideThreads), kWideThreads, 0, st>>>(
-        m, sp, p, (unsigned long long*)Tb, ds);
+    launch_early(k_deposit_wide, blocks_for(p.n, kWideThreads), kWideThreads, 0, st, early, m, sp, p, (unsigned long long*)Tb, ds);
   else if (p.n > 0)
-    k_kick_drift_deposit<<<blocks_for(4 * p.n, quad_threads(p.n)), quad_threads(p.n), 0, st>>>(
-        m, sp, p, (unsigned long long*)Tb, ds);
+    launch_early(k_kick_drift_deposit, blocks_for(4 * p.n, quad_threads(p.n)), quad_threads(p.n), 0, st, early, m, sp, p, (unsigned long long*)Tb, ds);
 }
 
 void launch_move_deposit(const Mesh& m, Particles p, const double* pos_new, const int* img_new,
@@ -2136,25 +2269,28 @@ void launch_move_deposit(const Mesh& m, Particles p, const double* pos_new, cons
 }
 
 void launch_apply(const Mesh& m, int prec, Particles p, long long* Tb, long long* Lg, void* D,
-                  double scale, cudaStream_t st, int64_t cmV) {
+                  double scale, cudaStream_t st, int64_t cmV, DevState* ds, int turn) {
   if (p.n <= 0) return;
   const int qt = quad_threads(p.n);
   const unsigned nb = blocks_for(4 * p.n, qt);
   if (prec == 1)
-    k_apply<float><<<nb, qt, 0, st>>>(m, p, (unsigned long long*)Tb, Lg, (float*)D, scale, cmV);
+    k_apply<float><<<nb, qt, 0, st>>>(m, p, (unsigned long long*)Tb, Lg, (float*)D, scale, cmV,
+                                   ds, turn);
   else
     k_apply<double><<<nb, qt, 0, st>>>(m, p, (unsigned long long*)Tb, Lg, (double*)D, scale,
-                                       cmV);
+                                    cmV, ds, turn);
 }
 
 void launch_apply_dense(int prec, int64_t nlinks, long long* Tb, long long* Lg, void* D,
-                        double scale, cudaStream_t st) {
+                        double scale, cudaStream_t st, DevState* ds, int turn) {
   if (nlinks <= 0) return;
   const unsigned nb = (unsigned)((nlinks + kApplyChunk - 1) / kApplyChunk);
   if (prec == 1)
-    k_apply_dense<float><<<nb, kApplyThreads, 0, st>>>(nlinks, Tb, Lg, (float*)D, scale);
+    k_apply_dense<float><<<nb, kApplyThreads, 0, st>>>(nlinks, Tb, Lg, (float*)D, scale, ds,
+                                                        turn);
   else
-    k_apply_dense<double><<<nb, kApplyThreads, 0, st>>>(nlinks, Tb, Lg, (double*)D, scale);
+    k_apply_dense<double><<<nb, kApplyThreads, 0, st>>>(nlinks, Tb, Lg, (double*)D, scale, ds,
+                                                         turn);
 }
 
 size_t batch_step_smem() { return rows_smem_bytes(kBatchStepThreads, 4); }
@@ -2291,19 +2427,42 @@ void launch_gather(const Mesh& m, int prec, const StepParams& sp, Particles p, c
                                                   ie64, ds, kick, finish);
 }
 
+void launch_turn(const Mesh& m, int prec, const StepParams& sp, Particles p, long long* Tb,
+                 const void* D, const void* ie, const double* ie64, DevState* ds,
+                 cudaStream_t st, bool early) {
+  if (p.n <= 0) return;
+  unsigned long long* T = (unsigned long long*)Tb;
+  if (p.n >= kWideMinCharges) {
+    const unsigned nw = blocks_for(p.n, kWideThreads);
+    if (prec == 1)
+      launch_early(k_turn_wide<float>, nw, kWideThreads, 0, st, early, m, sp, p, T, (const float*)D,
+                                                      (const float*)ie, ie64, ds);
+    else
+      launch_early(k_turn_wide<double>, nw, kWideThreads, 0, st, early, m, sp, p, T, (const double*)D,
+                                                       (const double*)ie, ie64, ds);
+    return;
+  }
+  const int qt = quad_threads(p.n);
+  const unsigned nb = blocks_for(4 * p.n, qt);
+  if (prec == 1)
+    launch_early(k_turn<float>, nb, qt, 0, st, early, m, sp, p, T, (const float*)D, (const float*)ie, ie64, ds);
+  else
+    launch_early(k_turn<double>, nb, qt, 0, st, early, m, sp, p, T, (const double*)D, (const double*)ie, ie64, ds);
+}
+
 void launch_step_end(DevState* ds, int advance, cudaStream_t st) {
   k_step_end<<<1, 32, 0, st>>>(ds, advance);
 }
 
 void launch_deposit_batch(const RepDesc* desc, const int* cta_rep, int nctas, int thermo,
-                          double gamma, double kT, cudaStream_t st) {
+                          double gamma, double kT, cudaStream_t st, bool early) {
   if (nctas > 0)
-    k_deposit_batch<<<nctas, kBatchQuadThreads, 0, st>>>(desc, cta_rep, thermo, gamma, kT);
+    launch_early(k_deposit_batch, nctas, kBatchQuadThreads, 0, st, early, desc, cta_rep, thermo, gamma, kT);
 }
 
 void launch_deposit_batch_wide(const RepDesc* desc, const int* cta_rep, int nctas,
-                               cudaStream_t st) {
-  if (nctas > 0) k_deposit_batch_wide<<<nctas, kWideThreads, 0, st>>>(desc, cta_rep);
+                               cudaStream_t st, bool early) {
+  if (nctas > 0) launch_early(k_deposit_batch_wide, nctas, kWideThreads, 0, st, early, desc, cta_rep);
 }
 
 void launch_gather_batch_wide(int prec, const RepDesc* desc, const int* cta_rep, int nctas,
@@ -2315,22 +2474,40 @@ void launch_gather_batch_wide(int prec, const RepDesc* desc, const int* cta_rep,
     k_gather_batch_wide<double><<<nctas, kWideThreads, 0, st>>>(desc, cta_rep, par, thermo);
 }
 
-void launch_apply_batch(int prec, const RepDesc* desc, const int* cta_rep, int nctas, int par,
-                        cudaStream_t st) {
+void launch_turn_batch_wide(int prec, const RepDesc* desc, const int* cta_rep, int nctas, int par,
+                            int thermo, cudaStream_t st, bool early) {
   if (nctas <= 0) return;
   if (prec == 1)
-    k_apply_batch<float><<<nctas, kBatchQuadThreads, 0, st>>>(desc, cta_rep, par);
+    launch_early(k_turn_batch_wide<float>, nctas, kWideThreads, 0, st, early, desc, cta_rep, par, thermo);
   else
-    k_apply_batch<double><<<nctas, kBatchQuadThreads, 0, st>>>(desc, cta_rep, par);
+    launch_early(k_turn_batch_wide<double>, nctas, kWideThreads, 0, st, early, desc, cta_rep, par, thermo);
+}
+
+void launch_turn_batch(int prec, const RepDesc* desc, const int* cta_rep, int nctas, int par,
+                       int thermo, double gamma, double kT, cudaStream_t st, bool early) {
+  if (nctas <= 0) return;
+  if (prec == 1)
+    launch_early(k_turn_batch<float>, nctas, kBatchQuadThreads, 0, st, early, desc, cta_rep, par, thermo, gamma, kT);
+  else
+    launch_early(k_turn_batch<double>, nctas, kBatchQuadThreads, 0, st, early, desc, cta_rep, par, thermo, gamma, kT);
+}
+
+void launch_apply_batch(int prec, const RepDesc* desc, const int* cta_rep, int nctas, int par,
+                        cudaStream_t st, int turn) {
+  if (nctas <= 0) return;
+  if (prec == 1)
+    k_apply_batch<float><<<nctas, kBatchQuadThreads, 0, st>>>(desc, cta_rep, par, turn);
+  else
+    k_apply_batch<double><<<nctas, kBatchQuadThreads, 0, st>>>(desc, cta_rep, par, turn);
 }
 
 void launch_apply_dense_batch(int prec, const RepDesc* desc, const int2* chunk, int nchunks,
-                              int par, cudaStream_t st) {
+                              int par, cudaStream_t st, int turn) {
   if (nchunks <= 0) return;
   if (prec == 1)
-    k_apply_dense_batch<float><<<nchunks, kApplyThreads, 0, st>>>(desc, chunk, par);
+    k_apply_dense_batch<float><<<nchunks, kApplyThreads, 0, st>>>(desc, chunk, par, turn);
   else
-    k_apply_dense_batch<double><<<nchunks, kApplyThreads, 0, st>>>(desc, chunk, par);
+    k_apply_dense_batch<double><<<nchunks, kApplyThreads, 0, st>>>(desc, chunk, par, turn);
 }
 
 void launch_gather_batch(int prec, const RepDesc* desc, const int* cta_rep, int nctas, int par,

@@ -90,6 +90,7 @@ __global__ void __launch_bounds__(32 * TY)
                 const __grid_constant__ CUtensorMap tB, Mesh m, const T* __restrict__ Din,
                 const T* __restrict__ Bin, const T* __restrict__ ie, T* __restrict__ Dout,
                 T* __restrict__ Bout, T cB, T cD, int zchunk, unsigned int* err) {
+  let_next_start();
   using G = TmaGeom<T, TY>;
   constexpr int TX = G::TX, HP = G::HP, BXW = G::BXW, BYH = G::BYH, BX = G::BX, BY = G::BY;
   constexpr int NT = TX * TY;
