@@ -131,8 +131,9 @@ typedef struct memd_options {
                              multiple of 4 sites for FP32, 2 for FP64; else the site
                              kernel).  All give the same results (TMA to rounding). */
   int32_t step_engine;    /* MEMD_STEP_AUTO: the single launch for small systems (at
-                             most 125000 sites, 110000 with FP64 fields, and 60
-                             particles per SM), else the graph;
+                             most 33000 sites and 60 particles per SM; in host round
+                             trips of one step up to 125000 sites, 110000 with FP64
+                             fields), else the graph;
                              MEMD_STEP_GRAPH: four kernels a step (field update beside
                              the deposition, transfers, gather); MEMD_STEP_SINGLE: the
                              whole step in one cooperative launch with one grid

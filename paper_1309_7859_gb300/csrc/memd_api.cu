@@ -1201,19 +1201,21 @@ memd_status memd_flush(memd_ctx* c) {
 
 extern "C" {
 
-// single launch or graph of four kernels for this system (decided when the
-// step graphs are built, once the particle count is known).  Left to choose,
-// the single launch runs where it was the faster of the two: FP32 32^3
-// 7.2-7.7 us a step against 16-19 (200 to 4800 charges), 48^3 14-17.6 against
-// 16.5-22.6 (200 to 9000), 56^3 18-24 against 16.5-21.6; FP64 40^3 21-30
-// against 30-37, 48^3 26-36.5 against 30-37, 56^3 37-49 against 38-45; and
-// from 16000 charges (four passes of its particle warps) 26-51 against
-// 25-47.
-static bool want_coop(const memd_ctx* c) {
+// single launch or graph for this call.  Left to choose, the single launch
+// runs where it was the faster of the two: up to 32^3, where a field tile of
+// few rows goes to every SM, FP32 7.5-8.0 us a step of a 20-step call against
+// 9.5-10.6 (200 to 3000 charges), FP64 13.8-16 against 15.5-18.  33^3 needs
+// larger tiles: FP32 11.8-13.7 against 9.9-10.7, FP64 20-23.5 against
+// 17.4-23.8; 48^3 14-17.7 and 27-37 against 9.8-12.7 and 19.4-30.7 (200 to
+// 9000 charges), and one step a call 36-39 and 50-58 against 31-34 and 44-52.
+// A host round trip of one step in place (io) has no launch but its own in
+// the single launch, and is faster there up to 48^3: FP32 26-31 us a call
+// against 30-45 (200 to 8000 charges), FP64 40-48.5 against 42-61.
+static bool want_coop(const memd_ctx* c, bool io) {
   if (c->coop_grid <= 0 || c->step_engine == MEMD_STEP_GRAPH) return false;
   if (c->step_engine == MEMD_STEP_SINGLE) return true;
-  return c->mesh.V <= (c->prec == MEMD_FP32 ? 125000 : 110000) &&
-         c->P.n <= (int64_t)60 * c->coop_grid;
+  const int64_t most = io || c->skewed ? (c->prec == MEMD_FP32 ? 125000 : 110000) : 33000;
+  return c->mesh.V <= most && c->P.n <= (int64_t)60 * c->coop_grid;
 }
 
 // Errors raised by kernels of earlier batches, without blocking: the flag is
@@ -1224,10 +1226,10 @@ static memd_status poll_err(memd_ctx* c, bool block) {
 }
 
 // what every step needs before it is launched: the per-particle constants
-// of this thermostat, the engine (decided when the step graphs are built),
-// the second transfer buffer of the single launch, applied transfers for the
-// graph engine, the tuned field kernel
-static memd_status step_prepare(memd_ctx* c, const memd_thermostat* th, StepParams& sp) {
+// of this thermostat, the engine, the transfer slots of the single launch,
+// applied transfers for the graph engine, the tuned field kernel
+static memd_status step_prepare(memd_ctx* c, const memd_thermostat* th, StepParams& sp,
+                                bool io = false) {
   const int thermo = th ? 1 : 0;
   const double gamma = th ? th->gamma : 0.0, kT = th ? th->kT : 0.0;
   sp = step_params(c, thermo, gamma, kT);
@@ -1240,7 +1242,7 @@ static memd_status step_prepare(memd_ctx* c, const memd_thermostat* th, StepPara
     c->graph_gamma = gamma;
     c->graph_kT = kT;
   }
-  if (!c->graph[0] && !c->graph[1] && !c->run.any) c->coop = want_coop(c);
+  c->coop = want_coop(c, io);
   if (c->coop && !c->Tb2) {
     // the single-launch step's transfer slots (3 V words each)
     c->Tb2 = (long long*)dalloc(c, kCoopSlots * 3 * c->mesh.V * sizeof(long long));
@@ -1448,7 +1450,10 @@ memd_status memd_inject(memd_ctx* c, int32_t kind, double wait_s) {
   c->wait_ns = wait_s > 0.0 ? (unsigned long long)(wait_s * 1e9) : kBarrierWaitNs;
   if (kind == MEMD_INJECT_BARRIER_SKEW) {
     if (!c->initialised) return fail(c, MEMD_ERR_STATE, "memd_init_field first");
-    if (!c->coop) return fail(c, MEMD_ERR_STATE, "the steps of this context have no grid barrier");
+    // a context whose round trips would take the single launch takes it from now on
+    if (!c->coop && !(c->fcfg_ready && want_coop(c, true)))
+      return fail(c, MEMD_ERR_STATE, "the steps of this context have no grid barrier");
+    c->skewed = true;
     // one extra arrival: the next barrier's count cannot reach its target
     unsigned long long n = 0;
     CK(cudaStreamSynchronize(c->stream));
@@ -1614,7 +1619,7 @@ memd_status memd_step_io(memd_ctx* c, int32_t load, int64_t nsteps, const memd_t
   if (load && nsteps == 1 && c->P.n > 0) {
     // the usual host loop: one launch a call
     StepParams sp;
-    s = step_prepare(c, th, sp);
+    s = step_prepare(c, th, sp, direct);
     if (s != MEMD_OK) return s;
     const bool timed = c->time_kernels != 0;
     const int par = c->cur;

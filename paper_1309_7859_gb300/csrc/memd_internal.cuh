@@ -139,7 +139,6 @@ constexpr int kRunSteps = 16;
 struct StepRuns {
   cudaGraphExec_t graph[2][kRunSteps + 1] = {};
   int asked[kRunSteps + 1] = {};
-  bool any = false;
 };
 // steps of the next launch when `left` remain; `single` (0 before the first)
 // counts down the rest of a run that is not recorded yet
@@ -150,10 +149,7 @@ inline int run_length(StepRuns& r, int par, int64_t left, int64_t* single) {
     return 1;
   }
   if (k < 2) return 1;
-  if (r.graph[par][k] || r.asked[k]++ >= 2) {
-    r.any = true;
-    return k;
-  }
+  if (r.graph[par][k] || r.asked[k]++ >= 2) return k;
   *single = k - 1;
   return 1;
 }

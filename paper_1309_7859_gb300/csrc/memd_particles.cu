@@ -2253,8 +2253,34 @@ void launch_particle_constants(const StepParams& sp, Particles p, cudaStream_t s
   if (p.n > 0) k_particle_constants<<<blocks_for(p.n), kThreads, 0, st>>>(sp, p);
 }
 
+namespace {
+// A quad kernel of few charges leaves an SM room for the row kernel that runs
+// beside it, so it asks for the row kernel's split of the SM's L1 and shared
+// memory: an SM changes its split only when it is empty, and one warp under
+// the default split kept the row kernel's CTAs off its SM until it ended
+// (FP64 32^3, 1000 charges: 22 us a step for 14).  The wide kernels fill the
+// SMs themselves and live off the L1 (64 replicas, 10 steps: 1180 us, with
+// the row kernel's split 1560-1590), so they keep the default.
+bool prefer_shared() {
+  const void* k[] = {
+      (const void*)k_kick_drift_deposit,  (const void*)k_deposit_batch,
+      (const void*)k_turn<float>,         (const void*)k_turn<double>,
+      (const void*)k_turn_batch<float>,   (const void*)k_turn_batch<double>};
+  for (const void* f : k)
+    if (cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+      cudaGetLastError();  // a preference: without it the results are the same
+  return true;
+}
+void set_split() {
+  static const bool done = prefer_shared();
+  (void)done;
+}
+}  // namespace
+
 void launch_kick_drift_deposit(const Mesh& m, const StepParams& sp, Particles p, long long* Tb,
                                DevState* ds, cudaStream_t st, bool early) {
+  set_split();
   if (p.n >= kWideMinCharges)
     launch_early(k_deposit_wide, blocks_for(p.n, kWideThreads), kWideThreads, 0, st, early, m, sp, p, (unsigned long long*)Tb, ds);
   else if (p.n > 0)
@@ -2430,6 +2456,7 @@ void launch_gather(const Mesh& m, int prec, const StepParams& sp, Particles p, c
 void launch_turn(const Mesh& m, int prec, const StepParams& sp, Particles p, long long* Tb,
                  const void* D, const void* ie, const double* ie64, DevState* ds,
                  cudaStream_t st, bool early) {
+  set_split();
   if (p.n <= 0) return;
   unsigned long long* T = (unsigned long long*)Tb;
   if (p.n >= kWideMinCharges) {
@@ -2456,6 +2483,7 @@ void launch_step_end(DevState* ds, int advance, cudaStream_t st) {
 
 void launch_deposit_batch(const RepDesc* desc, const int* cta_rep, int nctas, int thermo,
                           double gamma, double kT, cudaStream_t st, bool early) {
+  set_split();
   if (nctas > 0)
     launch_early(k_deposit_batch, nctas, kBatchQuadThreads, 0, st, early, desc, cta_rep, thermo, gamma, kT);
 }
@@ -2485,6 +2513,7 @@ void launch_turn_batch_wide(int prec, const RepDesc* desc, const int* cta_rep, i
 
 void launch_turn_batch(int prec, const RepDesc* desc, const int* cta_rep, int nctas, int par,
                        int thermo, double gamma, double kT, cudaStream_t st, bool early) {
+  set_split();
   if (nctas <= 0) return;
   if (prec == 1)
     launch_early(k_turn_batch<float>, nctas, kBatchQuadThreads, 0, st, early, desc, cta_rep, par, thermo, gamma, kT);

@@ -13,14 +13,14 @@ pytestmark = pytest.mark.gpu
 TH = (1.0, 1.0)
 
 
-def make(mesh, n, precision, **kw):
+def make(mesh, n, precision, engine="graph", **kw):
     from paper_1309_7859_gb300.memd import Memd
     rng = np.random.default_rng(n + mesh[0])
     box = tuple(float(N) for N in mesh)
     eps = EpsSpec("vertices", 0, (), inputs.smooth_random_vertices(rng, mesh, 1.0))
     x, q = inputs.uniform_positions(rng, n, box), inputs.neutral_charges(rng, n)
     m, v = rng.uniform(0.5, 2.0, n), inputs.thermal_velocities(rng, n)
-    g = Memd(mesh, box, eps, dt=0.005, precision=precision, seed=9, step_engine="graph", **kw)
+    g = Memd(mesh, box, eps, dt=0.005, precision=precision, seed=9, step_engine=engine, **kw)
     g.init_field(x, q, m, v)
     return g
 
@@ -80,3 +80,23 @@ def test_batch_runs_match_single_steps(counts, precision):
     b.close()
     for g in A + B:
         g.close()
+
+
+def test_engine_chosen_call_by_call_matches_graph():
+    """a mesh that takes the single launch in host round trips, the graph
+    otherwise"""
+    a, b = (make((40, 36, 38), 1200, "fp32", engine=e) for e in ("auto", "graph"))
+    seen = []
+    for n in (20, 1, 3, 1, 20, 20, 1):
+        for g in (a, b):
+            if n == 1:
+                io = g.io_buffers()
+                io["pos"][...], io["vel"][...], io["img"][...] = g.particles()
+                g.step_io(1, TH)
+            else:
+                g.step(n, TH)
+        seen.append(a.kernel_stats().single)
+    assert seen == [n == 1 for n in (20, 1, 3, 1, 20, 20, 1)]
+    same(a, b)
+    a.close()
+    b.close()
