@@ -61,6 +61,7 @@ struct memd_batch {
   int engine = MEMD_STEP_AUTO;
   bool single = false;
   bool single_graph_ok = true;  // its launch can be captured in a graph
+  bool left = false;    // every member has left (memd_batch_members_left)
   bool overlap = true;  // graph engine: the deposition beside the field pass
   int bs_grid = 0;
   int bs_field_ctas = -1;   // -1: half the grid
@@ -723,6 +724,8 @@ memd_status batch_refresh(memd_batch* b) {
 
 }  // namespace
 
+void memd_batch_members_left(memd_batch* b) { b->left = true; }
+
 // New members for an existing batch (the request server between rounds):
 // the tables are rebuilt with the batch's field-kernel choice, stream-ordered
 // behind the work already queued (the old tables and step graphs are released
@@ -746,7 +749,9 @@ memd_status memd_batch_update_members(memd_batch* b, int32_t count, memd_ctx* co
   }
   BCK(cudaSetDevice(b->device));
   harvest(b);
-  std::vector<memd_ctx*> old = b->m;
+  std::vector<memd_ctx*> old;
+  if (!b->left) old = b->m;
+  b->left = false;
   b->m.assign(members, members + count);
   b->gen.assign(count, -1);
   b->base.assign(count, 0);

@@ -132,3 +132,7 @@ memd_status memd_batch_update_members(memd_batch* b, int32_t count, memd_ctx* co
 // whether the deposition runs beside the field pass (the default) or after
 // it on the batch's stream; the step graphs are rebuilt at the next step
 void memd_batch_set_overlap(memd_batch* b, bool overlap);
+// every member has left and may be destroyed: the next memd_batch_update_members
+// takes all of its members for new ones (a new context can have the address of
+// an old one)
+void memd_batch_members_left(memd_batch* b);

@@ -484,6 +484,7 @@ memd_status memd_server_pump(memd_server* s, int32_t* n_active, int32_t* n_queue
       launched = true;
     }
   }
+  if (s->active.empty() && s->batch) memd_batch_members_left(s->batch);
   // 4. the quantum before this one has finished once the stream reaches this
   // point; results of the requests that left are copied on the server's
   // second stream meanwhile, so the quantum just queued keeps the GPU busy
