@@ -375,6 +375,16 @@ def particle_bytes(esz):
             "gather": 84 + 72 + 12 * 2 * esz}
 
 
+def batch_launches(ks, steps):
+    """Launches of our kernels in one call of `steps` batch steps, at least:
+    the graph engine runs up to 16 steps as one graph, in which a step's
+    gather and the next one's deposition are one launch (3 a step and one
+    more); steps of a length not yet recorded take 4."""
+    if ks.single:
+        return int(steps)
+    return 3 * int(steps) + -(-int(steps) // 16)
+
+
 def clock_preroll(step_fn, sync, seconds=1.0, max_steps=20000):
     """Untimed steps for about `seconds` so that the nvidia-smi sampler (200 ms
     period) sees the GPU under this load just before the timed steps."""
@@ -556,7 +566,7 @@ def batch_line(args, world, rank, local):
                            "application and gather, velocities, forces and error words "
                            "after it, one sync"},
             "clocks": clk.summary(),
-            "gpu_launches": int(ks0.launches_per_step * args.steps),
+            "gpu_launches": batch_launches(ks0, args.steps),
             "setup_s": setup_s,
             "gauss_exact": bool(exact),
         }
