@@ -140,12 +140,13 @@ def test_requests_after_the_batch_has_drained():
     """one request at a time, so every member leaves before the next one joins
     (and the next context may have the address of the last)"""
     from paper_1309_7859_gb300.memd import Server
-    reqs = requests(count=6, seed=23)
+    reqs = requests(count=12, seed=23)
+    refs = [alone(s) for s in reqs]
     srv = Server(precision="fp32", budget_bytes=64 << 20, max_slots=2, quantum=32, thermostat=TH)
-    for k, s in enumerate(reqs):
+    for k, (s, ref) in enumerate(zip(reqs, refs)):
         r = srv.submit(s)
         for _ in range(5000):
             if srv.pump()[2] == k + 1:
                 break
-        check_same(srv.result(r), alone(s))
+        check_same(srv.result(r), ref)
     srv.close()
