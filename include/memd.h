@@ -188,7 +188,9 @@ typedef struct memd_kernel_stats {
   double field_ms;        /* summed CUDA-event time of the field (curl) kernels */
   int64_t field_launches; /* launches timed */
   double field_bytes;     /* algorithmic bytes per field launch */
-  int64_t launches_per_step;
+  int64_t launches_per_step; /* of a step by itself; inside a call of several steps the
+                             graph's gather and next deposition are one launch, and
+                             the single launch takes up to 32 steps */
   int32_t field_tma;      /* field kernel chosen at create: 1 TMA-staged, 0 plain loads */
   int32_t field_ty;       /* its tile height (rows of field_tx sites) */
   int32_t field_zchunk;   /* its z planes per CTA */

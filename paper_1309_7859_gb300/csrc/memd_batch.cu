@@ -29,7 +29,7 @@ struct memd_batch {
   int device = 0;
   cudaStream_t stream = nullptr;
   cudaStream_t side = nullptr;
-  cudaEvent_t fork = nullptr, join = nullptr, ev0 = nullptr, ev1 = nullptr;
+  cudaEvent_t fork = nullptr, ev0 = nullptr, ev1 = nullptr;
   // memd_batch_step_io's one-step graph (per buffer parity) and its events
   cudaGraphExec_t io_graph[2] = {nullptr, nullptr};
   cudaEvent_t io_dep = nullptr, io_join = nullptr;
@@ -794,7 +794,6 @@ memd_status memd_batch_create_opt(int32_t count, memd_ctx* const* members, memd_
   if (cudaSetDevice(b->device) != cudaSuccess ||
       cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess ||
-      cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&b->io_dep, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&b->io_join, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreate(&b->ev0) != cudaSuccess || cudaEventCreate(&b->ev1) != cudaSuccess ||
@@ -843,7 +842,6 @@ void memd_batch_destroy(memd_batch* b) {
   free_tables(b);
   free_io(b);
   if (b->fork) cudaEventDestroy(b->fork);
-  if (b->join) cudaEventDestroy(b->join);
   if (b->io_dep) cudaEventDestroy(b->io_dep);
   if (b->io_join) cudaEventDestroy(b->io_join);
   if (b->ev0) cudaEventDestroy(b->ev0);
