@@ -236,7 +236,9 @@ void memd_destroy(memd_ctx *ctx);
  * mass (n, positive and finite; NULL = 1), vel (n x 3, NULL = 0).  Deposits
  * the charges, solves Gauss's law exactly in the int64 ledger, sets the k = 0
  * mode of D to -P/V, relaxes to curl E = 0 in FP64, sets B = 0 and computes
- * the forces.  A
+ * the forces.  (B one step later follows curl E of this field: zero in exact
+ * arithmetic, it holds the field's rounding alone until the charges have moved
+ * it, from the second step on.)  A
  * non-neutral system gets a uniform background, which must be an integer in
  * units of e 2^-48 per vertex.  Errors: INVALID, OOM, GAUSS, RELAX_NOCONV,
  * CUDA. */
