@@ -118,7 +118,7 @@ typedef struct memd_options {
   void *alloc_user;
   int32_t time_kernels;   /* 1: CUDA events around the field kernels, see
                              memd_get_kernel_stats */
-  int32_t field_kernel;   /* MEMD_FIELD_AUTO: the ROWS kernel (its two CTA widths
+  int32_t field_kernel;   /* MEMD_FIELD_AUTO: the ROWS kernel (its three CTA widths
                              timed) where the mesh fits it, else timed over the
                              kernels below;
                              MEMD_FIELD_LDG: plain-load kernel, halo loops per thread;
@@ -153,8 +153,8 @@ typedef struct memd_options {
                              the shape is fixed: {ty, zchunk, planes_ahead, rows_nt}:
                              tile height 4, 8 or 16 (16 needs FP32) and z planes per
                              CTA >= 1 of the LDG, SITE and TMA kernels (SITE: planes
-                             loaded ahead 1 or 2), threads a CTA 256 or 512 of the ROWS
-                             kernel; a value the chosen field_kernel does not use must be
+                             loaded ahead 1 or 2), threads a CTA 256, 512 or 576 of the
+                             ROWS kernel; a value the chosen field_kernel does not use must be
                              0, and field_kernel must not be AUTO.  Out of range:
                              INVALID at create.  A batch whose members all fix the same
                              ROWS width steps its field pass with that width, untuned. */

@@ -491,7 +491,7 @@ static memd_status autotune_fused(memd_ctx* c) {
   FusedCfg cand[160];
   int nc = 0;
   const int fk = c->field_kernel;
-  // Left to choose, the row kernel's two widths are the only candidates
+  // Left to choose, the row kernel's three widths are the only candidates
   // where the mesh fits it: in the step the field pass runs beside the
   // deposition, and there the row kernel was the fastest measured on every
   // such mesh (64^3 salt and colloid systems: 35.2 / 31.2 us a step against
@@ -822,7 +822,8 @@ memd_status memd_create(const int32_t mesh[3], const double box[3], const memd_e
       const int fk = o.field_kernel;
       if (fk == MEMD_FIELD_AUTO) return MEMD_ERR_INVALID;
       if (fk == MEMD_FIELD_ROWS) {
-        if (fs[0] || fs[1] || fs[2] || (fs[3] != 256 && fs[3] != 512)) return MEMD_ERR_INVALID;
+        if (fs[0] || fs[1] || fs[2] || (fs[3] != 256 && fs[3] != 512 && fs[3] != kRowsWide))
+          return MEMD_ERR_INVALID;
       } else {
         if (fs[3] || (fs[0] != 4 && fs[0] != 8 && fs[0] != 16) || fs[1] < 1) return MEMD_ERR_INVALID;
         if (fs[0] == 16 && o.precision != MEMD_FP32) return MEMD_ERR_INVALID;
