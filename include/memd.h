@@ -296,7 +296,8 @@ memd_status memd_dipole_check(memd_ctx *ctx, double limit, double *ratio);
  * its wait runs out after wait_s seconds (0: the default 0.2 s), the step is
  * void (fields and forces of that step are not to be used; reload a saved
  * state) and the next synchronising call reports MEMD_ERR_TIMEOUT and starts
- * the count afresh.  MEMD_INJECT_NONE only sets the wait bound (wait_s, 0:
+ * the count afresh.  (A context left to choose its engine takes the single
+ * launch from the injection to that report.)  MEMD_INJECT_NONE only sets the wait bound (wait_s, 0:
  * the default).  Errors: INVALID (unknown kind, wait_s outside [0, 10]),
  * STATE (not initialised, or no grid barrier in this context's steps), CUDA. */
 enum { MEMD_INJECT_NONE = 0, MEMD_INJECT_BARRIER_SKEW = 1 };

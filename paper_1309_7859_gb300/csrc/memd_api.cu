@@ -131,8 +131,10 @@ memd_status memd_check_err(memd_ctx* c) {
   CK(cudaStreamSynchronize(c->stream));
   if (err) {
     CK(cudaMemsetAsync(&c->ds->err, 0, sizeof(unsigned int), c->stream));
-    if (err & kErrTimeout)  // a grid barrier gave up: start its words afresh
+    if (err & kErrTimeout) {  // a grid barrier gave up: start its words afresh
       CK(cudaMemsetAsync(&c->ds->bar_arrivals, 0, sizeof(unsigned long long), c->stream));
+      c->skewed = false;  // an injected arrival is gone with them
+    }
     CK(cudaStreamSynchronize(c->stream));
     if (err & kErrCellJump) return fail(c, MEMD_ERR_CELL_JUMP, "a charge moved more than one cell");
     if (err & kErrGauss) return fail(c, MEMD_ERR_GAUSS, "Gauss scan did not close (system not neutral)");
@@ -1451,7 +1453,8 @@ memd_status memd_inject(memd_ctx* c, int32_t kind, double wait_s) {
   c->wait_ns = wait_s > 0.0 ? (unsigned long long)(wait_s * 1e9) : kBarrierWaitNs;
   if (kind == MEMD_INJECT_BARRIER_SKEW) {
     if (!c->initialised) return fail(c, MEMD_ERR_STATE, "memd_init_field first");
-    // a context whose round trips would take the single launch takes it from now on
+    // a context whose round trips would take the single launch takes it until
+    // the timeout has been reported
     if (!c->coop && !(c->fcfg_ready && want_coop(c, true)))
       return fail(c, MEMD_ERR_STATE, "the steps of this context have no grid barrier");
     c->skewed = true;

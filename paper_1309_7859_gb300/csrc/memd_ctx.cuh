@@ -66,7 +66,7 @@ struct memd_ctx {
   int* rows_first = nullptr;
   int rows_nctas = 0;
   int rows_nt = 0;       // a permittivity is mapped (memd_set_eps restores it on failure)
-  bool skewed = false;  // a barrier fault was injected: keeps the engine with a barrier
+  bool skewed = false;  // a barrier fault is injected and not yet reported: the engine with a barrier
   // step graphs, one per buffer parity
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   memd::StepRuns run;
