@@ -1126,11 +1126,12 @@ static memd_status record_step(memd_ctx* c, const StepParams& sp, int par, bool 
   // the charge transfer, in a run behind the gather of the step before, whose
   // D is this step's
   auto transfer = [&](bool behind_field) {
+    const bool join = behind_field && !c->use_graphs;
     if (first || !early)
-      launch_kick_drift_deposit(m, sp, c->P, c->Tb, c->ds, st, behind_field);
+      launch_kick_drift_deposit(m, sp, c->P, c->Tb, c->ds, st, behind_field, join);
     else
       launch_turn(m, c->prec, sp, c->P, c->Tb, c->Dbuf[par], c->ie, c->ie64, c->ds, st,
-                  behind_field);
+                  behind_field, join);
   };
   if (timed) {
     // instrumented: the field update alone between its event pair
@@ -1142,10 +1143,13 @@ static memd_status record_step(memd_ctx* c, const StepParams& sp, int par, bool 
     transfer(false);
     launch_field(c, par, sp.coefB, sp.coefD, c->fcfg, true);
   } else {
+    // the application is behind both: in a graph by an edge from the field
+    // pass, on a stream, where a kernel launched early need not be behind the
+    // one before it, by the end of the transfer (which costs 1-4% in a graph)
     launch_field(c, par, sp.coefB, sp.coefD, c->fcfg);
-    CK(cudaEventRecord(c->fork, st));
+    if (c->use_graphs) CK(cudaEventRecord(c->fork, st));
     transfer(early);
-    CK(cudaStreamWaitEvent(st, c->fork, 0));
+    if (c->use_graphs) CK(cudaStreamWaitEvent(st, c->fork, 0));
   }
   const int turn = early ? (first ? 0 : kTurnCount) | (last ? 0 : kTurnClose) : 0;
   if (apply_dense(c->apply_mode))
@@ -1294,10 +1298,17 @@ memd_status memd_step(memd_ctx* c, int64_t nsteps, const memd_thermostat* th) {
   for (int64_t s = 0; s < nsteps;) {
     const int par = c->cur;
     harvest_timing(c);
-    const int k = c->use_graphs && !timed ? run_length(c->run, par, nsteps - s, &single) : 1;
+    // without graphs a run is launched as it is, with nothing to record first
+    // (FP64, 20000 charges, 10 steps
+    // a call: 64^3 709 us step by step, 657 so; 95^3 1094 and 974)
+    const int k = timed           ? 1
+                  : c->use_graphs ? run_length(c->run, par, nsteps - s, &single)
+                                  : (int)std::min<int64_t>(nsteps - s, kRunSteps);
     if (!c->use_graphs) {
-      const memd_status r = record_step(c, sp, par, timed);
-      if (r != MEMD_OK) return r;
+      for (int j = 0; j < k; ++j) {
+        const memd_status r = record_step(c, sp, par ^ (j & 1), timed, j == 0, j == k - 1);
+        if (r != MEMD_OK) return r;
+      }
     } else {
       cudaGraphExec_t& gx = k > 1 ? c->run.graph[par][k] : c->graph[par];
       if (!gx) {

@@ -406,9 +406,11 @@ void launch_cic(const Mesh& m, Particles p, long long* Q, long long bg, cudaStre
 // cloud-in-cell deposit of |q| (int64, e 2^-48) at the vertices
 void launch_cic_abs(const Mesh& m, Particles p, long long* Q, cudaStream_t st);
 void launch_dipole(const Mesh& m, Particles p, DevState* ds, cudaStream_t st);
+// early: behind the field pass, which it does not wait for; join: it ends no
+// earlier than the pass, so that what follows it on a stream is behind both
 void launch_kick_drift_deposit(const Mesh& m, const StepParams& sp, Particles p,
                                long long* Tb, DevState* ds, cudaStream_t st,
-                               bool early = false);
+                               bool early = false, bool join = false);
 void launch_move_deposit(const Mesh& m, Particles p, const double* pos_new,
                          const int* img_new, long long* Tb, DevState* ds, cudaStream_t st);
 // cmV: the layout of Tb (tw_index); the ledger Lg is always the pairs'
@@ -440,7 +442,7 @@ void launch_step_end(DevState* ds, int advance, cudaStream_t st);
 constexpr int kTurnClose = 1, kTurnCount = 2;
 void launch_turn(const Mesh& m, int prec, const StepParams& sp, Particles p, long long* Tb,
                  const void* D, const void* ie, const double* ie64, DevState* ds,
-                 cudaStream_t st, bool early = false);
+                 cudaStream_t st, bool early = false, bool join = false);
 
 // ------------------------------------------------------- batched replicas
 // One independent system of a batch, as the batched kernels see it.

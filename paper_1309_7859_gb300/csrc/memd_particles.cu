@@ -586,20 +586,22 @@ __device__ __forceinline__ void deposit_wide(const Mesh& m, const StepParams& sp
 
 __global__ void __launch_bounds__(kWideThreads)
     k_deposit_wide(const __grid_constant__ Mesh m, const __grid_constant__ StepParams sp,
-                   Particles P, unsigned long long* __restrict__ Tb, DevState* ds) {
+                   Particles P, unsigned long long* __restrict__ Tb, DevState* ds, bool join) {
   let_next_start();
   long long U[3];
   deposit_wide(m, sp, P, Tb, ds, blockIdx.x * (int64_t)blockDim.x + threadIdx.x, U);
   cta_dipole_add3(ds->Pacc, U);
+  if (join) wait_for_previous();
 }
 
 __global__ void __launch_bounds__(kQuadThreads)
     k_kick_drift_deposit(const __grid_constant__ Mesh m, const __grid_constant__ StepParams sp,
                          Particles P, unsigned long long* __restrict__ Tb,
-                         DevState* ds) {
+                         DevState* ds, bool join) {
   let_next_start();
   cta_dipole_add(ds->Pacc,
                  deposit_body(m, sp, P, Tb, ds, blockIdx.x * (int64_t)blockDim.x + threadIdx.x));
+  if (join) wait_for_previous();
 }
 
 // prescribed move to (pos_new, img_new) with its charge transfer
@@ -1224,12 +1226,14 @@ template <typename T>
 __global__ void __launch_bounds__(kWideThreads)
     k_turn_wide(const __grid_constant__ Mesh m, const __grid_constant__ StepParams sp,
                 Particles P, unsigned long long* __restrict__ Tb, const T* __restrict__ D,
-                const T* __restrict__ ie, const double* __restrict__ ie64, DevState* ds) {
+                const T* __restrict__ ie, const double* __restrict__ ie64, DevState* ds,
+                bool join) {
   let_next_start();
   long long U[3];
   turn_wide<T>(m, sp, sp.thermo, P, Tb, D, ie, ie64, ds,
                blockIdx.x * (int64_t)blockDim.x + threadIdx.x, U);
   cta_dipole_add3(ds->Pacc, U);
+  if (join) wait_for_previous();
 }
 
 // quads: velocity and force go through memory, from a lane to itself
@@ -1251,10 +1255,11 @@ template <typename T>
 __global__ void __launch_bounds__(kQuadThreads)
     k_turn(const __grid_constant__ Mesh m, const __grid_constant__ StepParams sp, Particles P,
            unsigned long long* __restrict__ Tb, const T* __restrict__ D, const T* __restrict__ ie,
-           const double* __restrict__ ie64, DevState* ds) {
+           const double* __restrict__ ie64, DevState* ds, bool join) {
   let_next_start();
   cta_dipole_add(ds->Pacc, turn_body<T>(m, sp, sp.thermo, sp.gamma, sp.kT, P, Tb, D, ie, ie64, ds,
                                         blockIdx.x * (int64_t)blockDim.x + threadIdx.x));
+  if (join) wait_for_previous();
 }
 
 template <typename T>
@@ -2279,12 +2284,12 @@ void set_split() {
 }  // namespace
 
 void launch_kick_drift_deposit(const Mesh& m, const StepParams& sp, Particles p, long long* Tb,
-                               DevState* ds, cudaStream_t st, bool early) {
+                               DevState* ds, cudaStream_t st, bool early, bool join) {
   set_split();
   if (p.n >= kWideMinCharges)
-    launch_early(k_deposit_wide, blocks_for(p.n, kWideThreads), kWideThreads, 0, st, early, m, sp, p, (unsigned long long*)Tb, ds);
+    launch_early(k_deposit_wide, blocks_for(p.n, kWideThreads), kWideThreads, 0, st, early, m, sp, p, (unsigned long long*)Tb, ds, join);
   else if (p.n > 0)
-    launch_early(k_kick_drift_deposit, blocks_for(4 * p.n, quad_threads(p.n)), quad_threads(p.n), 0, st, early, m, sp, p, (unsigned long long*)Tb, ds);
+    launch_early(k_kick_drift_deposit, blocks_for(4 * p.n, quad_threads(p.n)), quad_threads(p.n), 0, st, early, m, sp, p, (unsigned long long*)Tb, ds, join);
 }
 
 void launch_move_deposit(const Mesh& m, Particles p, const double* pos_new, const int* img_new,
@@ -2455,7 +2460,7 @@ void launch_gather(const Mesh& m, int prec, const StepParams& sp, Particles p, c
 
 void launch_turn(const Mesh& m, int prec, const StepParams& sp, Particles p, long long* Tb,
                  const void* D, const void* ie, const double* ie64, DevState* ds,
-                 cudaStream_t st, bool early) {
+                 cudaStream_t st, bool early, bool join) {
   set_split();
   if (p.n <= 0) return;
   unsigned long long* T = (unsigned long long*)Tb;
@@ -2463,18 +2468,18 @@ void launch_turn(const Mesh& m, int prec, const StepParams& sp, Particles p, lon
     const unsigned nw = blocks_for(p.n, kWideThreads);
     if (prec == 1)
       launch_early(k_turn_wide<float>, nw, kWideThreads, 0, st, early, m, sp, p, T, (const float*)D,
-                                                      (const float*)ie, ie64, ds);
+                                                      (const float*)ie, ie64, ds, join);
     else
       launch_early(k_turn_wide<double>, nw, kWideThreads, 0, st, early, m, sp, p, T, (const double*)D,
-                                                       (const double*)ie, ie64, ds);
+                                                       (const double*)ie, ie64, ds, join);
     return;
   }
   const int qt = quad_threads(p.n);
   const unsigned nb = blocks_for(4 * p.n, qt);
   if (prec == 1)
-    launch_early(k_turn<float>, nb, qt, 0, st, early, m, sp, p, T, (const float*)D, (const float*)ie, ie64, ds);
+    launch_early(k_turn<float>, nb, qt, 0, st, early, m, sp, p, T, (const float*)D, (const float*)ie, ie64, ds, join);
   else
-    launch_early(k_turn<double>, nb, qt, 0, st, early, m, sp, p, T, (const double*)D, (const double*)ie, ie64, ds);
+    launch_early(k_turn<double>, nb, qt, 0, st, early, m, sp, p, T, (const double*)D, (const double*)ie, ie64, ds, join);
 }
 
 void launch_step_end(DevState* ds, int advance, cudaStream_t st) {
