@@ -132,7 +132,7 @@ typedef struct memd_options {
                              kernel).  All give the same results (TMA to rounding). */
   int32_t step_engine;    /* MEMD_STEP_AUTO: the single launch for small systems (at
                              most 33000 sites and 60 particles per SM; in host round
-                             trips of one step up to 125000 sites, 110000 with FP64
+                             trips of one step up to 125000 sites, 111000 with FP64
                              fields), else the graph;
                              MEMD_STEP_GRAPH: four kernels a step (field update beside
                              the deposition, transfers, gather); MEMD_STEP_SINGLE: the

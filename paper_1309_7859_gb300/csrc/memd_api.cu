@@ -1210,18 +1210,22 @@ extern "C" {
 
 // single launch or graph for this call.  Left to choose, the single launch
 // runs where it was the faster of the two: up to 32^3, where a field tile of
-// few rows goes to every SM, FP32 7.5-8.0 us a step of a 20-step call against
+// few rows goes to every SM, FP32 7.5-8.2 us a step of a 20-step call against
 // 9.5-10.6 (200 to 3000 charges), FP64 13.8-16 against 15.5-18.  33^3 needs
 // larger tiles: FP32 11.8-13.7 against 9.9-10.7, FP64 20-23.5 against
 // 17.4-23.8; 48^3 14-17.7 and 27-37 against 9.8-12.7 and 19.4-30.7 (200 to
 // 9000 charges), and one step a call 36-39 and 50-58 against 31-34 and 44-52.
+// The site count stands for the tiles of compact meshes; an elongated one
+// needs larger tiles sooner (24 x 20 x 68: FP32 9.8-10.9 us a step against
+// 9.5-10.7, FP64 17.5-20.4 against 16.8-19.3; 8 x 8 x 512: 13.4-15.4 and
+// 22-25.6 against 9.6-11.5 and 14.4-17.4).
 // A host round trip of one step in place (io) has no launch but its own in
-// the single launch, and is faster there up to 48^3: FP32 26-31 us a call
-// against 30-45 (200 to 8000 charges), FP64 40-48.5 against 42-61.
+// the single launch, and is faster there up to 48^3 and beyond: FP32 25-30 us
+// a call against 27-43 (200 to 8000 charges), FP64 39-48 against 39-58.
 static bool want_coop(const memd_ctx* c, bool io) {
   if (c->coop_grid <= 0 || c->step_engine == MEMD_STEP_GRAPH) return false;
   if (c->step_engine == MEMD_STEP_SINGLE) return true;
-  const int64_t most = io || c->skewed ? (c->prec == MEMD_FP32 ? 125000 : 110000) : 33000;
+  const int64_t most = io || c->skewed ? (c->prec == MEMD_FP32 ? 125000 : 111000) : 33000;
   return c->mesh.V <= most && c->P.n <= (int64_t)60 * c->coop_grid;
 }
 

@@ -2260,12 +2260,16 @@ void launch_particle_constants(const StepParams& sp, Particles p, cudaStream_t s
 
 namespace {
 // A quad kernel of few charges leaves an SM room for the row kernel that runs
-// beside it, so it asks for the row kernel's split of the SM's L1 and shared
-// memory: an SM changes its split only when it is empty, and one warp under
-// the default split kept the row kernel's CTAs off its SM until it ended
-// (FP64 32^3, 1000 charges: 22 us a step for 14).  The wide kernels fill the
-// SMs themselves and live off the L1 (64 replicas, 10 steps: 1180 us, with
-// the row kernel's split 1560-1590), so they keep the default.
+// beside it, so the quad kernels ask for the row kernel's split of the SM's L1
+// and shared memory: an SM changes its split only when it is empty, and one
+// warp under the default split kept the row kernel's CTAs off its SM until it
+// ended (FP64 32^3, 1000 charges: 22 us a step for 14; FP64 64^3, 10 steps,
+// 1000 and 4000 charges: 391 and 407 us for 341 and 375).  The split belongs
+// to the kernel, so it holds for all of its sizes: above ~8000 charges the
+// smaller L1 costs 1-3% beside the row kernel (64^3, 8000 to 16000 charges),
+// nothing beside the tiles.  The wide kernels fill the SMs themselves and live
+// off the L1 (64 replicas, 10 steps: 1180 us, with the row kernel's split
+// 1560-1590), so they keep the default.
 bool prefer_shared() {
   const void* k[] = {
       (const void*)k_kick_drift_deposit,  (const void*)k_deposit_batch,
