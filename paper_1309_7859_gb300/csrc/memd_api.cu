@@ -738,6 +738,8 @@ static memd_status setup_eps(memd_ctx* c, const memd_eps_profile* eps,
   }
   s = check_err(c);
   if (s != MEMD_OK) goto out;
+  dfree(c, vals);  // mapped: the stream is idle
+  vals = nullptr;
   psi = (double*)dalloc(c, n3 * sizeof(double));
   if (psi) {
     double ef[9];

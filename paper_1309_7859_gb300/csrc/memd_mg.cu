@@ -23,7 +23,7 @@
 // extent below 4, or at most 64 vertices) is swept.
 //
 // Every value and every sum is rounded in one fixed order, whatever the grid
-// and however many right-hand sides are solved at once: B of a system one
+// and the number of right-hand sides: B of a system one
 // step from its relaxed field is nothing but the rounding of that field
 // (curl E is zero in exact arithmetic), so a solver that is as accurate but
 // rounds elsewhere gives every such B anew.  Sums therefore run in the order
@@ -118,18 +118,16 @@ struct MgOut {
 
 struct MgArgs {
   int nl, nlg;  // levels, and how many of them are swept by the whole grid
-  int dir0;     // cells: direction of right-hand side 0
   int maxit;
   double tol;
   double inv_a, inv_a2;
   const double* ie64;
-  double* x;    // solution
+  double* x;    // solution (cells: psi)
   double* p;
-  double* q;
+  double* q;    // shared with the residual of level 0, which the cycle leaves behind
   double* part;       // kMgSlots x kMgQ sums of every warp
   unsigned* arrivals; // barrier count, 0 at launch
   MgOut* out;
-  double* psi;        // cells: written (3 V)
   double* D64;        // relax: in and out
   MgLv lv[kMgMaxLevels];
 };
@@ -554,8 +552,8 @@ __device__ __forceinline__ void cta_cycle(const MgLv* lv, int nc, const MgLv& to
 }
 
 // The whole solve for NR right-hand sides.
-//   cells: L psi_d = -div(eps e_d) for d = dir0 .. dir0 + NR - 1, psi_d of
-//   zero mean and the sums of the fluxes eps_e (delta_ed - grad_e psi_d)
+//   cells: L psi_d = -div(eps e_d) for d < NR, psi_d of zero mean and the
+//   sums of the fluxes eps_e (delta_ed - grad_e psi_d)
 //   relax: L phi = div D64; D64 <- -eps grad phi, and the sums of D64 before
 //   and after
 // The residual is looked at every second iteration.  Stops when |r| <= tol
@@ -622,9 +620,8 @@ __global__ void __launch_bounds__(kMgThreads, 1) k_mg_solve(const __grid_constan
         } else {
 #pragma unroll
           for (int r = 0; r < NR; ++r) {
-            const int d = a.dir0 + r;
-            const double* ie = a.ie64 + (int64_t)d * V;
-            const double f = mul_(-sub_(__drcp_rn(ie[v]), __drcp_rn(ie[vm[d]])), inv_a);
+            const double* ie = a.ie64 + (int64_t)r * V;
+            const double f = mul_(-sub_(__drcp_rn(ie[v]), __drcp_rn(ie[vm[r]])), inv_a);
             L.f[r * V + v] = f;
             s[r] = add_(s[r], f);
           }
@@ -913,12 +910,11 @@ __global__ void __launch_bounds__(kMgThreads, 1) k_mg_solve(const __grid_constan
   }
   MG_GRID();
   total_sums<NR>(a.part, 5, nW, m, sums);
-  double* const y = MODE == kMgCells ? a.psi + (int64_t)a.dir0 * V : a.x;
   for (int v = t0; v < V; v += stride)
 #pragma unroll
-    for (int r = 0; r < NR; ++r) y[(int64_t)r * V + v] = sub_(a.x[r * V + v], m[r] / nV);
+    for (int r = 0; r < NR; ++r) a.x[r * V + v] = sub_(a.x[r * V + v], m[r] / nV);
   MG_GRID();
-  // the fluxes eps (e_d - grad y), in the relaxation -eps grad y in D64 (left
+  // the fluxes eps (e_d - grad x), in the relaxation -eps grad x in D64 (left
   // as it came when the solve has not converged)
   if (MODE == kMgRelax && !all) {
     if (blockIdx.x == 0 && threadIdx.x == 0) a.out->iters = its;
@@ -938,8 +934,8 @@ __global__ void __launch_bounds__(kMgThreads, 1) k_mg_solve(const __grid_constan
         const double ie = a.ie64[(int64_t)e * V + v];
 #pragma unroll
         for (int r = 0; r < NR; ++r) {
-          const double* p = y + (int64_t)r * V;
-          const double g = MODE == kMgCells && e == a.dir0 + r ? 1.0 : 0.0;
+          const double* p = a.x + r * V;
+          const double g = MODE == kMgCells && e == r ? 1.0 : 0.0;
           const double F = fma_(-sub_(p[vp[e]], p[v]), inv_a, g) / ie;
           if (MODE == kMgRelax) a.D64[(int64_t)e * V + v] = F;
           s[3 * r + e] = add_(s[3 * r + e], F);
@@ -958,7 +954,7 @@ __global__ void __launch_bounds__(kMgThreads, 1) k_mg_solve(const __grid_constan
         a.out->sum[3 + e] = s[e];
       } else {
 #pragma unroll
-        for (int r = 0; r < NR; ++r) a.out->sum[3 * e + a.dir0 + r] = s[3 * r + e];
+        for (int r = 0; r < NR; ++r) a.out->sum[3 * e + r] = s[3 * r + e];
       }
     }
     a.out->converged = all ? 1 : 0;
@@ -1033,7 +1029,8 @@ struct MgPlan {
   size_t smem = 0;
   int grid = 0;
 
-  bool build(memd_ctx* c, int nr) {
+  // x: the cell problems' potentials, or null for one of the plan's own
+  bool build(memd_ctx* c, int nr, double* x) {
     const Mesh& m = c->mesh;
     int sms = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess)
@@ -1071,7 +1068,7 @@ struct MgPlan {
     smem = 9 * sites * sizeof(double);
     const size_t head = (sizeof(MgOut) + 64) / sizeof(double) + 1;  // result, barrier count
     const size_t parts = (size_t)kMgSlots * kMgQ * std::min<int64_t>(kSumWarps, (m.V + 31) / 32);
-    const size_t total = head + parts + words + (size_t)3 * nr * m.V;
+    const size_t total = head + parts + words + (size_t)(x ? nr : nr + 1) * m.V;
     block = (double*)memd_dalloc(c, total * sizeof(double));
     if (!block) return false;
     a.out = (MgOut*)block;
@@ -1091,9 +1088,9 @@ struct MgPlan {
       L.phi = L.r + nr * V;
       L.alt = L.rb ? nullptr : L.phi + nr * V;
     }
-    a.x = base + words;
-    a.p = a.x + (size_t)nr * m.V;
-    a.q = a.p + (size_t)nr * m.V;
+    a.p = base + words;
+    a.q = a.lv[0].r;
+    a.x = x ? x : a.p + (size_t)nr * m.V;
     a.inv_a = 1.0 / m.a;
     a.inv_a2 = 1.0 / (m.a * m.a);
     a.ie64 = c->ie64;
@@ -1113,33 +1110,19 @@ struct MgPlan {
   }
 };
 
-// Set on a thread (the request server's admission workers): that thread's
-// cell problems are solved in turn, with one right-hand side's scratch.
-thread_local bool t_cells_in_turn = false;
-
 }  // namespace
-
-void memd_mg_cells_in_turn(bool on) { t_cells_in_turn = on; }
 
 // Cell problems: psi_d (3V, stored), and eps_eff[e][d] = mean over links of
 // eps_e (delta_ed - grad_e psi_d) (row e, column d).
 memd_status mg_eps_eff(memd_ctx* c, double* psi, double eps_eff[9], double tol, int maxit) {
-  const int nr = t_cells_in_turn ? 1 : 3;
   MgPlan plan;
-  if (!plan.build(c, nr)) return MEMD_ERR_OOM;
-  plan.a.psi = psi;
+  if (!plan.build(c, 3, psi)) return MEMD_ERR_OOM;
   plan.a.tol = tol;
   plan.a.maxit = maxit < 400 ? maxit : 400;
-  memd_status s = MEMD_OK;
-  for (int d = 0; d < 3 && s == MEMD_OK; d += nr) {
-    plan.a.dir0 = d;
-    MgOut h;
-    s = nr == 1 ? plan.run<1, kMgCells>(c, h) : plan.run<3, kMgCells>(c, h);
-    if (s == MEMD_OK)
-      for (int r = 0; r < nr; ++r)
-        for (int e = 0; e < 3; ++e)
-          eps_eff[3 * e + d + r] = h.sum[3 * e + d + r] / (double)c->mesh.V;
-  }
+  MgOut h;
+  const memd_status s = plan.run<3, kMgCells>(c, h);
+  if (s == MEMD_OK)
+    for (int t = 0; t < 9; ++t) eps_eff[t] = h.sum[t] / (double)c->mesh.V;
   memd_dfree(c, plan.block);
   return s;
 }
@@ -1150,7 +1133,7 @@ memd_status mg_eps_eff(memd_ctx* c, double* psi, double eps_eff[9], double tol, 
 memd_status mg_relax(memd_ctx* c, double* D64, const double* psi, const double eps_eff_inv[9],
                      double tol, int maxit, int* iters) {
   MgPlan plan;
-  if (!plan.build(c, 1)) return MEMD_ERR_OOM;
+  if (!plan.build(c, 1, nullptr)) return MEMD_ERR_OOM;
   plan.a.D64 = D64;
   plan.a.tol = tol;
   plan.a.maxit = maxit < 400 ? maxit : 400;
